@@ -229,8 +229,11 @@ extern "C" int oq_clover_build_ex(oq_handle h, int lat, const oq_clover_params* 
     rc = clover_build_halo(h, lat, kappa, csw, s);
     if (rc) return rc;
   } else {
-    const double* links = L.uclov_valid ? (const double*)L.uclov.p : (const double*)L.u64.p;
-    if (build_clover(L.g, links, L.has_u1 ? (const double*)L.au1.p : nullptr, L.qcharge, prm->qed_split, kappa, csw,
+    // the U(3) clover of a QCD+QED lattice: the hopping links hold the phases
+    // already (Schroedinger-functional ones are masked: the phases are formed anew)
+    const bool u3 = L.has_u1 && !prm->qed_split && L.g.bc_t != 0.f;
+    const double* links = L.uclov_valid && !u3 ? (const double*)L.uclov.p : (const double*)L.u64.p;
+    if (build_clover(L.g, links, L.has_u1 && !u3 ? (const double*)L.au1.p : nullptr, L.qcharge, prm->qed_split, kappa, csw,
                      prm->csw_qed, prm->cF, (double*)L.a64.p, (float*)L.a32.p, (double*)L.i64.p, (float*)L.i32.p,
                      h->status_dev, s) != cudaSuccess)
       return OQ_ERR_CUDA;
