@@ -116,11 +116,57 @@ __global__ void __launch_bounds__(PB) ptc_layer_kernel(const PtcArgs a) {
   for (int co = 0; co < COUT; ++co) store_spinor<P_F32>(a.out + co * a.fbytes + (long)p * a.hbytes, a.g.Vh, i, acc[co]);
 }
 
+// Sums over the warp of 64 binary32 values per lane: out[j] of lane l is the
+// sum of v[2l + j].  A transposing exchange (each step halves the values a lane
+// holds: 62 additions per lane instead of 5 per value), in double-float: the
+// first additions are exact, the others err by ~2^-47, against the 2^-24 of the
+// binary32 sums that come in.  In binary64 (1/64 of the binary32 rate) the warp
+// sums were half of the gradient kernels' time; they are taken that way where a
+// value of the warp is not finite or above 2^100 (binary32 sums could overflow).
+__device__ __forceinline__ void warp_sum64(const float (&v)[64], double (&out)[2]) {
+  const int lane = threadIdx.x & 31;
+  bool big = false;
+#pragma unroll
+  for (int k = 0; k < 64; ++k) big |= !(fabsf(v[k]) <= 1.2676506e30f);
+  if (__any_sync(0xffffffffu, big)) {
+    out[0] = out[1] = 0.0;
+#pragma unroll
+    for (int k = 0; k < 64; ++k) {
+      const double t = warp_sum((double)v[k]);
+      if (lane == k / 2) out[k % 2] = t;
+    }
+    return;
+  }
+  dfloat d[32];
+  {
+    const bool up = lane & 16;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+      const float keep = up ? v[k + 32] : v[k], send = up ? v[k] : v[k + 32];
+      d[k] = df_two_sum(keep, __shfl_xor_sync(0xffffffffu, send, 16));
+    }
+  }
+#pragma unroll
+  for (int h = 16; h >= 2; h >>= 1) {
+    const int o = h >> 1;  // lane distance of this step
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const dfloat keep = up ? d[k + h] : d[k], send = up ? d[k] : d[k + h];
+      const dfloat got(__shfl_xor_sync(0xffffffffu, send.hi, o), __shfl_xor_sync(0xffffffffu, send.lo, o));
+      d[k] = keep + got;
+    }
+  }
+  out[0] = (double)d[0];
+  out[1] = (double)d[1];
+}
+
 // Weight-gradient partials for one path (blockIdx.y): COUT*CIN*16 complex per
-// CTA, binary64, written to part[q][cta][k].
+// CTA, written in binary64 to part[q][cta][k].
 template <int FMT, int CIN, int COUT>
 __global__ void __launch_bounds__(PB) ptc_dw_kernel(const PtcArgs a, const char* grad, double* part) {
   constexpr int NW = COUT * CIN * 16;  // complex entries per path
+  static_assert(NW == 32, "the warp sum holds 64 reals per path");
   __shared__ double red[PB / 32][2 * NW];
   const int q = blockIdx.y;
   float accr[NW], acci[NW];
@@ -153,16 +199,18 @@ __global__ void __launch_bounds__(PB) ptc_dw_kernel(const PtcArgs a, const char*
           }
     }
   }
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // the warp's sum of the 2 NW = 64 values: lane l ends with values 2l, 2l + 1
+  float v[2 * NW];
 #pragma unroll
   for (int k = 0; k < NW; ++k) {
-    double r = warp_sum((double)accr[k]);
-    double m = warp_sum((double)acci[k]);
-    if (lane == 0) {
-      red[wid][2 * k] = r;
-      red[wid][2 * k + 1] = m;
-    }
+    v[2 * k] = accr[k];
+    v[2 * k + 1] = acci[k];
   }
+  double t[2];
+  warp_sum64(v, t);
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  red[wid][2 * lane] = t[0];
+  red[wid][2 * lane + 1] = t[1];
   __syncthreads();
   for (int k = threadIdx.x; k < 2 * NW; k += blockDim.x) {
     double s = 0.0;
@@ -171,14 +219,25 @@ __global__ void __launch_bounds__(PB) ptc_dw_kernel(const PtcArgs a, const char*
   }
 }
 
-// sum the per-CTA partials in a fixed order: dw[q][k] += sum_cta part[q][cta][k]
-__global__ void ptc_dw_finish(const double* part, int ncta, int nw2, double* dw) {
-  const int q = blockIdx.x;
-  for (int k = threadIdx.x; k < nw2; k += blockDim.x) {
-    double s = 0.0;
-    for (int c = 0; c < ncta; ++c) s += part[((long)q * ncta + c) * nw2 + k];
-    dw[(long)q * nw2 + k] += s;
-  }
+// sum the per-CTA partials in a fixed order: dw[q][k] += sum_cta part[q][cta][k].
+// One CTA per path, thread (k, j) adds the partials j, j + FIN, ... of value k
+// and the FIN sums are added in order (one thread per value, its loads one
+// after the other, took 108 us for 256 partials on 32x16^3, a fifth of the
+// gradient; this form 8.7 us).
+static const int FIN = 16;
+__global__ void __launch_bounds__(64 * FIN) ptc_dw_finish(const double* part, int ncta, double* dw) {
+  constexpr int NV = 64;
+  __shared__ double sum[FIN][NV];
+  const int q = blockIdx.x, k = threadIdx.x % NV, j = threadIdx.x / NV;
+  double s = 0.0;
+#pragma unroll 4
+  for (int c = j; c < ncta; c += FIN) s += part[((long)q * ncta + c) * NV + k];
+  sum[j][k] = s;
+  __syncthreads();
+  if (j) return;
+#pragma unroll
+  for (int w = 1; w < FIN; ++w) s += sum[w][k];
+  dw[(long)q * NV + k] += s;
 }
 
 // bfloat16 forward weights and the adjoint layer's weights from binary32 masters:
@@ -411,7 +470,9 @@ extern "C" int oq_nnprec_grad(oq_handle h, int lat, const float* weights_dev, co
   const int ncta = reduce_grid(2 * Vh) < 256 ? reduce_grid(2 * Vh) : 256;
   void* part;
   rc = h->workspace(lat, "nn_part", sizeof(double) * NPATH * ncta * 2 * 32, &part);
-  if (!rc) rc = h->ensure_reduce(2, reduce_grid(2 * Vh));
+  const int GRP = 32;
+  double en2[32];
+  if (!rc) rc = h->ensure_reduce(2 * GRP, reduce_grid(2 * Vh));
   if (rc) return rc;
   const int fmt = L.link_fmt;
   const int nreal = 2 * (NW1 + NW2);
@@ -419,36 +480,43 @@ extern "C" int oq_nnprec_grad(oq_handle h, int lat, const float* weights_dev, co
   double* gw1 = grad_dev;
   double* gw2 = grad_dev + 2 * NW1;
   double loss = 0.0;
+  // pairs in groups of GRP: the norms of the group's e in one launch per parity
+  // (one wait), the losses read back together at the group's end (another);
+  // a wait for the norm and one for the loss of every pair left the GPU idle
+  // between its kernels
   for (int k = 0; k < n; ++k) {
+    const int kg = k % GRP, ng = n - (k - kg) < GRP ? n - (k - kg) : GRP;
     const char* r = (const char*)r_dev + (long)k * f32;
     const char* e = (const char*)e_dev + (long)k * f32;
-    // ||e||^2
     RedArgs ra = h->red_args(FIN_STORE, 0);
-    h->launches += 2;
-    if (reduce_norm2(P_F32, e, Vh, 0, 1, ra, s) != cudaSuccess) return OQ_ERR_CUDA;
-    ra.result = h->results + 1;
-    if (reduce_norm2(P_F32, e + hb, Vh, 0, 1, ra, s) != cudaSuccess) return OQ_ERR_CUDA;
-    if (cudaMemcpyAsync(h->results_host, h->results, 2 * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-      return OQ_ERR_CUDA;
-    const double en2 = h->results_host[0] + h->results_host[1];
-    if (!(en2 > 0.0)) return OQ_ERR_ARG;
+    if (kg == 0) {
+      // ||e||^2 of the group: parity halves in results[0 .. ng) and [ng .. 2 ng)
+      h->launches += 2;
+      if (reduce_norm2(P_F32, e, Vh, f32, ng, ra, s) != cudaSuccess) return OQ_ERR_CUDA;
+      ra.result = h->results + ng;
+      if (reduce_norm2(P_F32, e + hb, Vh, f32, ng, ra, s) != cudaSuccess) return OQ_ERR_CUDA;
+      if (cudaMemcpyAsync(h->results_host, h->results, 2 * ng * sizeof(double), cudaMemcpyDeviceToHost, s) !=
+              cudaSuccess ||
+          cudaStreamSynchronize(s) != cudaSuccess)
+        return OQ_ERR_CUDA;
+      for (int j = 0; j < ng; ++j) {
+        en2[j] = h->results_host[j] + h->results_host[ng + j];
+        if (!(en2[j] > 0.0)) return OQ_ERR_ARG;
+      }
+    }
     rc = nn_forward(h, lat, b, r, b.y, s);
     if (rc) return rc;
     ra = h->red_args(FIN_STORE, 0);
+    ra.result = h->results + kg;
     // mean over the n pairs: loss_k / n and its gradient
-    ptc_loss_kernel<<<reduce_grid(2 * Vh), 256, 0, s>>>(b.y, e, b.gy, 1.0 / (en2 * n), Vh, hb, ra);
+    ptc_loss_kernel<<<reduce_grid(2 * Vh), 256, 0, s>>>(b.y, e, b.gy, 1.0 / (en2[kg] * n), Vh, hb, ra);
     h->launches += 1;
-    if (cudaMemcpyAsync(h->results_host, h->results, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-      return OQ_ERR_CUDA;
-    loss += h->results_host[0];
     // layer 2: dW2 from (hid, gy); g_hid = L2^dag gy
     PtcArgs a = nn_args(h, lat);
     a.in = b.hid;
     a.w = b.w2;
     if (ptc_dw<CH, 1>(a, fmt, b.gy, (double*)part, ncta, s) != cudaSuccess) return OQ_ERR_CUDA;
-    ptc_dw_finish<<<NPATH, 128, 0, s>>>((const double*)part, ncta, 2 * CH * 16, gw2);
+    ptc_dw_finish<<<NPATH, 64 * FIN, 0, s>>>((const double*)part, ncta, gw2);
     a.in = b.gy;
     a.out = b.ghid;
     a.w = b.w2a;
@@ -458,9 +526,16 @@ extern "C" int oq_nnprec_grad(oq_handle h, int lat, const float* weights_dev, co
     a.in = r;
     a.w = b.w1;
     if (ptc_dw<1, CH>(a, fmt, b.ghid, (double*)part, ncta, s) != cudaSuccess) return OQ_ERR_CUDA;
-    ptc_dw_finish<<<NPATH, 128, 0, s>>>((const double*)part, ncta, 2 * CH * 16, gw1);
+    ptc_dw_finish<<<NPATH, 64 * FIN, 0, s>>>((const double*)part, ncta, gw1);
     h->launches += 5;
     if (cudaGetLastError() != cudaSuccess) return OQ_ERR_CUDA;
+    if (kg == ng - 1) {
+      if (cudaMemcpyAsync(h->results_host, h->results, ng * sizeof(double), cudaMemcpyDeviceToHost, s) !=
+              cudaSuccess ||
+          cudaStreamSynchronize(s) != cudaSuccess)
+        return OQ_ERR_CUDA;
+      for (int j = 0; j < ng; ++j) loss += h->results_host[j];
+    }
   }
   if (loss_host) *loss_host = loss;
   return OQ_OK;
