@@ -21,23 +21,11 @@
 
 namespace oq {
 
-// Accumulate one transported hop: with weight w (times the time-boundary
-// factor when the hop crosses it) for binary64 / binary32, where the weight
-// folds into FMAs; double-float sums the hops unweighted (a sign flip for
-// the boundary) and hop_site scales once by w = +-1/2 (exact).
+// Accumulate one transported hop with weight w (times the time-boundary
+// factor when the hop crosses it).
 template <int MU, int S, typename R>
 __device__ __forceinline__ void hop_accum(Spinor<R>& acc, HalfSpinor<R>& t, R w, bool cr, float bc_t) {
-  if constexpr (std::is_same<R, dfloat>::value) {
-    if (cr && bc_t < 0.f) {
-#pragma unroll
-      for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) t.c[s][c] = -t.c[s][c];
-    }
-    accum_reconstruct<MU, S, R, false>(acc, t, w);
-  } else {
-    accum_reconstruct<MU, S>(acc, t, cr ? w * (R)bc_t : w);
-  }
+  accum_reconstruct<MU, S>(acc, t, cr ? w * (R)bc_t : w);
 }
 
 // fnext / fprev (sub-domain launches, this rhs and output parity): the time
@@ -196,7 +184,7 @@ __device__ __forceinline__ RedT<P> hop_site(const HopArgs& a, long i, int rhs, i
 #pragma unroll
       for (int c = 0; c < 3; ++c) acc.c[s][c] = cx<R>{0, 0};
     const R w = (MODE == HOP_P2) ? (R)0.5 : (R)-0.5;
-    constexpr bool DF = std::is_same<R, dfloat>::value;
+    constexpr bool DF = std::is_same<R, dfloat>::value, F64 = std::is_same<R, double>::value;
     if constexpr (DF && MODE != HOP_P1) {
       // double-float: A in2 / w first (w = +-1/2, so the scaling is exact)
       // while few registers are live; the unweighted hops add onto it and
@@ -210,6 +198,12 @@ __device__ __forceinline__ RedT<P> hop_site(const HopArgs& a, long i, int rhs, i
 #pragma unroll
         for (int c = 0; c < 3; ++c)
           acc.c[s][c] = cx<R>{df_scale(acc.c[s][c].re, iw), df_scale(acc.c[s][c].im, iw)};
+    }
+    if constexpr (F64 && MODE != HOP_P1) {
+      // binary64: the hops add onto A in2 (24 additions fewer on the binary64 pipe)
+      Spinor<R> loc;
+      load_spinor<P>((const char*)a.in2 + rhs * a.in2_stride + par_out, a.g.Vh, i, loc);
+      clover_apply<R>(a.clov, a.g.Vh, p, i, loc, acc);
     }
     if constexpr (DF) {
       hop_loop_df<P, FMT, DAG>(a, in, p, i, x, acc);
@@ -237,7 +231,7 @@ __device__ __forceinline__ RedT<P> hop_site(const HopArgs& a, long i, int rhs, i
     Spinor<R> res;
     if constexpr (MODE == HOP_P1) {
       clover_apply<R>(a.cinv, a.g.Vh, p, i, acc, res);
-    } else if constexpr (DF) {
+    } else if constexpr (DF || F64) {
       res = acc;
     } else {
       const char* in2 = (const char*)a.in2 + rhs * a.in2_stride + par_out;
