@@ -317,9 +317,9 @@ int oq_tune_set(oq_handle h, int lat, int prec, int mode, int nrhs, int bx, int 
  *   CUDA-core layers of oq_nnprec_apply (measured faster on GB300 for this
  *   small network). */
 /* OQ_OPT_SAP_KERNEL: the SAP block kernel (one CTA per block, one thread per
- *   block site).  0 (default) = the block's links (18 reals) and clover
- *   blocks are staged in shared memory once and the MR steps read only shared
- *   memory (falls back to 2 when they do not fit in 227 KB); 1 = operands from
+ *   block site).  0 (default) = the block's links are held in registers, its
+ *   clover blocks staged in shared memory once, and the MR steps read only
+ *   shared memory; 1 = operands from
  *   global memory, ~217 registers, one 256-site block per SM; 2 = operands
  *   from global memory, registers capped so that two blocks run per SM.
  *   Other values: OQ_ERR_ARG. */

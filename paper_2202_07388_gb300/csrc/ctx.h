@@ -108,7 +108,7 @@ struct oq_ctx {
   bool df64_resets = true;   // OQ_OPT_DF64_RESETS
   // test hook: the tensor-core PTC layer issues no MMA, so its bounded wait runs out
   bool hook_tc_skip_commit = false;
-  // SAP block kernel: 0 operands staged in shared memory, 1 operands from
+  // SAP block kernel: 0 links in registers and clover in shared memory, 1 operands from
   // global memory, 2 the same register-capped for two CTAs per SM
   int sap_kernel = 0;        // OQ_OPT_SAP_KERNEL
   // NN-preconditioned GCR applies the network with the tensor-core layers

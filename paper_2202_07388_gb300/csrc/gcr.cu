@@ -243,14 +243,12 @@ extern "C" int oq_sap_apply(oq_handle h, int lat, const oq_solver_params* prm, c
   // shifted (C*) wraps keep the block colouring only if the x1 shift is an even number of blocks
   if (L.g.cs_shift && ((L.g.L[1] / 2) / prm->bs[1]) % 2) return OQ_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
-  const long f32 = 2 * spinor_half_bytes(L.g.Vh, P_F32);
-  if (cudaMemsetAsync(phi_dev, 0, f32, s) != cudaSuccess) return OQ_ERR_CUDA;
   const float alpha = (float)(prm->alpha > 0.0 ? prm->alpha : 0.9);
   for (int cy = 0; cy < prm->ncy; ++cy)
     for (int colour = 0; colour < 2; ++colour) {
       h->launches += 1;
       if (sap_colour(L.g, prm->bs, colour, L.link_fmt, L.u32.p, L.a32.p, L.i32.p, rho_dev, phi_dev, prm->nmr,
-                     prm->adaptive, alpha, mr_tol, nullptr, h->sap_kernel, prm->sap_eo, s) != cudaSuccess)
+                     prm->adaptive, alpha, mr_tol, nullptr, h->sap_kernel, prm->sap_eo, cy, s) != cudaSuccess)
         return OQ_ERR_CUDA;
     }
   return OQ_OK;
@@ -400,9 +398,9 @@ static int gcr_impl(oq_handle h, int lat, const oq_solver_params* prm, const flo
         } else if (prm->ncy == 0) {
           CK(cudaMemcpyAsync(phik, rho, f32, cudaMemcpyDeviceToDevice, s));
         } else {
-          CK(cudaMemsetAsync(phik, 0, f32, s));
           double prev = 0.0;
           if (prm->adaptive) {
+            CK(cudaMemsetAsync(phik, 0, f32, s));
             KL((vec_diff_norm_kernel<P_F32><<<rgrid, rblock, 0, s>>>(nullptr, (const char*)rho, (const char*)phik,
                                                                      Vh, hb32, ra),
                 cudaGetLastError()));
@@ -412,7 +410,7 @@ static int gcr_impl(oq_handle h, int lat, const oq_solver_params* prm, const flo
             for (int colour = 0; colour < 2; ++colour)
               KL(sap_colour(L.g, prm->bs, colour, L.link_fmt, L.u32.p, L.a32.p, L.i32.p, rho, phik, prm->nmr,
                             prm->adaptive, (float)(prm->alpha > 0.0 ? prm->alpha : 0.9), prm->res * eta_n / nblk,
-                            (unsigned*)mrc, h->sap_kernel, prm->sap_eo, s));
+                            (unsigned*)mrc, h->sap_kernel, prm->sap_eo, cy, s));
             cycles_total += 1;
             if (prm->adaptive) {
               // cycle test on the global SAP residual ||rho - D phi||

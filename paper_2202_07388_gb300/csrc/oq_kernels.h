@@ -64,12 +64,13 @@ int nnprec_forward(struct ::oq_ctx* h, int lat, const void* r, void* y, cudaStre
 // takes the binary32 master weights, synchronises s, OQ_ERR_TIMEOUT on a failed wait
 int nnprec_forward_tc(struct ::oq_ctx* h, int lat, const float* master, const void* r, void* y, cudaStream_t s);
 
-// one SAP half cycle: every block of `colour` (binary32 fields); eo: MR on
-// the blocks' even-odd Schur complements (needs clov_inv and blocks whose
-// operands fit in shared memory, else cudaErrorInvalidValue)
+// one SAP half cycle: every block of `colour` (binary32 fields); cycle: the
+// Schwarz cycle's number (in cycle 0 phi counts as zero whatever it holds, and
+// colours 0, 1 set all of it); eo: MR on the blocks' even-odd Schur complements
+// (needs clov_inv and blocks whose operands fit in shared memory, else
+// cudaErrorInvalidValue)
 cudaError_t sap_colour(const Geom& g, const int bs[4], int colour, int fmt, const void* links, const void* clov,
                        const void* clov_inv, const void* rho, void* phi, int nmr, int adaptive, float alpha,
-                       double tol, unsigned* mr_steps, int kernel, int eo, cudaStream_t s);
-size_t sap_smem_bytes(const int bs[4]);
+                       double tol, unsigned* mr_steps, int kernel, int eo, int cycle, cudaStream_t s);
 
 }  // namespace oq

@@ -18,8 +18,8 @@
 //   3. phi_i += x.
 // sap_smem_eo_kernel replaces 2 by MR steps on the block's even-odd Schur
 // complement (see below).  Block reductions are binary64.  Arithmetic and storage binary32.
-// sap_smem_kernel (the default) stages the block's links and clover in
-// shared memory first; sap_kernel reads them from global memory.
+// sap_block_kernel (the default) keeps a site's links in registers and the
+// block's clover in shared memory; sap_kernel reads them from global memory.
 #include "oq_internal.h"
 #include "oq_kernels.h"
 #include "hop_impl.cuh"
@@ -31,6 +31,7 @@ struct SapArgs {
   int bs[4];
   int nb[4];
   int colour;
+  int first;           // first cycle: phi is zero on this colour (colour 0: everywhere)
   const void* links;   // binary32 packed links
   const void* clov;    // binary32 packed clover
   const void* clov_inv;  // binary32 packed inverse clover (even-odd block solver)
@@ -272,14 +273,338 @@ __global__ void __launch_bounds__(256, MINB) sap_kernel(const SapArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// The same block solve with the block's operands staged in shared memory
-// once: the 4 forward links of every block site (18 reals, rebuilt from 12
-// where stored compressed) and its two clover blocks.  The MR steps then
-// read only shared memory (the residual, the links, the clover) instead of
-// fetching ~670 bytes per site and step from L2.  Static MR (not adaptive)
-// needs no norm reduction per step, only the barrier before the residual is
-// read again.  Shared memory: 24 + 4*18 + 72 floats per block site.
+// The default block solve.  A site's thread keeps its four forward links (18
+// reals each) and its residual in registers; the block's clover is staged in
+// shared memory once.  The backward hop of x along mu is U_mu(x-mu)^dag times
+// the projected residual of x-mu, both of which the thread of x-mu holds: every
+// thread transports its own residual along its four links and leaves the half
+// spinors in shared memory for its forward neighbours ("sends"), next to the
+// residual itself, from which the forward hops read.  An MR step then moves
+// 288 words per site through shared memory (24 + 48 written, 4 x 24 residuals,
+// 48 received, 72 clover), all in 16-byte accesses, against 456 in 4-byte and
+// 8-byte ones when every hop read the neighbour's residual and a link, and needs
+// two barriers instead of three.  Hops that leave the block are dropped by a
+// zero weight rather than a branch, so that the loads of several hops overlap.
+//
+// The block residual rho - D phi takes the in-block part of D phi through the
+// same shared-memory operator and reads only the neighbours outside the block
+// from global memory.  In the first cycle (FIRST) phi is zero on the blocks of
+// this colour (and, with colour 0, everywhere), so those terms are left out.
+// Bound by latency at one block of 8 warps per SM (255 registers, 147 KB): issue
+// 38 % active, a third of the time in staging.  48x24^3, 4^4 blocks, 5 MR steps:
+// 233 us a launch against 338 us with links and residual in shared memory as
+// described above.
+// Shared memory: 72 + 24 + 48 floats per block site.
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ void cp_async16(float4* smem, const float4* gmem) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(a), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+
+struct SapShared {
+  float4* a;  // [18][nsite] clover (two blocks: 6 diagonal + 15 complex each)
+  float4* r;  // [6][nsite] residual, two complex components per chunk
+  float4* s;  // [mu][3][nsite] half spinors sent to the site above along mu
+  int nsite;
+};
+
+__device__ __forceinline__ void sm4_load(const float4* b, int nsite, int t, Spinor<float>& v) {
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const float4 w = b[c * nsite + t];
+    v.c[(2 * c) / 3][(2 * c) % 3] = cx<float>{w.x, w.y};
+    v.c[(2 * c + 1) / 3][(2 * c + 1) % 3] = cx<float>{w.z, w.w};
+  }
+}
+__device__ __forceinline__ void sm4_store(float4* b, int nsite, int t, const Spinor<float>& v) {
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const cx<float> x = v.c[(2 * c) / 3][(2 * c) % 3], y = v.c[(2 * c + 1) / 3][(2 * c + 1) % 3];
+    b[c * nsite + t] = make_float4(x.re, x.im, y.re, y.im);
+  }
+}
+
+// out = A in, one clover block at a time from shared memory
+__device__ __forceinline__ void sm4_clover(const float4* a, int nsite, int t, const Spinor<float>& in,
+                                           Spinor<float>& out) {
+  const cx<float>* v = &in.c[0][0];
+  cx<float>* o = &out.c[0][0];
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    float r[36];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const float4 w = a[(9 * b + k) * nsite + t];
+      r[4 * k] = w.x;
+      r[4 * k + 1] = w.y;
+      r[4 * k + 2] = w.z;
+      r[4 * k + 3] = w.w;
+    }
+    const cx<float>* x = v + 6 * b;
+    cx<float>* y = o + 6 * b;
+#pragma unroll
+    for (int r0 = 0; r0 < 6; ++r0) y[r0] = r[r0] * x[r0];
+    int k = 0;
+#pragma unroll
+    for (int r0 = 0; r0 < 6; ++r0)
+#pragma unroll
+      for (int c0 = r0 + 1; c0 < 6; ++c0) {
+        const cx<float> off{r[6 + 2 * k], r[7 + 2 * k]};
+        cfma(y[r0], off, x[c0]);
+        cfmac(y[c0], off, x[r0]);
+        ++k;
+      }
+  }
+}
+
+// the sends of a site: U_mu(x)^dag (1 + g_mu) v for its forward neighbours
+template <int MU>
+__device__ __forceinline__ void sm4_send(const SapShared& m, int t, const Su3<float>& u, const Spinor<float>& v) {
+  HalfSpinor<float> h, y;
+  project<MU, +1>(v, h);
+  su3_dag_mul(u, h, y);
+  const cx<float>* c = &y.c[0][0];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    m.s[(MU * 3 + k) * m.nsite + t] = make_float4(c[2 * k].re, c[2 * k].im, c[2 * k + 1].re, c[2 * k + 1].im);
+}
+__device__ __forceinline__ void sm4_publish(const SapShared& m, int t, const Su3<float> (&u)[4],
+                                            const Spinor<float>& v) {
+  sm4_store(m.r, m.nsite, t, v);
+  sm4_send<0>(m, t, u[0], v);
+  sm4_send<1>(m, t, u[1], v);
+  sm4_send<2>(m, t, u[2], v);
+  sm4_send<3>(m, t, u[3], v);
+}
+
+// the in-block hops along mu of the published field; up / down: the site has
+// a neighbour in the block on that side
+template <int MU>
+__device__ __forceinline__ void sm4_hop(const SapShared& m, int t, int stride, bool up, bool down,
+                                        const Su3<float>& u, Spinor<float>& acc) {
+  Spinor<float> nb;
+  sm4_load(m.r, m.nsite, up ? t + stride : t, nb);
+  HalfSpinor<float> h, y, z;
+  const int td = down ? t - stride : t;
+  cx<float>* c = &z.c[0][0];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float4 w = m.s[(MU * 3 + k) * m.nsite + td];
+    c[2 * k] = cx<float>{w.x, w.y};
+    c[2 * k + 1] = cx<float>{w.z, w.w};
+  }
+  project<MU, -1>(nb, h);
+  su3_mul(u, h, y);
+  accum_reconstruct<MU, -1>(acc, y, up ? -0.5f : 0.f);
+  accum_reconstruct<MU, +1>(acc, z, down ? -0.5f : 0.f);
+}
+
+// p = D_i v for the published field v (own value passed in registers)
+__device__ __forceinline__ void sm4_apply(const SapShared& m, int t, const int (&stride)[4], unsigned up,
+                                          unsigned down, const Su3<float> (&u)[4], const Spinor<float>& v,
+                                          Spinor<float>& p) {
+  sm4_clover(m.a, m.nsite, t, v, p);
+  sm4_hop<0>(m, t, stride[0], up & 1, down & 1, u[0], p);
+  sm4_hop<1>(m, t, stride[1], up & 2, down & 2, u[1], p);
+  sm4_hop<2>(m, t, stride[2], up & 4, down & 4, u[2], p);
+  sm4_hop<3>(m, t, stride[3], up & 8, down & 8, u[3], p);
+}
+
+// the hops along mu that come from outside the block, from global memory
+template <int FMT, int MU>
+__device__ __forceinline__ void outer_hop(const SapArgs& a, const char* nbf, int p, const int x[4], bool up,
+                                          bool down, const Su3<float>& u, Spinor<float>& acc) {
+  bool cr;
+  if (!up) {
+    const long j = eo_neighbour(a.g, x, MU, +1, &cr);
+    Spinor<float> nb;
+    load_spinor<P_F32>(nbf, a.g.Vh, j, nb);
+    HalfSpinor<float> h, y;
+    project<MU, -1>(nb, h);
+    su3_mul(u, h, y);
+    hop_accum<MU, -1>(acc, y, -0.5f, cr, a.g.bc_t);
+  }
+  if (!down) {
+    const long j = eo_neighbour(a.g, x, MU, -1, &cr);
+    Spinor<float> nb;
+    load_spinor<P_F32>(nbf, a.g.Vh, j, nb);
+    Su3<float> v;
+    load_link<float, FMT>(a.links, a.g.Vh, 1 - p, MU, j, v);
+    HalfSpinor<float> h, y;
+    project<MU, +1>(nb, h);
+    su3_dag_mul(v, h, y);
+    hop_accum<MU, +1>(acc, y, -0.5f, cr, a.g.bc_t);
+  }
+}
+
+template <int FMT>
+__global__ void __launch_bounds__(256, 1) sap_block_kernel(const SapArgs a) {
+  extern __shared__ float4 sm4[];
+  const int nsite = a.bs[0] * a.bs[1] * a.bs[2] * a.bs[3];
+  SapShared m;
+  m.nsite = nsite;
+  m.a = sm4;
+  m.r = sm4 + 18 * nsite;
+  m.s = sm4 + 24 * nsite;
+  float* red = reinterpret_cast<float*>(sm4 + 36 * nsite);  // 3 partials per warp (binary64: block_sum1)
+  const int t = threadIdx.x;
+  const bool act = t < nsite;
+  const int half3 = a.nb[3] / 2;
+  int row = blockIdx.x / half3;
+  const int mb = blockIdx.x % half3;
+  const int bc2 = row % a.nb[2];
+  row /= a.nb[2];
+  const int bc1 = row % a.nb[1];
+  const int bc0 = row / a.nb[1];
+  const int bc3 = 2 * mb + ((a.colour + bc0 + bc1 + bc2) & 1);
+  const int stride[4] = {a.bs[1] * a.bs[2] * a.bs[3], a.bs[2] * a.bs[3], a.bs[3], 1};
+  int l[4], x[4];
+  {
+    int tt = act ? t : 0;
+    l[3] = tt % a.bs[3];
+    tt /= a.bs[3];
+    l[2] = tt % a.bs[2];
+    tt /= a.bs[2];
+    l[1] = tt % a.bs[1];
+    l[0] = tt / a.bs[1];
+  }
+  x[0] = bc0 * a.bs[0] + l[0];
+  x[1] = bc1 * a.bs[1] + l[1];
+  x[2] = bc2 * a.bs[2] + l[2];
+  x[3] = bc3 * a.bs[3] + l[3];
+  const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
+  const long i = eo_index(a.g, x);
+  unsigned up = 0, down = 0;
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    if (l[mu] + 1 < a.bs[mu]) up |= 1u << mu;
+    if (l[mu] > 0) down |= 1u << mu;
+  }
+  const int w = t >> 5, nw = (blockDim.x + 31) >> 5;
+
+  Spinor<float> r, xs;
+  Su3<float> u[4];
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) r.c[s][c] = xs.c[s][c] = cx<float>{0.f, 0.f};
+  char* phi = a.phi + (long)p * a.half_bytes;
+  if (act) {
+    const float4* q = reinterpret_cast<const float4*>(a.clov) + (long)p * 18 * a.g.Vh + i;
+#pragma unroll
+    for (int k = 0; k < 18; ++k) cp_async16(m.a + k * nsite + t, q + k * a.g.Vh);
+    cp_async_commit();
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) load_link<float, FMT>(a.links, a.g.Vh, p, mu, i, u[mu]);
+    // 1. block residual rho - D phi: the hops from outside the block
+    if (!(a.first && a.colour == 0)) {
+      const char* nbf = a.phi + (long)(1 - p) * a.half_bytes;
+      outer_hop<FMT, 3>(a, nbf, p, x, up & 8, down & 8, u[3], r);
+      outer_hop<FMT, 2>(a, nbf, p, x, up & 4, down & 4, u[2], r);
+      outer_hop<FMT, 1>(a, nbf, p, x, up & 2, down & 2, u[1], r);
+      outer_hop<FMT, 0>(a, nbf, p, x, up & 1, down & 1, u[0], r);
+    }
+    Spinor<float> rh;
+    load_spinor<P_F32>(a.rho + (long)p * a.half_bytes, a.g.Vh, i, rh);
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) r.c[s][c] = rh.c[s][c] - r.c[s][c];
+    if (!a.first) {
+      load_spinor<P_F32>(phi, a.g.Vh, i, xs);  // the block's phi
+      sm4_publish(m, t, u, xs);
+    }
+    cp_async_wait();
+  }
+  __syncthreads();  // the staged clover (each site reads its own) and the published phi
+  if (!a.first) {
+    // the part of D phi inside the block
+    if (act) {
+      Spinor<float> pv;
+      sm4_apply(m, t, stride, up, down, u, xs, pv);
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          r.c[s][c] = r.c[s][c] - pv.c[s][c];
+          xs.c[s][c] = cx<float>{0.f, 0.f};
+        }
+    }
+    __syncthreads();  // every read of the published phi is done
+  }
+  double rn_prev = 0.0;
+  if (a.adaptive) rn_prev = sqrt(block_sum1(act ? site_norm2(r) : 0.0, reinterpret_cast<double*>(red)));
+
+  // 2. MR on D_i
+  int steps = 0;
+  for (int k = 1; k <= a.nmr; ++k) {
+    if (act) sm4_publish(m, t, u, r);
+    __syncthreads();
+    Spinor<float> pv;
+    float d0 = 0.f, d1 = 0.f, d2 = 0.f;  // <p, r>, <p, p>
+    if (act) {
+      sm4_apply(m, t, stride, up, down, u, r, pv);
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const cx<float> q = pv.c[s][c], v = r.c[s][c];
+          d0 += q.re * v.re + q.im * v.im;
+          d1 += q.re * v.im - q.im * v.re;
+          d2 += q.re * q.re + q.im * q.im;
+        }
+    }
+    d0 = warp_sum_f(d0);
+    d1 = warp_sum_f(d1);
+    d2 = warp_sum_f(d2);
+    if ((t & 31) == 0) {
+      red[3 * w] = d0;
+      red[3 * w + 1] = d1;
+      red[3 * w + 2] = d2;
+    }
+    __syncthreads();  // the partial sums; every read of the published residual is done
+    d0 = d1 = d2 = 0.f;
+    for (int j = 0; j < nw; ++j) {
+      d0 += red[3 * j];
+      d1 += red[3 * j + 1];
+      d2 += red[3 * j + 2];
+    }
+    cx<float> om{0.f, 0.f};
+    if (d2 > 0.f) om = cx<float>{d0 / d2, d1 / d2};
+    if (act) {
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          cfma(xs.c[s][c], om, r.c[s][c]);
+          r.c[s][c] = r.c[s][c] - om * pv.c[s][c];
+        }
+    }
+    steps = k;
+    if (a.adaptive) {
+      const double rn_new = sqrt(block_sum1(act ? site_norm2(r) : 0.0, reinterpret_cast<double*>(red)));
+      if ((k >= 4 && rn_new > (double)a.alpha * rn_prev) || rn_new > rn_prev || rn_new < a.tol) break;
+      rn_prev = rn_new;
+    }
+  }
+  // 3. phi_i += x
+  if (act) {
+    if (!a.first) {
+      Spinor<float> ph;
+      load_spinor<P_F32>(phi, a.g.Vh, i, ph);
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) xs.c[s][c] = ph.c[s][c] + xs.c[s][c];
+    }
+    store_spinor<P_F32>(phi, a.g.Vh, i, xs);
+  }
+  if (a.mr_steps && t == 0) atomicAdd(a.mr_steps, (unsigned)steps);
+}
+
+// operands of the even-odd block solver in shared memory
 struct SapSm {
   float* r;        // [24][nsite] block residual
   float2* u;       // [mu][9][nsite] forward links, 18 reals
@@ -324,194 +649,6 @@ __device__ __forceinline__ void sm_clover(const SapSm& m, int t, const Spinor<fl
         ++k;
       }
   }
-}
-
-// in-block hop along +mu / -mu, all operands from shared memory
-template <int MU>
-__device__ __forceinline__ void sm_block_hop(const SapSm& m, const int bs[4], int t, const int l[4],
-                                             Spinor<float>& acc) {
-  int stride = 1;
-  for (int nu = 3; nu > MU; --nu) stride *= bs[nu];
-  if (l[MU] + 1 < bs[MU]) {
-    Spinor<float> nb;
-    load_smem(m.r, m.nsite, t + stride, nb);
-    HalfSpinor<float> h, r;
-    project<MU, -1>(nb, h);
-    Su3<float> u;
-    sm_link(m, MU, t, u);
-    su3_mul(u, h, r);
-    accum_reconstruct<MU, -1>(acc, r, -0.5f);
-  }
-  if (l[MU] > 0) {
-    Spinor<float> nb;
-    load_smem(m.r, m.nsite, t - stride, nb);
-    HalfSpinor<float> h, r;
-    project<MU, +1>(nb, h);
-    Su3<float> u;
-    sm_link(m, MU, t - stride, u);  // U_mu(x - mu): the forward link of the site below
-    su3_dag_mul(u, h, r);
-    accum_reconstruct<MU, +1>(acc, r, -0.5f);
-  }
-}
-
-template <int FMT>
-__global__ void __launch_bounds__(256) sap_smem_kernel(const SapArgs a) {
-  extern __shared__ float4 sm4[];
-  const int nsite = a.bs[0] * a.bs[1] * a.bs[2] * a.bs[3];
-  SapSm m;
-  m.nsite = nsite;
-  m.a = sm4;                                                   // 18 float4 per site
-  m.u = reinterpret_cast<float2*>(sm4 + 18 * nsite);           // 36 float2 per site
-  m.r = reinterpret_cast<float*>(m.u + 36 * nsite);            // 24 floats per site
-  double* red = reinterpret_cast<double*>(m.r + 24 * nsite);
-  const int t = threadIdx.x;
-  const bool act = t < nsite;
-  const int half3 = a.nb[3] / 2;
-  int row = blockIdx.x / half3;
-  const int mb = blockIdx.x % half3;
-  const int bc2 = row % a.nb[2];
-  row /= a.nb[2];
-  const int bc1 = row % a.nb[1];
-  const int bc0 = row / a.nb[1];
-  const int bc3 = 2 * mb + ((a.colour + bc0 + bc1 + bc2) & 1);
-  int l[4], x[4];
-  {
-    int tt = act ? t : 0;
-    l[3] = tt % a.bs[3];
-    tt /= a.bs[3];
-    l[2] = tt % a.bs[2];
-    tt /= a.bs[2];
-    l[1] = tt % a.bs[1];
-    l[0] = tt / a.bs[1];
-  }
-  x[0] = bc0 * a.bs[0] + l[0];
-  x[1] = bc1 * a.bs[1] + l[1];
-  x[2] = bc2 * a.bs[2] + l[2];
-  x[3] = bc3 * a.bs[3] + l[3];
-  const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
-  const long i = eo_index(a.g, x);
-
-  Spinor<float> r;
-  if (act) {
-    // stage the operands: forward links (18 reals) and clover of this site
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-      Su3<float> u;
-      load_link<float, FMT>(a.links, a.g.Vh, p, mu, i, u);
-#pragma unroll
-      for (int k = 0; k < 9; ++k) m.u[(mu * 9 + k) * nsite + t] = make_float2(u.m[k / 3][k % 3].re, u.m[k / 3][k % 3].im);
-    }
-    const float4* q = reinterpret_cast<const float4*>(a.clov) + (long)p * 18 * a.g.Vh;
-#pragma unroll
-    for (int k = 0; k < 18; ++k) m.a[k * nsite + t] = __ldg(q + k * a.g.Vh + i);
-    // 1. block residual r = rho - D phi (full stencil, global operands)
-    HopArgs ha;
-    ha.g = a.g;
-    ha.links = a.links;
-    const char* nbf = a.phi + (long)(1 - p) * a.half_bytes;
-    Spinor<float> acc;
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) acc.c[s][c] = cx<float>{0.f, 0.f};
-    hop_dir<P_F32, FMT, 0, false>(ha, nbf, p, i, x, acc, -0.5f);
-    hop_dir<P_F32, FMT, 1, false>(ha, nbf, p, i, x, acc, -0.5f);
-    hop_dir<P_F32, FMT, 2, false>(ha, nbf, p, i, x, acc, -0.5f);
-    hop_dir<P_F32, FMT, 3, false>(ha, nbf, p, i, x, acc, -0.5f);
-    Spinor<float> ph, aph, rh;
-    load_spinor<P_F32>(a.phi + (long)p * a.half_bytes, a.g.Vh, i, ph);
-    clover_apply<float>(a.clov, a.g.Vh, p, i, ph, aph);
-    load_spinor<P_F32>(a.rho + (long)p * a.half_bytes, a.g.Vh, i, rh);
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) r.c[s][c] = rh.c[s][c] - (aph.c[s][c] + acc.c[s][c]);
-    store_smem(m.r, nsite, t, r);
-  }
-  double n0 = 0.0;
-  if (a.adaptive) {
-    if (act) n0 = site_norm2(r);
-    n0 = block_sum1(n0, red);  // also the barrier after the staging
-  } else {
-    __syncthreads();
-  }
-  double rn_prev = sqrt(n0);
-
-  // 2. MR on D_i, operands in shared memory
-  Spinor<float> xs;
-#pragma unroll
-  for (int s = 0; s < 4; ++s)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) xs.c[s][c] = cx<float>{0.f, 0.f};
-  int steps = 0;
-  for (int k = 1; k <= a.nmr; ++k) {
-    Spinor<float> pv;
-    float pr_re = 0.f, pr_im = 0.f, pp = 0.f;
-    if (act) {
-      Spinor<float> own;
-      load_smem(m.r, nsite, t, own);
-      sm_clover(m, t, own, pv);
-      sm_block_hop<0>(m, a.bs, t, l, pv);
-      sm_block_hop<1>(m, a.bs, t, l, pv);
-      sm_block_hop<2>(m, a.bs, t, l, pv);
-      sm_block_hop<3>(m, a.bs, t, l, pv);
-      float ar = 0.f, ai = 0.f, a2 = 0.f;
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          cx<float> q2 = pv.c[s][c], v = own.c[s][c];
-          ar += q2.re * v.re + q2.im * v.im;
-          ai += q2.re * v.im - q2.im * v.re;
-          a2 += q2.re * q2.re + q2.im * q2.im;
-        }
-      pr_re = ar;
-      pr_im = ai;
-      pp = a2;
-    }
-    block_sum3(pr_re, pr_im, pp, red);  // contains __syncthreads: all neighbour reads done
-    float om_re = 0.f, om_im = 0.f;
-    if (pp > 0.f) {
-      om_re = pr_re / pp;
-      om_im = pr_im / pp;
-    }
-    const cx<float> om{om_re, om_im};
-    double n1 = 0.0;
-    if (act) {
-      Spinor<float> own;
-      load_smem(m.r, nsite, t, own);
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          cfma(xs.c[s][c], om, own.c[s][c]);
-          own.c[s][c] = own.c[s][c] - om * pv.c[s][c];
-        }
-      store_smem(m.r, nsite, t, own);
-      n1 = site_norm2(own);
-    }
-    steps = k;
-    if (a.adaptive) {
-      n1 = block_sum1(n1, red);
-      const double rn_new = sqrt(n1);
-      if ((k >= 4 && rn_new > (double)a.alpha * rn_prev) || rn_new > rn_prev || rn_new < a.tol) break;
-      rn_prev = rn_new;
-    } else {
-      __syncthreads();  // the updated residual is read by the neighbours next step
-    }
-  }
-  // 3. phi_i += x
-  if (act) {
-    char* pp = a.phi + (long)p * a.half_bytes;
-    Spinor<float> ph;
-    load_spinor<P_F32>(pp, a.g.Vh, i, ph);
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) ph.c[s][c] = ph.c[s][c] + xs.c[s][c];
-    store_spinor<P_F32>(pp, a.g.Vh, i, ph);
-  }
-  if (a.mr_steps && t == 0) atomicAdd(a.mr_steps, (unsigned)steps);
 }
 
 // ---------------------------------------------------------------------------
@@ -632,24 +769,28 @@ __global__ void __launch_bounds__(256) sap_smem_eo_kernel(const SapArgs a) {
     const float4* q = reinterpret_cast<const float4*>(p ? a.clov_inv : a.clov) + (long)p * 18 * a.g.Vh;
 #pragma unroll
     for (int k = 0; k < 18; ++k) m.a[k * nsite + t] = __ldg(q + k * a.g.Vh + i);
-    HopArgs ha;
-    ha.g = a.g;
-    ha.links = a.links;
-    const char* nbf = a.phi + (long)(1 - p) * a.half_bytes;
-    Spinor<float> acc;
-    zero_spinor(acc);
-    hop_dir<P_F32, FMT, 0, false>(ha, nbf, p, i, x, acc, -0.5f);
-    hop_dir<P_F32, FMT, 1, false>(ha, nbf, p, i, x, acc, -0.5f);
-    hop_dir<P_F32, FMT, 2, false>(ha, nbf, p, i, x, acc, -0.5f);
-    hop_dir<P_F32, FMT, 3, false>(ha, nbf, p, i, x, acc, -0.5f);
-    Spinor<float> ph, aph, rh;
-    load_spinor<P_F32>(a.phi + (long)p * a.half_bytes, a.g.Vh, i, ph);
-    clover_apply<float>(a.clov, a.g.Vh, p, i, ph, aph);
+    Spinor<float> rh;
     load_spinor<P_F32>(a.rho + (long)p * a.half_bytes, a.g.Vh, i, rh);
+    r = rh;
+    if (!(a.first && a.colour == 0)) {  // phi is zero before the first half cycle
+      HopArgs ha;
+      ha.g = a.g;
+      ha.links = a.links;
+      const char* nbf = a.phi + (long)(1 - p) * a.half_bytes;
+      Spinor<float> acc;
+      zero_spinor(acc);
+      hop_dir<P_F32, FMT, 0, false>(ha, nbf, p, i, x, acc, -0.5f);
+      hop_dir<P_F32, FMT, 1, false>(ha, nbf, p, i, x, acc, -0.5f);
+      hop_dir<P_F32, FMT, 2, false>(ha, nbf, p, i, x, acc, -0.5f);
+      hop_dir<P_F32, FMT, 3, false>(ha, nbf, p, i, x, acc, -0.5f);
+      Spinor<float> ph, aph;
+      load_spinor<P_F32>(a.phi + (long)p * a.half_bytes, a.g.Vh, i, ph);
+      clover_apply<float>(a.clov, a.g.Vh, p, i, ph, aph);
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
+      for (int s = 0; s < 4; ++s)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) r.c[s][c] = rh.c[s][c] - (aph.c[s][c] + acc.c[s][c]);
+        for (int c = 0; c < 3; ++c) r.c[s][c] = rh.c[s][c] - (aph.c[s][c] + acc.c[s][c]);
+    }
   }
   __syncthreads();  // the staged links and clover are read by the neighbours below
   // odd sites: w_o = A^{-1} r_o into the shared field
@@ -772,16 +913,24 @@ __global__ void __launch_bounds__(256) sap_smem_eo_kernel(const SapArgs a) {
   if (a.mr_steps && t == 0) atomicAdd(a.mr_steps, (unsigned)steps);
 }
 
-size_t sap_smem_bytes(const int bs[4]) {
+// operands in shared memory: clover, links and residual (even-odd kernel), or
+// clover, residual and sends (sap_block_kernel); at most 172 KB for 256 sites
+static size_t sap_smem_bytes(const int bs[4], int words) {
   const int nsite = bs[0] * bs[1] * bs[2] * bs[3];
   const int threads = (nsite + 31) / 32 * 32;
-  return sizeof(float) * (72 + 72 + 24) * (size_t)nsite + sizeof(double) * 3 * (threads / 32);
+  return sizeof(float) * words * (size_t)nsite + sizeof(double) * 3 * (threads / 32);
 }
 
 cudaError_t sap_colour(const Geom& g, const int bs[4], int colour, int fmt, const void* links, const void* clov,
                        const void* clov_inv, const void* rho, void* phi, int nmr, int adaptive, float alpha,
-                       double tol, unsigned* mr_steps, int kernel, int eo, cudaStream_t s) {
+                       double tol, unsigned* mr_steps, int kernel, int eo, int cycle, cudaStream_t s) {
   SapArgs a;
+  a.first = cycle == 0;
+  // every block is written in the first cycle; the kernels that read phi there need zeros
+  if (cycle == 0 && colour == 0 && (eo || kernel != 0)) {
+    const cudaError_t e = cudaMemsetAsync(phi, 0, 2 * spinor_half_bytes(g.Vh, P_F32), s);
+    if (e != cudaSuccess) return e;
+  }
   a.g = g;
   int nblk = 1;
   for (int mu = 0; mu < 4; ++mu) {
@@ -807,7 +956,7 @@ cudaError_t sap_colour(const Geom& g, const int bs[4], int colour, int fmt, cons
   dim3 grid(nblk / 2), block(threads);
   if (eo) {
     // even-odd reduced block solver: shared-memory operands only
-    const size_t sm2 = sap_smem_bytes(bs);
+    const size_t sm2 = sap_smem_bytes(bs, 72 + 72 + 24);
     if (sm2 > 227 * 1024 || !clov_inv || bs[3] % 2) return cudaErrorInvalidValue;
     if (fmt == LINK_12) {
       cudaFuncSetAttribute(sap_smem_eo_kernel<LINK_12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
@@ -818,20 +967,16 @@ cudaError_t sap_colour(const Geom& g, const int bs[4], int colour, int fmt, cons
     }
     return cudaGetLastError();
   }
-  if (kernel == 0) {
-    // operands in shared memory (the default), if they fit
-    const size_t sm2 = sap_smem_bytes(bs);
-    if (sm2 <= 227 * 1024) {
-      if (fmt == LINK_12) {
-        cudaFuncSetAttribute(sap_smem_kernel<LINK_12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-        sap_smem_kernel<LINK_12><<<grid, block, sm2, s>>>(a);
-      } else {
-        cudaFuncSetAttribute(sap_smem_kernel<LINK_18>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-        sap_smem_kernel<LINK_18><<<grid, block, sm2, s>>>(a);
-      }
-      return cudaGetLastError();
+  if (kernel == 0) {  // the default
+    const size_t sm2 = sap_smem_bytes(bs, 72 + 24 + 48);
+    if (fmt == LINK_12) {
+      cudaFuncSetAttribute(sap_block_kernel<LINK_12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+      sap_block_kernel<LINK_12><<<grid, block, sm2, s>>>(a);
+    } else {
+      cudaFuncSetAttribute(sap_block_kernel<LINK_18>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+      sap_block_kernel<LINK_18><<<grid, block, sm2, s>>>(a);
     }
-    kernel = 2;
+    return cudaGetLastError();
   }
   if (kernel == 2) {
     if (fmt == LINK_12)
