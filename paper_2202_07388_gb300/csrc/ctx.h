@@ -284,6 +284,23 @@ struct oq_ctx {
     } else if (nrhs == 1) {
       l.bx = 128;
       l.by = 1;
+    } else if ((prec == oq::P_F32 || prec == oq::P_BF16 || prec == oq::P_F16) && !lats[lat].halo_t) {
+      // Several right-hand sides of a binary32-arithmetic type: two per thread,
+      // so that links, clover and indices serve both.  64-site CTAs: staged
+      // hops at 168 registers for the 16-bit types on 12-real links, else
+      // capped at 128 registers; within 10 % of the tuner's choice from 8^4 to
+      // 48x24^3 with 2 to 12 rhs, where one rhs per thread in 32 x nrhs CTAs
+      // took 1.2 to 1.9 times as long (12 rhs F16 Dhat on 48x24^3: 495 against
+      // 814 us; 4 rhs F32 on 32x16^3: 62 against 78 us; 8^4: 16 us either way).
+      // The reductions of the norm and CG epilogues want more threads on small
+      // problems: below 2^18 (norm) or 2^17 (CG) site-rhs one rhs per thread
+      // (where the tuner's choice changes between 16^4 and 32x16^3).
+      const long work = lats[lat].g.Vh * nrhs;
+      const bool few = (epi == oq::EPI_NORM && work < (1L << 18)) || (epi == oq::EPI_CG && work < (1L << 17));
+      l.bx = 64;
+      l.by = 1;
+      l.nr = few ? 1 : 2;
+      l.regcap = few ? 0 : (prec != oq::P_F32 && l.link_fmt == oq::LINK_12) ? 3 : 1;
     } else {
       // several right-hand sides: 32 sites x (largest divisor of nrhs <= 8) rows
       l.bx = 32;
