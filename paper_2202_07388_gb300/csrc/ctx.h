@@ -281,6 +281,15 @@ struct oq_ctx {
       l.nr = it->second.nr;
       l.regcap = it->second.regcap;
       if (it->second.link_fmt >= 0) l.link_fmt = it->second.link_fmt;
+    } else if (prec == oq::P_DF64 && !lats[lat].halo_t) {
+      // the double-float site is latency- and issue-bound: 12 warps per SM at
+      // 168 registers (Dhat, 12 rhs on 48x24^3: 4.0 ms against 6.5 ms
+      // uncapped in 32 x 6 CTAs, 4 rhs on 32x16^3: 304 against 370 us), 16
+      // with some spilling where a launch fills few waves (1 rhs on 32x16^3:
+      // 113 against 121 us)
+      l.bx = 128;
+      l.by = 1;
+      l.regcap = lats[lat].g.Vh * nrhs < (1L << 17) ? 1 : 2;
     } else if (nrhs == 1) {
       l.bx = 128;
       l.by = 1;

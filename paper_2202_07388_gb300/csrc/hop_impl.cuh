@@ -17,6 +17,7 @@
 // (norm of the output, the CG update of x and r, or the binary64 residual
 // eta - out of a reset step) with a deterministic binary64 grid reduction.
 #pragma once
+#include "df_pack.cuh"
 #include "reduce.cuh"
 
 namespace oq {
@@ -80,28 +81,47 @@ __device__ __forceinline__ void hop_dir(const HopArgs& a, const char* in, int p,
   }
 }
 
-// z * i^c for c in 0..3 (double-float): a swap of the parts for odd c and
-// sign flips, all by selects
-__device__ __forceinline__ cx<dfloat> rot_ic(const cx<dfloat>& z, int c) {
-  const bool sw = c & 1;
-  dfloat re = sw ? z.im : z.re, im = sw ? z.re : z.im;
-  if (c == 1 || c == 2) re = -re;
-  if (c >= 2) im = -im;
-  return cx<dfloat>{re, im};
-}
-
-// The hopping sum in double-float as one runtime loop over the 8 hops: the
-// fully unrolled double-float stencil is ~14k instructions, far beyond the
-// instruction cache, while one loop body (~1k) stays resident.  The spin
+// The double-float site, one right-hand side per thread, two lanes per
+// instruction (df_pack.cuh).  In the hops the lanes are the two spins of the
+// half spinor (the link is shared, the upper and lower spin pairs of the sum
+// are two lanes each); in the clover term they are the two chiral blocks.  No
+// lane belongs to another right-hand side, so the kernel keeps the registers
+// of a scalar one (the two-rhs form of hop_df2.cuh needs 255).
+//
+// The hopping sum is one runtime loop over the 8 hops: unrolled, the
+// double-float stencil is far beyond the instruction cache.  The spin
 // projection for hop (mu, projector sign S) is h0 = p0 + i^c0 p[q0],
 // h1 = p1 + i^c1 p[q1], the reconstruction acc2 += i^d0 t[r0],
-// acc3 += i^d1 t[r1] (the same linear maps as project / accum_reconstruct,
-// as tables; S = +1 adds 2 to every power); a backward hop applies
-// U(x - mu)^dag by conjugate-transposing the link in registers.
-template <int P, int FMT, bool DAG>
-__device__ __forceinline__ void hop_loop_df(const HopArgs& a, const char* in, int p, long i, const int x[4],
-                                            Spinor<dfloat>& acc) {
+// acc3 += i^d1 t[r1] (the maps of project / accum_reconstruct as tables;
+// S = +1 adds 2 to every power): c0 and c1 (d0 and d1) are both even or both
+// odd, so a power of i is one exchange of the real and imaginary pairs and
+// per-lane signs.  A backward hop reads the link transposed and moves the
+// conjugation into signed copies of h.
+// 12 rhs on 48x24^3, both Dhat passes: 4.0 ms against 4.7 ms for the scalar
+// form (16.5k instructions per site, 55 % of the binary32 pipe), each in its best
+// launch; 1 rhs: 420 against 475 us.
+namespace dfs {
+using namespace df2;
+
+// (sign of the real part, of the imaginary part) that i^c brings, see i_pow
+__device__ __forceinline__ float ic_re(int c) { return (c & 3) == 1 || (c & 3) == 2 ? -1.f : 1.f; }
+__device__ __forceinline__ float ic_im(int c) { return (c & 3) >= 2 ? -1.f : 1.f; }
+// z i^c per lane: odd = the powers are odd, (sr, si) their signs
+__device__ __forceinline__ C2 i_pow(const C2& z, bool odd, F2 sr, F2 si) {
+  return C2{dsign(odd ? z.im : z.re, sr), dsign(odd ? z.re : z.im, si)};
+}
+// complex chunks of two components as a pair
+__device__ __forceinline__ C2 pair(const float4& a, const float4& b) {
+  return C2{D2{make_float2(a.x, b.x), make_float2(a.y, b.y)}, D2{make_float2(a.z, b.z), make_float2(a.w, b.w)}};
+}
+
+// up[c], lo[c]: colour c of the spin pairs (0, 1) and (2, 3); the hops are
+// added without renormalising
+template <bool DAG>
+__device__ __forceinline__ void hop_loop(const HopArgs& a, const float4* in, int p, long i, const int x[4],
+                                         C2 (&up)[3], C2 (&lo)[3]) {
   constexpr int SF = DAG ? +1 : -1;  // projector sign of the forward hop
+  const long Vh = a.g.Vh;
 #pragma unroll 1
   for (int k = 0; k < 8; ++k) {
     const int mu = k >> 1;
@@ -109,56 +129,197 @@ __device__ __forceinline__ void hop_loop_df(const HopArgs& a, const char* in, in
     const int sh = ((fwd ? SF : -SF) > 0) ? 2 : 0;
     bool cr;
     const long j = eo_neighbour_rt(a.g, x, mu, fwd ? +1 : -1, &cr);
-    Spinor<dfloat> nb;
-    load_spinor<P>(in, a.g.Vh, j, nb);
-    Su3<dfloat> u;
-    load_link<dfloat, FMT>(a.links, a.g.Vh, fwd ? p : 1 - p, mu, fwd ? i : j, u);
-    if (!fwd) {
-      Su3<dfloat> v = u;
+    // the link's elements (row r, column c), transposed for a backward hop
+    const float4* ub =
+        reinterpret_cast<const float4*>(a.links) + ((long)((fwd ? p : 1 - p) * 4 + mu) * 9) * Vh + (fwd ? i : j);
+    const long sr = fwd ? 3 * Vh : Vh, sc = fwd ? Vh : 3 * Vh;
+    float4 u[3][3];
 #pragma unroll
-      for (int r = 0; r < 3; ++r)
+    for (int r = 0; r < 3; ++r)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) u.m[r][c] = conj(v.m[c][r]);
-    }
-    // projection tables (mu = 0..3): partners q0, q1 and powers of i
-    const bool swq = (mu == 1 || mu == 2);       // q0 = 3, q1 = 2
+      for (int c = 0; c < 3; ++c) u[r][c] = ldg_nc(ub + r * sr + c * sc);
+    const bool swq = (mu == 1 || mu == 2);  // q0 = 3, q1 = 2 (r0 = 1, r1 = 0)
     const int c0 = ((mu == 1 || mu == 3) ? 1 : 0) + sh;
     const int c1 = (mu == 0 ? 0 : mu == 1 ? 1 : mu == 2 ? 2 : 3) + sh;
-    HalfSpinor<dfloat> h, t;
+    const F2 csr = make_float2(ic_re(c0), ic_re(c1)), csi = make_float2(ic_im(c0), ic_im(c1));
+    const float4* nb = in + j;
+    const float4* nq0 = nb + (swq ? 9 : 6) * Vh;
+    const float4* nq1 = nb + (swq ? 6 : 9) * Vh;
+    C2 h[3], g[3];  // the half spinor; its copy for the imaginary parts of the link
+    const F2 cj = bc(fwd ? 1.f : -1.f);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const cx<dfloat> pa = swq ? nb.c[3][c] : nb.c[2][c];
-      const cx<dfloat> pb = swq ? nb.c[2][c] : nb.c[3][c];
-      const cx<dfloat> ra = rot_ic(pa, c0 & 3), rb = rot_ic(pb, c1 & 3);
-      h.c[0][c] = cx<dfloat>{df_add_lazy(nb.c[0][c].re, ra.re), df_add_lazy(nb.c[0][c].im, ra.im)};
-      h.c[1][c] = cx<dfloat>{df_add_lazy(nb.c[1][c].re, rb.re), df_add_lazy(nb.c[1][c].im, rb.im)};
+      const C2 n = pair(ldg_nc(nb + c * Vh), ldg_nc(nb + (3 + c) * Vh));
+      const C2 m = i_pow(pair(ldg_nc(nq0 + c * Vh), ldg_nc(nq1 + c * Vh)), c0 & 1, csr, csi);
+      h[c] = C2{add_lazy(n.re, m.re), add_lazy(n.im, m.im)};
+      // u h = (ur + i s ui) h: re += ui (-s h.im), im += ui (s h.re), s = +-1
+      g[c] = C2{dsign(h[c].re, cj), dneg(dsign(h[c].im, cj))};
     }
-    su3_mul(u, h, t);
-    if (cr && a.g.bc_t < 0.f) {
-#pragma unroll
-      for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) t.c[s][c] = -t.c[s][c];
-    }
-    // reconstruction tables: r0 = 1, r1 = 0 for mu = 1, 2
+    const bool flip = cr && a.g.bc_t < 0.f;
     const int d0 = (mu == 0 ? 0 : mu == 1 ? 3 : mu == 2 ? 2 : 3) + sh;
     const int d1 = (mu == 0 ? 0 : mu == 1 ? 3 : mu == 2 ? 0 : 1) + sh;
+    const F2 dsr = make_float2(ic_re(d0), ic_re(d1)), dsi = make_float2(ic_im(d0), ic_im(d1));
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const cx<dfloat> ta = rot_ic(swq ? t.c[1][c] : t.c[0][c], d0 & 3);
-      const cx<dfloat> tb = rot_ic(swq ? t.c[0][c] : t.c[1][c], d1 & 3);
-      const cx<dfloat> up[4] = {t.c[0][c], t.c[1][c], ta, tb};
+    for (int r = 0; r < 3; ++r) {
+      Acc re, im;
 #pragma unroll
-      for (int s2 = 0; s2 < 4; ++s2)
-        acc.c[s2][c] = cx<dfloat>{df_add_lazy(acc.c[s2][c].re, up[s2].re), df_add_lazy(acc.c[s2][c].im, up[s2].im)};
+      for (int b = 0; b < 3; ++b) {
+        const dfloat ur(u[r][b].x, u[r][b].y), ui(u[r][b].z, u[r][b].w);
+        if (b == 0) {
+          acc_first(re, ur, h[b].re);
+          acc_first(im, ur, h[b].im);
+        } else {
+          acc_add(re, ur, h[b].re);
+          acc_add(im, ur, h[b].im);
+        }
+        acc_add(re, ui, g[b].im);
+        acc_add(im, ui, g[b].re);
+      }
+      C2 t{acc_get(re), acc_get(im)};
+      if (flip) t = cneg(t);
+      up[r] = C2{add_lazy(up[r].re, t.re), add_lazy(up[r].im, t.im)};
+      if (swq) {  // exchange the lanes
+        t.re = D2{make_float2(t.re.hi.y, t.re.hi.x), make_float2(t.re.lo.y, t.re.lo.x)};
+        t.im = D2{make_float2(t.im.hi.y, t.im.hi.x), make_float2(t.im.lo.y, t.im.lo.x)};
+      }
+      const C2 l = i_pow(t, d0 & 1, dsr, dsi);
+      lo[r] = C2{add_lazy(lo[r].re, l.re), add_lazy(lo[r].im, l.im)};
     }
   }
-  // the hops were summed without renormalising
 #pragma unroll
-  for (int s2 = 0; s2 < 4; ++s2)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) acc.c[s2][c] = cx<dfloat>{df_norm(acc.c[s2][c].re), df_norm(acc.c[s2][c].im)};
+  for (int r = 0; r < 3; ++r) {
+    up[r] = C2{dnorm(up[r].re), dnorm(up[r].im)};
+    lo[r] = C2{dnorm(lo[r].re), dnorm(lo[r].im)};
+  }
 }
+
+// y = K x for both chiral blocks of a site (lane b: block b, component r =
+// 3 (local spin) + colour); every component's products are summed in the order
+// of its row (diagonal first), one entry of the blocks in registers at a time
+__device__ __forceinline__ void clover(const void* base, long Vh, int p, long i, const C2 (&x)[6], C2 (&y)[6]) {
+  const float4* q = reinterpret_cast<const float4*>(base) + (long)p * 36 * Vh + i;
+  Acc re[6], im[6];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float4 w0 = ldg_nc(q + k * Vh), w1 = ldg_nc(q + (18 + k) * Vh);
+    const D2 da{make_float2(w0.x, w1.x), make_float2(w0.y, w1.y)}, db{make_float2(w0.z, w1.z), make_float2(w0.w, w1.w)};
+    acc_first(re[2 * k], da, x[2 * k].re);
+    acc_first(im[2 * k], da, x[2 * k].im);
+    acc_first(re[2 * k + 1], db, x[2 * k + 1].re);
+    acc_first(im[2 * k + 1], db, x[2 * k + 1].im);
+  }
+  int n = 0;
+#pragma unroll
+  for (int r = 0; r < 6; ++r)
+#pragma unroll
+    for (int c = r + 1; c < 6; ++c) {
+      const C2 o = pair(ldg_nc(q + (3 + n) * Vh), ldg_nc(q + (21 + n) * Vh));
+      ++n;
+      // y[r] += o x[c]
+      acc_add(re[r], o.re, x[c].re);
+      acc_add(re[r], o.im, dneg(x[c].im));
+      acc_add(im[r], o.re, x[c].im);
+      acc_add(im[r], o.im, x[c].re);
+      // y[c] += conj(o) x[r]
+      acc_add(re[c], o.re, x[r].re);
+      acc_add(re[c], o.im, x[r].im);
+      acc_add(im[c], o.re, x[r].im);
+      acc_add(im[c], o.im, dneg(x[r].re));
+    }
+#pragma unroll
+  for (int r = 0; r < 6; ++r) y[r] = C2{acc_get(re[r]), acc_get(im[r])};
+}
+
+// lanes (spin 0, spin 1) / (2, 3) of colour c <-> lanes (block 0, block 1) of
+// component r = 3 s + c
+__device__ __forceinline__ D2 lanes(D2 a, int la, D2 b, int lb) {
+  return D2{make_float2(la ? a.hi.y : a.hi.x, lb ? b.hi.y : b.hi.x),
+            make_float2(la ? a.lo.y : a.lo.x, lb ? b.lo.y : b.lo.x)};
+}
+__device__ __forceinline__ C2 lanes(const C2& a, int la, const C2& b, int lb) {
+  return C2{lanes(a.re, la, b.re, lb), lanes(a.im, la, b.im, lb)};
+}
+__device__ __forceinline__ cx<dfloat> lane(const C2& z, int l) {
+  return cx<dfloat>{dfloat(l ? z.re.hi.y : z.re.hi.x, l ? z.re.lo.y : z.re.lo.x),
+                    dfloat(l ? z.im.hi.y : z.im.hi.x, l ? z.im.lo.y : z.im.lo.x)};
+}
+
+// One output site i (parity p) of right-hand side rhs; the site's
+// contribution to the residual epilogue's norm (0 otherwise).  A in2 / w is
+// formed first (w = +-1/2, so the scaling is exact), the unweighted hops add
+// onto it and one final scaling gives A in2 + w H in.
+template <int MODE, bool DAG, int EPI>
+__device__ __forceinline__ double site(const HopArgs& a, long i, int rhs, int p) {
+  int x[4];
+  eo_coords(a.g, p, i, x);
+  const long Vh = a.g.Vh;
+  const long par_in = (MODE == HOP_DW) ? (long)(1 - p) * a.half_bytes : 0;
+  const long par_out = (MODE == HOP_DW) ? (long)p * a.half_bytes : 0;
+  const float4* in = reinterpret_cast<const float4*>((const char*)a.in + rhs * a.in_stride + par_in);
+  constexpr float w = (MODE == HOP_P2) ? 0.5f : -0.5f;
+  C2 up[3], lo[3], v[6], y[6];
+  if constexpr (MODE != HOP_P1) {
+    const float4* l = reinterpret_cast<const float4*>((const char*)a.in2 + rhs * a.in2_stride + par_out) + i;
+#pragma unroll
+    for (int r = 0; r < 6; ++r) v[r] = pair(ldg_nc(l + r * Vh), ldg_nc(l + (6 + r) * Vh));
+    clover(a.clov, Vh, p, i, v, y);
+#pragma unroll
+    for (int r = 0; r < 6; ++r) y[r] = C2{dscale(y[r].re, 1.f / w), dscale(y[r].im, 1.f / w)};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      up[c] = lanes(y[c], 0, y[3 + c], 0);
+      lo[c] = lanes(y[c], 1, y[3 + c], 1);
+    }
+  } else {
+    const D2 z{bc(0.f), bc(0.f)};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) up[c] = lo[c] = C2{z, z};
+  }
+  hop_loop<DAG>(a, in, p, i, x, up, lo);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    up[c] = C2{dscale(up[c].re, w), dscale(up[c].im, w)};
+    lo[c] = C2{dscale(lo[c].re, w), dscale(lo[c].im, w)};
+  }
+  Spinor<dfloat> res;
+  if constexpr (MODE == HOP_P1) {
+#pragma unroll
+    for (int r = 0; r < 6; ++r) v[r] = lanes(up[r % 3], r / 3, lo[r % 3], r / 3);
+    clover(a.cinv, Vh, p, i, v, y);
+#pragma unroll
+    for (int r = 0; r < 6; ++r) {
+      res.c[r / 3][r % 3] = lane(y[r], 0);
+      res.c[2 + r / 3][r % 3] = lane(y[r], 1);
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      res.c[0][c] = lane(up[c], 0);
+      res.c[1][c] = lane(up[c], 1);
+      res.c[2][c] = lane(lo[c], 0);
+      res.c[3][c] = lane(lo[c], 1);
+    }
+  }
+  double red = 0.0;
+  if constexpr (EPI == EPI_RESID64) {
+    Spinor<dfloat> e;
+    load_spinor<P_DF64>((const char*)a.ep_eta + rhs * a.ep_eta_stride, Vh, i, e);
+    // the site's 24 squares summed in double-float, one conversion
+    dfloat acc2(0.f);
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        res.c[s][c] = e.c[s][c] - res.c[s][c];
+        acc2 = fma(res.c[s][c].re, res.c[s][c].re, fma(res.c[s][c].im, res.c[s][c].im, acc2));
+      }
+    red = (double)acc2;
+  }
+  store_spinor<P_DF64>((char*)a.out + rhs * a.out_stride + par_out, Vh, i, res);
+  return red;
+}
+
+}  // namespace dfs
 
 // value type of a site's reduction contribution: binary32 for the
 // binary32-arithmetic types (their per-site norms are binary32 sums), else
@@ -171,8 +332,11 @@ using RedT = typename std::conditional<P == P_F64 || P == P_DF64, double, float>
 // epilogue's reduction (0 if none).
 template <int P, int FMT, int MODE, bool DAG, int EPI>
 __device__ __forceinline__ RedT<P> hop_site(const HopArgs& a, long i, int rhs, int p) {
-  typedef typename PrecTraits<P>::R R;
-  RedT<P> red = 0;
+  if constexpr (P == P_DF64) {
+    return dfs::site<MODE, DAG, EPI>(a, i, rhs, p);
+  } else {
+    typedef typename PrecTraits<P>::R R;
+    RedT<P> red = 0;
     int x[4];
     eo_coords(a.g, p, i, x);
     const long par_in = (MODE == HOP_DW) ? (long)(1 - p) * a.half_bytes : 0;
@@ -184,54 +348,29 @@ __device__ __forceinline__ RedT<P> hop_site(const HopArgs& a, long i, int rhs, i
 #pragma unroll
       for (int c = 0; c < 3; ++c) acc.c[s][c] = cx<R>{0, 0};
     const R w = (MODE == HOP_P2) ? (R)0.5 : (R)-0.5;
-    constexpr bool DF = std::is_same<R, dfloat>::value, F64 = std::is_same<R, double>::value;
-    if constexpr (DF && MODE != HOP_P1) {
-      // double-float: A in2 / w first (w = +-1/2, so the scaling is exact)
-      // while few registers are live; the unweighted hops add onto it and
-      // one final scaling by w gives A in2 + w H in
-      Spinor<R> loc;
-      load_spinor<P>((const char*)a.in2 + rhs * a.in2_stride + par_out, a.g.Vh, i, loc);
-      clover_apply<R>(a.clov, a.g.Vh, p, i, loc, acc);
-      const float iw = 1.f / w.hi;
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-          acc.c[s][c] = cx<R>{df_scale(acc.c[s][c].re, iw), df_scale(acc.c[s][c].im, iw)};
-    }
+    constexpr bool F64 = std::is_same<R, double>::value;
     if constexpr (F64 && MODE != HOP_P1) {
       // binary64: the hops add onto A in2 (24 additions fewer on the binary64 pipe)
       Spinor<R> loc;
       load_spinor<P>((const char*)a.in2 + rhs * a.in2_stride + par_out, a.g.Vh, i, loc);
       clover_apply<R>(a.clov, a.g.Vh, p, i, loc, acc);
     }
-    if constexpr (DF) {
-      hop_loop_df<P, FMT, DAG>(a, in, p, i, x, acc);
-    } else {
-      const char* fn = nullptr;
-      const char* fp = nullptr;
-      if (a.halo_next) {  // sub-domain launch: faces of this rhs and output parity
-        const long po = (MODE == HOP_DW) ? (long)p * a.halo_pstride : 0;
-        fn = (const char*)a.halo_next + rhs * a.halo_stride + po;
-        fp = (const char*)a.halo_prev + rhs * a.halo_stride + po;
-      }
-      hop_dir<P, FMT, 0, DAG>(a, in, p, i, x, acc, w, fn, fp);
-      hop_dir<P, FMT, 1, DAG>(a, in, p, i, x, acc, w);
-      hop_dir<P, FMT, 2, DAG>(a, in, p, i, x, acc, w);
-      hop_dir<P, FMT, 3, DAG>(a, in, p, i, x, acc, w);
+    const char* fn = nullptr;
+    const char* fp = nullptr;
+    if (a.halo_next) {  // sub-domain launch: faces of this rhs and output parity
+      const long po = (MODE == HOP_DW) ? (long)p * a.halo_pstride : 0;
+      fn = (const char*)a.halo_next + rhs * a.halo_stride + po;
+      fp = (const char*)a.halo_prev + rhs * a.halo_stride + po;
     }
-    if constexpr (DF) {
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-          acc.c[s][c] = cx<R>{df_scale(acc.c[s][c].re, w.hi), df_scale(acc.c[s][c].im, w.hi)};
-    }
+    hop_dir<P, FMT, 0, DAG>(a, in, p, i, x, acc, w, fn, fp);
+    hop_dir<P, FMT, 1, DAG>(a, in, p, i, x, acc, w);
+    hop_dir<P, FMT, 2, DAG>(a, in, p, i, x, acc, w);
+    hop_dir<P, FMT, 3, DAG>(a, in, p, i, x, acc, w);
 
     Spinor<R> res;
     if constexpr (MODE == HOP_P1) {
       clover_apply<R>(a.cinv, a.g.Vh, p, i, acc, res);
-    } else if constexpr (DF || F64) {
+    } else if constexpr (F64) {
       res = acc;
     } else {
       const char* in2 = (const char*)a.in2 + rhs * a.in2_stride + par_out;
@@ -280,27 +419,18 @@ __device__ __forceinline__ RedT<P> hop_site(const HopArgs& a, long i, int rhs, i
 #pragma unroll
         for (int c = 0; c < 3; ++c) res.c[s][c] = e.c[s][c] - res.c[s][c];
       store_spinor<P>((char*)a.out + rhs * a.out_stride, a.g.Vh, i, res);
-      if constexpr (P == P_DF64) {
-        // the site's 24 squares summed in double-float, one conversion
-        dfloat acc2(0.f);
+      double acc2 = 0.0;
 #pragma unroll
-        for (int s = 0; s < 4; ++s)
+      for (int s = 0; s < 4; ++s)
 #pragma unroll
-          for (int c = 0; c < 3; ++c) acc2 = fma(res.c[s][c].re, res.c[s][c].re, fma(res.c[s][c].im, res.c[s][c].im, acc2));
-        red = (double)acc2;
-      } else {
-        double acc2 = 0.0;
-#pragma unroll
-        for (int s = 0; s < 4; ++s)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const double re = (double)res.c[s][c].re, im = (double)res.c[s][c].im;
-            acc2 += re * re + im * im;
-          }
-        red = acc2;
-      }
+        for (int c = 0; c < 3; ++c) {
+          const double re = (double)res.c[s][c].re, im = (double)res.c[s][c].im;
+          acc2 += re * re + im * im;
+        }
+      red = acc2;
     }
-  return red;
+    return red;
+  }
 }
 
 template <int P, int FMT, int MODE, bool DAG, int EPI>
