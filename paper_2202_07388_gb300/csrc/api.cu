@@ -35,6 +35,23 @@ cudaError_t launch_hop(const HopLaunch& L, const HopArgs& a, cudaStream_t s) {
   }
   return cudaErrorInvalidValue;
 }
+
+cudaError_t launch_hop_reduced(const HopLaunch& L, const HopArgs& a, cudaStream_t s, long long* kernels) {
+  *kernels += 1;
+  const unsigned nb = (unsigned)((a.g.Vh + L.bx - 1) / L.bx);
+  const unsigned rows = (unsigned)((a.nrhs + L.by * L.nr - 1) / (L.by * L.nr));
+  // From 2048 CTAs (several per SM one after the other) the CTAs' waits cost
+  // more than the extra launch: 12 rhs F16 on 48x24^3, norm 312 against 365 us,
+  // CG 432 against 475 us; 1 rhs F32 (2592 CTAs) 73 against 76 us; 32x16^3
+  // (512 CTAs) 19.0 against 18.7 us.
+  if (L.epi == EPI_NONE || nb * rows < 2048u) return launch_hop(L, a, s);
+  HopArgs b = a;
+  b.red.defer = 1;
+  const cudaError_t e = launch_hop(L, b, s);
+  if (e != cudaSuccess) return e;
+  *kernels += 1;
+  return reduce_finish(b.red, a.nrhs, nb, s);
+}
 }  // namespace oq
 
 extern "C" const char* oq_error_string(int code) {

@@ -264,6 +264,7 @@ extern "C" int oq_cgne_solve_batch(oq_handle h, int nsys, const int* lats, const
     r.cg = cg + s2;
     r.fin = fin;
     r.gate = gate;
+    r.defer = 0;
     return r;
   };
   // argument sets: 0 P1, 1 P2+norm, 2 P1^dag, 3 P2^dag+CG (small type); 4..7 the binary64 reset

@@ -92,6 +92,32 @@ cudaError_t reduce_dot(int prec, const void* x, const void* y, long Vh, long str
   return cudaGetLastError();
 }
 
+// the partials of right-hand side blockIdx.x, summed by one CTA in a fixed
+// order (thread t: t, t + 256, ...; then the threads by warps), and the finisher
+__global__ void __launch_bounds__(RED_BX) reduce_finish_kernel(RedArgs ra, unsigned ncta) {
+  __shared__ double smem[RED_BX / 32];
+  const int rhs = blockIdx.x;
+  if (ra.fin != FIN_STORE && ra.cg[rhs].mode != ra.gate) return;  // not live in the launch
+  const double* part = ra.partials + (long)rhs * ncta;
+  double acc = 0.0;
+#pragma unroll 4
+  for (unsigned k = threadIdx.x; k < ncta; k += RED_BX) acc += part[k];
+  acc = warp_sum(acc);
+  if ((threadIdx.x & 31) == 0) smem[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < RED_BX / 32; ++w) s += smem[w];
+    run_finisher(ra, rhs, s);
+  }
+}
+
+cudaError_t reduce_finish(const RedArgs& ra, int nrhs, unsigned ncta, cudaStream_t s) {
+  reduce_finish_kernel<<<nrhs, RED_BX, 0, s>>>(ra, ncta);
+  return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------------------
 // CGNE vector steps
 // ---------------------------------------------------------------------------

@@ -225,6 +225,7 @@ struct oq_ctx {
     r.cg = cg_dev;
     r.fin = fin;
     r.gate = gate;
+    r.defer = 0;
     return r;
   }
 
@@ -394,8 +395,7 @@ struct oq_ctx {
     }
     oq::HopArgs b = with_links(l, a);
     b.live_rec = (prof_on && rec.slot >= 0) ? prof_live + rec.slot : nullptr;
-    cudaError_t e = oq::launch_hop(l, b, s);
-    launches += 1;
+    cudaError_t e = oq::launch_hop_reduced(l, b, s, &launches);
     if (prof_on) {
       cudaEventRecord(rec.e1, s);
       prof.push_back(rec);

@@ -40,6 +40,7 @@ struct RedArgs {
   CgState* cg;         // [nrhs]
   int fin;
   int gate;            // CG finishers act only on rhs with cg[rhs].mode == gate
+  int defer;           // the CTAs only write their partials; reduce_finish sums them and runs the finisher
 };
 
 enum HopMode : int { HOP_DW = 0, HOP_P1 = 1, HOP_P2 = 2 };
@@ -113,6 +114,11 @@ struct HopLaunch {
 };
 
 cudaError_t launch_hop(const HopLaunch& L, const HopArgs& a, cudaStream_t s);
+// launch_hop, with the reduction of its epilogue finished by a kernel of its
+// own where that pays; *kernels counts the launches
+cudaError_t launch_hop_reduced(const HopLaunch& L, const HopArgs& a, cudaStream_t s, long long* kernels);
+// sum nrhs rows of ncta partials each and run their finishers (RedArgs::defer)
+cudaError_t reduce_finish(const RedArgs& ra, int nrhs, unsigned ncta, cudaStream_t s);
 cudaError_t launch_hop_f64(const HopLaunch& L, const HopArgs& a, cudaStream_t s);
 cudaError_t launch_hop_f32(const HopLaunch& L, const HopArgs& a, cudaStream_t s);
 cudaError_t launch_hop_bf16(const HopLaunch& L, const HopArgs& a, cudaStream_t s);

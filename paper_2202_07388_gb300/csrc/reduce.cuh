@@ -8,6 +8,11 @@
 // the finisher that turns the sum into solver scalars (CG alpha / beta,
 // restart norms).  The order of the additions never depends on timing, so
 // results are bitwise reproducible.
+//
+// The fence and the ticket hold a CTA back by about two memory latencies after
+// its last store.  In a launch of many CTAs per SM that is time in which its
+// registers serve no one, so there the partials are only written (defer) and
+// reduce_finish sums them in a launch of its own.
 #pragma once
 #include "oq_internal.h"
 
@@ -133,9 +138,11 @@ __device__ __forceinline__ void grid_reduce(T v, const RedArgs& ra, int rhs, int
       if (tx == 0) {
         for (int w = 0; w < nw; ++w) s += smem[ty * nw + w];
         ra.partials[(long)rhs * ncta + cta] = s;
-        __threadfence();
-        unsigned t = atomicAdd(ra.counters + rhs, 1u);
-        last = (t == ncta - 1);
+        if (!ra.defer) {
+          __threadfence();
+          unsigned t = atomicAdd(ra.counters + rhs, 1u);
+          last = (t == ncta - 1);
+        }
       }
       last = __shfl_sync(0xffffffffu, last, 0);
       if (last) {
@@ -175,9 +182,11 @@ __device__ __forceinline__ void grid_reduce_nr(const T (&v)[NR], const RedArgs& 
       double s = 0.0;
       for (int w = 0; w < nw; ++w) s += smem[(ty * NR + k) * nw + w];
       ra.partials[(long)rhs * ncta + cta] = s;
-      __threadfence();
-      const unsigned t = atomicAdd(ra.counters + rhs, 1u);
-      last = (t == ncta - 1);
+      if (!ra.defer) {
+        __threadfence();
+        const unsigned t = atomicAdd(ra.counters + rhs, 1u);
+        last = (t == ncta - 1);
+      }
     }
     last = __shfl_sync(0xffffffffu, last, 0);
     if (last) {

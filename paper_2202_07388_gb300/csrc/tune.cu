@@ -239,13 +239,12 @@ extern "C" int oq_autotune(oq_handle h, int lat, int prec, int nrhs, void* strea
         l.link_fmt = fmt;
         const HopArgs b = h->with_links(l, a);
         for (int w = 0; w < 2; ++w)
-          if (launch_hop(l, b, s) != cudaSuccess) ret = OQ_ERR_CUDA;
+          if (launch_hop_reduced(l, b, s, &h->launches) != cudaSuccess) ret = OQ_ERR_CUDA;
         const int reps = 5;
         cudaEventRecord(e0, s);
         for (int r = 0; r < reps; ++r)
-          if (launch_hop(l, b, s) != cudaSuccess) ret = OQ_ERR_CUDA;
+          if (launch_hop_reduced(l, b, s, &h->launches) != cudaSuccess) ret = OQ_ERR_CUDA;
         cudaEventRecord(e1, s);
-        h->launches += 2 + reps;
         if (cudaEventSynchronize(e1) != cudaSuccess) ret = OQ_ERR_CUDA;
         if (ret) break;
         float ms = 0.f;
