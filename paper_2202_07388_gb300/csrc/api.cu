@@ -26,6 +26,14 @@ cudaError_t launch_hop(const HopLaunch& L, const HopArgs& a, cudaStream_t s) {
     }
     return cudaErrorInvalidValue;
   }
+  if (L.pair) {
+    switch (L.prec) {
+      case P_F32: return launch_hop_pair_f32(L, a, s);
+      case P_BF16: return launch_hop_pair_bf16(L, a, s);
+      case P_F16: return launch_hop_pair_f16(L, a, s);
+    }
+    return cudaErrorInvalidValue;
+  }
   switch (L.prec) {
     case P_F64: return launch_hop_f64(L, a, s);
     case P_F32: return launch_hop_f32(L, a, s);

@@ -3,9 +3,10 @@
 // and medium lattices at once (QCD+QED: several charges and volumes).
 //
 // Same algorithm as oq_cgne_solve (Sec. 2), organised for launch overhead:
-//  * every stencil pass of every system is ONE launch of a persistent grid
-//    that walks a tile list (system, site block) (hop_batch_kernel); the
-//    vector steps are batched the same way;
+//  * every stencil pass of every system is ONE launch over a tile list
+//    (system, site block), a CTA per tile (hop_batch_kernel, and
+//    hop_pair_batch_kernel for the regular steps); the vector steps are one
+//    launch of a grid that walks such a list;
 //  * per-system arguments, solver state and reduction scratch live in
 //    device memory, so a chunk of CHUNK regular iterations has no host
 //    dependency: it is captured once into a CUDA graph and replayed;
@@ -181,7 +182,9 @@ extern "C" int oq_cgne_solve_batch(oq_handle h, int nsys, const int* lats, const
   if (rc) return rc;
   cudaStream_t s = h->work_stream;
   const int XP = P == P_F64 ? P_F64 : P_F32;
-  const int bx_lo = 128, bx_64 = 64;
+  // the regular steps of the binary32-arithmetic types: two threads per site
+  const bool pair = P != P_F64;
+  const int bx_lo = pair ? 64 : 128, bx_64 = 64;
   // per-system buffers
   std::vector<long> Vh(nsys);
   std::vector<void*> eta64(nsys), xd(nsys), rd(nsys), t64(nsys), u64v(nsys), pv(nsys), rv(nsys), uv(nsys),
@@ -370,6 +373,7 @@ extern "C" int oq_cgne_solve_batch(oq_handle h, int nsys, const int* lats, const
     const bool f64 = prec == P_F64 || prec == P_DF64;
     l.bx = f64 ? bx_64 : bx_lo;
     l.by = 1;
+    l.pair = !f64 && pair;
     l.sys = dargs + (long)argset * nsys;
     l.tiles = f64 ? t_64 : t_lo;
     l.ntiles = (int)(f64 ? tiles_64.size() : tiles_lo.size());

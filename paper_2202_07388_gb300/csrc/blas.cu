@@ -97,6 +97,8 @@ cudaError_t reduce_dot(int prec, const void* x, const void* y, long Vh, long str
 __global__ void __launch_bounds__(RED_BX) reduce_finish_kernel(RedArgs ra, unsigned ncta) {
   __shared__ double smem[RED_BX / 32];
   const int rhs = blockIdx.x;
+  dep_trigger();
+  dep_wait();
   if (ra.fin != FIN_STORE && ra.cg[rhs].mode != ra.gate) return;  // not live in the launch
   const double* part = ra.partials + (long)rhs * ncta;
   double acc = 0.0;
@@ -114,8 +116,7 @@ __global__ void __launch_bounds__(RED_BX) reduce_finish_kernel(RedArgs ra, unsig
 }
 
 cudaError_t reduce_finish(const RedArgs& ra, int nrhs, unsigned ncta, cudaStream_t s) {
-  reduce_finish_kernel<<<nrhs, RED_BX, 0, s>>>(ra, ncta);
-  return cudaGetLastError();
+  return launch_dep(reduce_finish_kernel, dim3(nrhs), dim3(RED_BX), 0, s, ra, ncta);
 }
 
 // ---------------------------------------------------------------------------
@@ -133,6 +134,8 @@ __global__ void __launch_bounds__(256) cg_p_kernel(char* p, const char* r, long 
   typedef typename PrecTraits<P>::R R;
   const int rhs = blockIdx.y;
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  dep_trigger();
+  dep_wait();
   if (hist && i == 0) {
     const CgState& c = cg[rhs];
     if (c.steps >= 1 && c.steps <= hcap) hist[(long)rhs * hcap + c.steps - 1] = sqrt(c.rr) * c.scale;
@@ -158,13 +161,12 @@ cudaError_t cg_update_p(int prec, void* p, const void* r, long Vh, long stride, 
   char* pp = (char*)p;
   const char* rr = (const char*)r;
   switch (prec) {
-    case P_F64: cg_p_kernel<P_F64><<<grid, block, 0, s>>>(pp, rr, Vh, stride, cg, hist, hcap); break;
-    case P_F32: cg_p_kernel<P_F32><<<grid, block, 0, s>>>(pp, rr, Vh, stride, cg, hist, hcap); break;
-    case P_BF16: cg_p_kernel<P_BF16><<<grid, block, 0, s>>>(pp, rr, Vh, stride, cg, hist, hcap); break;
-    case P_F16: cg_p_kernel<P_F16><<<grid, block, 0, s>>>(pp, rr, Vh, stride, cg, hist, hcap); break;
-    default: return cudaErrorInvalidValue;
+    case P_F64: return launch_dep(cg_p_kernel<P_F64>, grid, block, 0, s, pp, rr, Vh, stride, cg, hist, hcap);
+    case P_F32: return launch_dep(cg_p_kernel<P_F32>, grid, block, 0, s, pp, rr, Vh, stride, cg, hist, hcap);
+    case P_BF16: return launch_dep(cg_p_kernel<P_BF16>, grid, block, 0, s, pp, rr, Vh, stride, cg, hist, hcap);
+    case P_F16: return launch_dep(cg_p_kernel<P_F16>, grid, block, 0, s, pp, rr, Vh, stride, cg, hist, hcap);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 // x_d += scale * x_s   (right-hand sides in MODE_RESET)

@@ -79,6 +79,7 @@ struct TuneVal {
   int nr = 1;            // right-hand sides per thread
   int regcap = 0;        // register-capped multi-rhs variant
   int link_fmt = -1;     // binary32 link format (-1: the uploaded one)
+  bool pair = false;     // two threads per site (bx = 64, by = nr = 1; chosen by the tuner)
   float ms = 0.f;        // tuner's time per launch (0 if set by hand)
 };
 
@@ -267,6 +268,18 @@ struct oq_ctx {
     return OQ_OK;
   }
 
+  // Two threads per site by default (hop_pair.cuh; binary32-arithmetic types):
+  // every launch with one right-hand side (F32 Dhat on 48x24^3: 105 against
+  // 120 us with one thread per site, on 32x24x16x16 34 against 43 us, equal on
+  // 32x16^3); with several, the plain passes of up to 2^15 site-rhs (2 rhs F32
+  // on 16x16x12x12: 16 against 19 us; 4 rhs F16 on the same: 21 against 17 us)
+  // and those with a reduction below 2^18 (CG, 4 rhs F16 on 16^4: 29 against 32
+  // us with two rhs per thread; 12 rhs on 32x16^3: 122 against 98 us).
+  static bool pair_pays(int prec, int epi, long work, int nrhs) {
+    if (prec != oq::P_F32 && prec != oq::P_BF16 && prec != oq::P_F16) return false;
+    return nrhs == 1 || work <= (1L << 15) || (epi != oq::EPI_NONE && work < (1L << 18));
+  }
+
   oq::HopLaunch hop_launch(int lat, int prec, int mode, int dagger, int epi, int nrhs) {
     oq::HopLaunch l;
     l.prec = prec;
@@ -281,7 +294,12 @@ struct oq_ctx {
       l.by = it->second.by;
       l.nr = it->second.nr;
       l.regcap = it->second.regcap;
+      l.pair = it->second.pair;
       if (it->second.link_fmt >= 0) l.link_fmt = it->second.link_fmt;
+    } else if (pair_pays(prec, epi, lats[lat].g.Vh * nrhs, nrhs) && !lats[lat].halo_t) {
+      l.bx = 64;
+      l.by = 1;
+      l.pair = true;
     } else if (prec == oq::P_DF64 && !lats[lat].halo_t) {
       // the double-float site is latency- and issue-bound: 12 warps per SM at
       // 168 registers (Dhat, 12 rhs on 48x24^3: 4.0 ms against 6.5 ms
@@ -301,16 +319,11 @@ struct oq_ctx {
       // capped at 128 registers; within 10 % of the tuner's choice from 8^4 to
       // 48x24^3 with 2 to 12 rhs, where one rhs per thread in 32 x nrhs CTAs
       // took 1.2 to 1.9 times as long (12 rhs F16 Dhat on 48x24^3: 495 against
-      // 814 us; 4 rhs F32 on 32x16^3: 62 against 78 us; 8^4: 16 us either way).
-      // The reductions of the norm and CG epilogues want more threads on small
-      // problems: below 2^18 (norm) or 2^17 (CG) site-rhs one rhs per thread
-      // (where the tuner's choice changes between 16^4 and 32x16^3).
-      const long work = lats[lat].g.Vh * nrhs;
-      const bool few = (epi == oq::EPI_NORM && work < (1L << 18)) || (epi == oq::EPI_CG && work < (1L << 17));
+      // 814 us; 4 rhs F32 on 32x16^3: 62 against 78 us).
       l.bx = 64;
       l.by = 1;
-      l.nr = few ? 1 : 2;
-      l.regcap = few ? 0 : (prec != oq::P_F32 && l.link_fmt == oq::LINK_12) ? 3 : 1;
+      l.nr = 2;
+      l.regcap = (prec != oq::P_F32 && l.link_fmt == oq::LINK_12) ? 3 : 1;
     } else {
       // several right-hand sides: 32 sites x (largest divisor of nrhs <= 8) rows
       l.bx = 32;

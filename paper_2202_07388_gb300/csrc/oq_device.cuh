@@ -315,6 +315,13 @@ __device__ __forceinline__ uint32_t pack_f16x2(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
+// Fields that another kernel of the stream may still be writing when this one
+// starts (programmatic dependent launch) are read with ordinary loads: a
+// non-coherent load may be moved above the wait for that kernel.  Links and
+// clover blocks never change under a launch and keep the non-coherent path.
+template <typename T>
+__device__ __forceinline__ T ld_field(const T* p) { return *p; }
+
 // Load the 12 complex components of site i from a packed spinor field.
 template <int P>
 __device__ __forceinline__ void load_spinor(const void* base, long Vh, long i,
@@ -325,7 +332,7 @@ __device__ __forceinline__ void load_spinor(const void* base, long Vh, long i,
     const double2* b = reinterpret_cast<const double2*>(base);
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
-      double2 v = ldg_nc(b + c * Vh + i);
+      double2 v = ld_field(b + c * Vh + i);
       f[c] = cx<R>{R(v.x), R(v.y)};
     }
   } else if constexpr (P == P_DF64) {
@@ -333,14 +340,14 @@ __device__ __forceinline__ void load_spinor(const void* base, long Vh, long i,
     const float4* b = reinterpret_cast<const float4*>(base);
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
-      float4 v = ldg_nc(b + c * Vh + i);
+      float4 v = ld_field(b + c * Vh + i);
       f[c] = cx<R>{dfloat(v.x, v.y), dfloat(v.z, v.w)};
     }
   } else if constexpr (P == P_F32) {
     const float4* b = reinterpret_cast<const float4*>(base);
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
-      float4 v = ldg_nc(b + c * Vh + i);
+      float4 v = ld_field(b + c * Vh + i);
       f[2 * c] = cx<R>{v.x, v.y};
       f[2 * c + 1] = cx<R>{v.z, v.w};
     }
@@ -348,7 +355,7 @@ __device__ __forceinline__ void load_spinor(const void* base, long Vh, long i,
     const uint4* b = reinterpret_cast<const uint4*>(base);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      uint4 v = ldg_nc(b + c * Vh + i);
+      uint4 v = ld_field(b + c * Vh + i);
       uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
       for (int k = 0; k < 4; ++k) {

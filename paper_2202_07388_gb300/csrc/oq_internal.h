@@ -43,6 +43,29 @@ struct RedArgs {
   int defer;           // the CTAs only write their partials; reduce_finish sums them and runs the finisher
 };
 
+// Programmatic dependent launch: a kernel launched with launch_dep may start
+// while the kernel before it on the stream still runs.  It calls dep_wait
+// before it touches anything that an earlier kernel writes (and before any
+// return): the wait ends when that kernel has completed, and since every CTA of
+// that one has waited for its own predecessor, when all earlier ones have.
+// dep_trigger lets the next kernel's CTAs start as soon as there is room.
+__device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... KA, typename... A>
+inline cudaError_t launch_dep(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<KA>(args)...);
+}
+
 enum HopMode : int { HOP_DW = 0, HOP_P1 = 1, HOP_P2 = 2 };
 enum HopEpi : int { EPI_NONE = 0, EPI_NORM = 1, EPI_CG = 2, EPI_RESID64 = 3 };
 
@@ -105,6 +128,7 @@ struct HopLaunch {
   int bx, by;    // CTA shape: bx sites x by groups of nr right-hand sides
   int nr = 1;    // right-hand sides per thread (1: hop_kernel; 2, 4: hop_mr_kernel)
   int regcap = 0;  // hop_mr_kernel: 1 = register-capped variant
+  bool pair = false;  // two threads per site (hop_pair_kernel; F32 / BF16 / F16, nr = 1, bx = 64, by = 1)
   // batched launch over several systems (hop_batch_kernel) when sys != null:
   // per-system arguments and the (system, site block) tile list in device memory
   const HopArgs* sys = nullptr;
@@ -131,6 +155,10 @@ cudaError_t launch_hop_mr2_bf16(const HopLaunch& L, const HopArgs& a, cudaStream
 cudaError_t launch_hop_mr4_bf16(const HopLaunch& L, const HopArgs& a, cudaStream_t s);
 cudaError_t launch_hop_mr2_f16(const HopLaunch& L, const HopArgs& a, cudaStream_t s);
 cudaError_t launch_hop_mr4_f16(const HopLaunch& L, const HopArgs& a, cudaStream_t s);
+// two threads per site (binary32 arithmetic types)
+cudaError_t launch_hop_pair_f32(const HopLaunch& L, const HopArgs& a, cudaStream_t s);
+cudaError_t launch_hop_pair_bf16(const HopLaunch& L, const HopArgs& a, cudaStream_t s);
+cudaError_t launch_hop_pair_f16(const HopLaunch& L, const HopArgs& a, cudaStream_t s);
 // double-float, 2 right-hand sides per thread (packed two-lane arithmetic)
 cudaError_t launch_hop_df2(const HopLaunch& L, const HopArgs& a, cudaStream_t s);
 

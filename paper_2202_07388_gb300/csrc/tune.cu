@@ -64,6 +64,13 @@ std::vector<TuneVal> candidates(int prec, int nrhs) {
       v.by = by;
       c.push_back(v);
     }
+  // two threads per site (binary32 arithmetic types)
+  if (prec == P_F32 || prec == P_BF16 || prec == P_F16) {
+    TuneVal v;
+    v.bx = 64;
+    v.pair = true;
+    c.push_back(v);
+  }
   // double-float: the register-capped kernel (<= 128 threads per CTA)
   if (prec == P_DF64) {
     const size_t n0 = c.size();
@@ -236,6 +243,7 @@ extern "C" int oq_autotune(oq_handle h, int lat, int prec, int nrhs, void* strea
         l.by = c.by;
         l.nr = c.nr;
         l.regcap = c.regcap;
+        l.pair = c.pair;
         l.link_fmt = fmt;
         const HopArgs b = h->with_links(l, a);
         for (int w = 0; w < 2; ++w)

@@ -1,12 +1,13 @@
-"""The launch chosen without the tuner for several right-hand sides: both sides
-of its rule (problem sizes, storage types, link formats, odd counts) against
-one right-hand side per thread, pinned."""
+"""The launch chosen without the tuner: both sides of its rules (one and several
+right-hand sides, problem sizes, storage types, link formats, odd counts)
+against one thread per site and right-hand side, pinned."""
 import pytest
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dims,nrhs", [((4, 6, 2, 8), 3), ((8, 8, 16, 16), 5), ((16, 16, 16, 16), 9)])
+@pytest.mark.parametrize("dims,nrhs", [((4, 6, 2, 8), 3), ((8, 8, 16, 16), 5), ((16, 16, 16, 16), 9),
+                                       ((2, 2, 2, 2), 1), ((4, 6, 10, 6), 1), ((16, 32, 32, 18), 1)])
 @pytest.mark.parametrize("prec", [1, 2, 3])
 @pytest.mark.parametrize("link_fmt", [0, 1])
 def test_default_against_pinned(dims, nrhs, prec, link_fmt):
