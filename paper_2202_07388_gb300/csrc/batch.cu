@@ -359,8 +359,6 @@ extern "C" int oq_cgne_solve_batch(oq_handle h, int nsys, const int* lats, const
   const VecSys* dvs = (const VecSys*)bvsys;
   int nsm = 152;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device);
-  const int grid_lo = (int)std::min<long>((long)tiles_lo.size(), (long)nsm * 8);
-  const int grid_64 = (int)std::min<long>((long)tiles_64.size(), (long)nsm * 8);
   const int grid_v = (int)std::min<long>((long)tiles_v.size(), (long)nsm * 8);
 
   auto hop = [&](int argset, int prec, int mode, int dag, int epi) -> cudaError_t {
@@ -377,7 +375,6 @@ extern "C" int oq_cgne_solve_batch(oq_handle h, int nsys, const int* lats, const
     l.sys = dargs + (long)argset * nsys;
     l.tiles = f64 ? t_64 : t_lo;
     l.ntiles = (int)(f64 ? tiles_64.size() : tiles_lo.size());
-    l.grid = f64 ? grid_64 : grid_lo;
     HopArgs dummy;
     memset(&dummy, 0, sizeof(dummy));
     h->launches += 1;

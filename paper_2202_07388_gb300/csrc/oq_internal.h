@@ -134,7 +134,6 @@ struct HopLaunch {
   const HopArgs* sys = nullptr;
   const int2* tiles = nullptr;
   int ntiles = 0;
-  int grid = 0;
 };
 
 cudaError_t launch_hop(const HopLaunch& L, const HopArgs& a, cudaStream_t s);
