@@ -241,132 +241,127 @@ __global__ void __launch_bounds__(PB, CIN == 1 && FMT == LINK_12 ? 3 : 2) ptc_la
   }
 }
 
-// Sums over the warp of 64 binary32 values per lane: out[j] of lane l is the
-// sum of v[2l + j].  A transposing exchange (each step halves the values a lane
-// holds: 62 additions per lane instead of 5 per value), in double-float: the
-// first additions are exact, the others err by ~2^-47, against the 2^-24 of the
+// The sum over the warp of 32 binary32 values per lane; lane l returns that of
+// v[l].  A transposing exchange (each step halves the values a lane holds: 31
+// additions per lane instead of 5 per value), in double-float: the first
+// additions are exact, the others err by ~2^-47, against the 2^-24 of the
 // binary32 sums that come in.  In binary64 (1/64 of the binary32 rate) the warp
 // sums were half of the gradient kernels' time; they are taken that way where a
 // value of the warp is not finite or above 2^100 (binary32 sums could overflow).
-__device__ __forceinline__ void warp_sum64(const float (&v)[64], double (&out)[2]) {
+__device__ __forceinline__ double warp_sum32(const float (&v)[32]) {
   const int lane = threadIdx.x & 31;
   bool big = false;
 #pragma unroll
-  for (int k = 0; k < 64; ++k) big |= !(fabsf(v[k]) <= 1.2676506e30f);
+  for (int k = 0; k < 32; ++k) big |= !(fabsf(v[k]) <= 1.2676506e30f);
   if (__any_sync(0xffffffffu, big)) {
-    out[0] = out[1] = 0.0;
+    double out = 0.0;
 #pragma unroll
-    for (int k = 0; k < 64; ++k) {
+    for (int k = 0; k < 32; ++k) {
       const double t = warp_sum((double)v[k]);
-      if (lane == k / 2) out[k % 2] = t;
+      if (lane == k) out = t;
     }
-    return;
+    return out;
   }
-  dfloat d[32];
+  dfloat d[16];
   {
     const bool up = lane & 16;
 #pragma unroll
-    for (int k = 0; k < 32; ++k) {
-      const float keep = up ? v[k + 32] : v[k], send = up ? v[k] : v[k + 32];
+    for (int k = 0; k < 16; ++k) {
+      const float keep = up ? v[k + 16] : v[k], send = up ? v[k] : v[k + 16];
       d[k] = df_two_sum(keep, __shfl_xor_sync(0xffffffffu, send, 16));
     }
   }
 #pragma unroll
-  for (int h = 16; h >= 2; h >>= 1) {
-    const int o = h >> 1;  // lane distance of this step
-    const bool up = lane & o;
+  for (int h = 8; h >= 1; h >>= 1) {
+    const bool up = lane & h;
 #pragma unroll
     for (int k = 0; k < h; ++k) {
       const dfloat keep = up ? d[k + h] : d[k], send = up ? d[k] : d[k + h];
-      const dfloat got(__shfl_xor_sync(0xffffffffu, send.hi, o), __shfl_xor_sync(0xffffffffu, send.lo, o));
+      const dfloat got(__shfl_xor_sync(0xffffffffu, send.hi, h), __shfl_xor_sync(0xffffffffu, send.lo, h));
       d[k] = keep + got;
     }
   }
-  out[0] = (double)d[0];
-  out[1] = (double)d[1];
+  return (double)d[0];
 }
 
-// Weight-gradient partials for one path (blockIdx.y): COUT*CIN*16 complex per
-// CTA, written in binary64 to part[q][cta][k].
-template <int FMT, int CIN, int COUT>
-__global__ void __launch_bounds__(PB) ptc_dw_kernel(const PtcArgs a, const char* grad, double* part) {
-  constexpr int NW = COUT * CIN * 16;  // complex entries per path
-  static_assert(NW == 32, "the warp sum holds 64 reals per path");
-  __shared__ double red[PB / 32][2 * NW];
-  const int q = blockIdx.y;
-  float2 acc[NW];
+// Weight-gradient partials of one path (blockIdx.y) and one pair of channels
+// (blockIdx.z = co * CIN + ci): 16 complex per CTA, written in binary64 to
+// part[q][cta][32 z ..].  (One CTA for both channel pairs shares the transport
+// of a single input but needs 255 registers, 8 warps per SM that wait for their
+// gathers: the gradient of 4 pairs on 32x16^3 1.32 against 1.26 ms.)  Bound by
+// the gathers from L2, 240 bytes per site and path.
+template <int FMT, int CIN>
+__global__ void __launch_bounds__(PB, 4) ptc_dw_kernel(const PtcArgs a, const char* grad, double* part) {
+  __shared__ double red[PB / 32][32];
+  const int q = blockIdx.y, ci = blockIdx.z % CIN, co = blockIdx.z / CIN;
+  const char* in = a.in + ci * a.fbytes;
+  const char* gf = grad + co * a.fbytes;
+  float2 acc[16];
 #pragma unroll
-  for (int k = 0; k < NW; ++k) acc[k] = make_float2(0.f, 0.f);
+  for (int k = 0; k < 16; ++k) acc[k] = make_float2(0.f, 0.f);
   for (long j = (long)blockIdx.x * blockDim.x + threadIdx.x; j < 2 * a.g.Vh; j += (long)gridDim.x * blockDim.x) {
     const int p = j >= a.g.Vh ? 1 : 0;
     const long i = j - p * a.g.Vh;
     int x[4];
     eo_coords(a.g, p, i, x);
-    Spinor<float> gv[COUT];
+    Spinor<float> gv, t;
+    load_spinor<P_F32>(gf + (long)p * a.hbytes, a.g.Vh, i, gv);
+    transport<FMT>(a, in, q, p, i, x, t);
 #pragma unroll
-    for (int co = 0; co < COUT; ++co) load_spinor<P_F32>(grad + co * a.fbytes + (long)p * a.hbytes, a.g.Vh, i, gv[co]);
+    for (int tt = 0; tt < 4; ++tt)
 #pragma unroll
-    for (int ci = 0; ci < CIN; ++ci) {
-      Spinor<float> t;
-      transport<FMT>(a, a.in + ci * a.fbytes, q, p, i, x, t);
+      for (int s = 0; s < 4; ++s) {
+        // g[s] conj(t[tt]), lanes (re, im)
+        float2 v = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int co = 0; co < COUT; ++co)
-#pragma unroll
-        for (int s = 0; s < 4; ++s)
-#pragma unroll
-          for (int tt = 0; tt < 4; ++tt) {
-            // g[s] conj(t[t]), lanes (re, im)
-            float2 v = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              const cx<float> g = gv[co].c[s][c], z = t.c[tt][c];
-              v = __ffma2_rn(make_float2(z.im, z.im), make_float2(g.im, -g.re), v);
-              v = __ffma2_rn(make_float2(z.re, z.re), make_float2(g.re, g.im), v);
-            }
-            const int k = (co * CIN + ci) * 16 + s * 4 + tt;
-            acc[k] = __fadd2_rn(acc[k], v);
-          }
-    }
+        for (int c = 0; c < 3; ++c) {
+          const cx<float> g = gv.c[s][c], z = t.c[tt][c];
+          v = __ffma2_rn(make_float2(z.im, z.im), make_float2(g.im, -g.re), v);
+          v = __ffma2_rn(make_float2(z.re, z.re), make_float2(g.re, g.im), v);
+        }
+        acc[s * 4 + tt] = __fadd2_rn(acc[s * 4 + tt], v);
+      }
   }
-  // the warp's sum of the 2 NW = 64 values: lane l ends with values 2l, 2l + 1
-  float v[2 * NW];
+  float v[32];
 #pragma unroll
-  for (int k = 0; k < NW; ++k) {
+  for (int k = 0; k < 16; ++k) {
     v[2 * k] = acc[k].x;
     v[2 * k + 1] = acc[k].y;
   }
-  double t[2];
-  warp_sum64(v, t);
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  red[wid][2 * lane] = t[0];
-  red[wid][2 * lane + 1] = t[1];
+  red[wid][lane] = warp_sum32(v);
   __syncthreads();
-  for (int k = threadIdx.x; k < 2 * NW; k += blockDim.x) {
+  if (threadIdx.x < 32) {
     double s = 0.0;
-    for (int w = 0; w < PB / 32; ++w) s += red[w][k];
-    part[((long)q * gridDim.x + blockIdx.x) * 2 * NW + k] = s;
+#pragma unroll
+    for (int w = 0; w < PB / 32; ++w) s += red[w][lane];
+    part[((long)q * gridDim.x + blockIdx.x) * 64 + 32 * blockIdx.z + lane] = s;
   }
 }
 
-// sum the per-CTA partials in a fixed order: dw[q][k] += sum_cta part[q][cta][k].
-// One CTA per path, thread (k, j) adds the partials j, j + FIN, ... of value k
-// and the FIN sums are added in order (one thread per value, its loads one
-// after the other, took 108 us for 256 partials on 32x16^3, a fifth of the
-// gradient; this form 8.7 us).
+// sum the per-CTA partials of np pairs in a fixed order:
+// dw[layer][q][k] += sum_pair sum_cta part[pair][layer][q][cta][k].  One CTA per
+// path (blockIdx.x) and layer (blockIdx.y), thread (k, j) adds the partials j,
+// j + FIN, ... of value k, then the FIN sums are added in order (one thread per value, its loads one after the other, took 108
+// us for 256 partials on 32x16^3, a fifth of the gradient; this form 9 us for a pair's).
 static const int FIN = 16;
-__global__ void __launch_bounds__(64 * FIN) ptc_dw_finish(const double* part, int ncta, double* dw) {
+__global__ void __launch_bounds__(64 * FIN) ptc_dw_finish(const double* part, int np, int ncta, double* dw) {
+  const int layer = blockIdx.y;
   constexpr int NV = 64;
   __shared__ double sum[FIN][NV];
   const int q = blockIdx.x, k = threadIdx.x % NV, j = threadIdx.x / NV;
   double s = 0.0;
-#pragma unroll 4
-  for (int c = j; c < ncta; c += FIN) s += part[((long)q * ncta + c) * NV + k];
+  for (int r = 0; r < np; ++r) {
+    const double* p = part + (((long)r * 2 + layer) * NPATH + q) * ncta * NV + k;
+#pragma unroll 8
+    for (int c = j; c < ncta; c += FIN) s += p[(long)c * NV];
+  }
   sum[j][k] = s;
   __syncthreads();
   if (j) return;
 #pragma unroll
   for (int w = 1; w < FIN; ++w) s += sum[w][k];
-  dw[(long)q * NV + k] += s;
+  dw[((long)layer * NPATH + q) * NV + k] += s;
 }
 
 // bfloat16 forward weights and the adjoint layer's weights from binary32 masters:
@@ -442,11 +437,12 @@ static cudaError_t ptc_layer(const PtcArgs& a, int fmt, cudaStream_t s) {
 
 template <int CIN, int COUT>
 static cudaError_t ptc_dw(const PtcArgs& a, int fmt, const char* grad, double* part, int ncta, cudaStream_t s) {
-  dim3 grid(ncta, NPATH), block(PB);
+  static_assert(CIN * COUT == 2, "the partials hold two channel pairs per path");
+  dim3 grid(ncta, NPATH, CIN * COUT), block(PB);
   if (fmt == LINK_12)
-    ptc_dw_kernel<LINK_12, CIN, COUT><<<grid, block, 0, s>>>(a, grad, part);
+    ptc_dw_kernel<LINK_12, CIN><<<grid, block, 0, s>>>(a, grad, part);
   else
-    ptc_dw_kernel<LINK_18, CIN, COUT><<<grid, block, 0, s>>>(a, grad, part);
+    ptc_dw_kernel<LINK_18, CIN><<<grid, block, 0, s>>>(a, grad, part);
   return cudaGetLastError();
 }
 
@@ -598,21 +594,21 @@ extern "C" int oq_nnprec_grad(oq_handle h, int lat, const float* weights_dev, co
   const long hb = spinor_half_bytes(Vh, P_F32), f32 = 2 * hb;
   const int ncta = reduce_grid(2 * Vh) < 256 ? reduce_grid(2 * Vh) : 256;
   void* part;
-  rc = h->workspace(lat, "nn_part", sizeof(double) * NPATH * ncta * 2 * 32, &part);
-  const int GRP = 32;
-  double en2[32];
+  const int GRP = 8;
+  const size_t npart = (size_t)NPATH * ncta * 64;  // partials of one pair and layer
+  rc = h->workspace(lat, "nn_part", sizeof(double) * 2 * npart * (n < GRP ? n : GRP), &part);
+  double en2[GRP];
   if (!rc) rc = h->ensure_reduce(2 * GRP, reduce_grid(2 * Vh));
   if (rc) return rc;
   const int fmt = L.link_fmt;
   const int nreal = 2 * (NW1 + NW2);
   if (cudaMemsetAsync(grad_dev, 0, sizeof(double) * nreal, s) != cudaSuccess) return OQ_ERR_CUDA;
-  double* gw1 = grad_dev;
-  double* gw2 = grad_dev + 2 * NW1;
+  static_assert(2 * NW1 == NPATH * 64 && NW1 == NW2, "gradients of layer 1, then of layer 2");
   double loss = 0.0;
   // pairs in groups of GRP: the norms of the group's e in one launch per parity
-  // (one wait), the losses read back together at the group's end (another);
-  // a wait for the norm and one for the loss of every pair left the GPU idle
-  // between its kernels
+  // (one wait), the losses read back together at the group's end (another) and
+  // the weight gradients' partials summed there; a wait for the norm and one for
+  // the loss of every pair left the GPU idle between its kernels
   for (int k = 0; k < n; ++k) {
     const int kg = k % GRP, ng = n - (k - kg) < GRP ? n - (k - kg) : GRP;
     const char* r = (const char*)r_dev + (long)k * f32;
@@ -644,8 +640,9 @@ extern "C" int oq_nnprec_grad(oq_handle h, int lat, const float* weights_dev, co
     PtcArgs a = nn_args(h, lat);
     a.in = b.hid;
     a.w = b.w2;
-    if (ptc_dw<CH, 1>(a, fmt, b.gy, (double*)part, ncta, s) != cudaSuccess) return OQ_ERR_CUDA;
-    ptc_dw_finish<<<NPATH, 64 * FIN, 0, s>>>((const double*)part, ncta, gw2);
+    double* part1 = (double*)part + 2 * npart * kg;
+    double* part2 = part1 + npart;
+    if (ptc_dw<CH, 1>(a, fmt, b.gy, part2, ncta, s) != cudaSuccess) return OQ_ERR_CUDA;
     a.in = b.gy;
     a.out = b.ghid;
     a.w = b.w2a;
@@ -654,11 +651,12 @@ extern "C" int oq_nnprec_grad(oq_handle h, int lat, const float* weights_dev, co
     a = nn_args(h, lat);
     a.in = r;
     a.w = b.w1;
-    if (ptc_dw<1, CH>(a, fmt, b.ghid, (double*)part, ncta, s) != cudaSuccess) return OQ_ERR_CUDA;
-    ptc_dw_finish<<<NPATH, 64 * FIN, 0, s>>>((const double*)part, ncta, gw1);
-    h->launches += 5;
+    if (ptc_dw<1, CH>(a, fmt, b.ghid, part1, ncta, s) != cudaSuccess) return OQ_ERR_CUDA;
+    h->launches += 3;
     if (cudaGetLastError() != cudaSuccess) return OQ_ERR_CUDA;
     if (kg == ng - 1) {
+      ptc_dw_finish<<<dim3(NPATH, 2), 64 * FIN, 0, s>>>((const double*)part, ng, ncta, grad_dev);
+      h->launches += 1;
       if (cudaMemcpyAsync(h->results_host, h->results, ng * sizeof(double), cudaMemcpyDeviceToHost, s) !=
               cudaSuccess ||
           cudaStreamSynchronize(s) != cudaSuccess)
