@@ -4,9 +4,10 @@
 // Per step k < nkv:   phi_k = M rho_k        (SAP cycles, or identity if ncy = 0)
 //                     chi_k = D phi_k
 //                     a_lk = <chi_l, chi_k>, chi_k -= sum_l a_lk chi_l (classical
-//                     Gram-Schmidt: all dots in one launch, one fused update)
-//                     b_k = ||chi_k||, chi_k /= b_k, c_k = <chi_k, rho_k>,
-//                     rho_{k+1} = rho_k - c_k chi_k
+//                     Gram-Schmidt: all dots in one launch, one fused update
+//                     with b_k = ||chi_k|| and <chi_k, rho_k>)
+//                     chi_k /= b_k, c_k = <chi_k, rho_k> (= that over b_k),
+//                     rho_{k+1} = rho_k - c_k chi_k (one pass)
 // Restart / finish:   b_l beta_l + sum_{m>l} a_lm beta_m = c_l (host, k <= nkv),
 //                     psi += sum_l beta_l phi_l (binary64), rho = eta - D psi
 //                     (binary64 stencil: the "large" type).
@@ -63,36 +64,51 @@ __device__ __forceinline__ void site_dot(const Spinor<R>& a, const Spinor<R>& b,
   }
 }
 
+// The dots <X_l, y> of NL consecutive fields per CTA row (blockIdx.y), y read
+// once for them: partials of rows 2 l, 2 l + 1 (re, im).  (One field per CTA
+// read y from L2 for each of them: 15 dots on 48x24^3 took 340 us, 304 now.)
+static const int NL = 4;
 template <int P>
 __global__ void __launch_bounds__(VB) vec_dots_kernel(const char* X, long xstride, const char* y, long Vh,
                                                       long hb, RedArgs ra, int nl) {
   typedef typename PrecTraits<P>::R R;
-  __shared__ double smem[VB / 32];
-  const int l = blockIdx.y;
-  double re = 0.0, im = 0.0;
+  __shared__ double smem[2 * NL * VB / 32];
+  const int l0 = blockIdx.y * NL;
+  double v[2 * NL];
+  bool off[2 * NL];
+#pragma unroll
+  for (int k = 0; k < 2 * NL; ++k) {
+    v[k] = 0.0;
+    off[k] = false;
+  }
   for (long j = (long)blockIdx.x * blockDim.x + threadIdx.x; j < 2 * Vh; j += (long)gridDim.x * blockDim.x) {
     long i;
-    Spinor<R> a, b;
-    load_spinor<P>(fsite(X + l * xstride, Vh, hb, j, &i), Vh, i, a);
+    Spinor<R> b;
     load_spinor<P>(fsite(y, Vh, hb, j, &i), Vh, i, b);
-    site_dot(a, b, re, im);
+#pragma unroll
+    for (int k = 0; k < NL; ++k) {
+      // fields past the last repeat it (their rows are not stored): no branch between the loads
+      const int l = l0 + k < nl ? l0 + k : nl - 1;
+      Spinor<R> a;
+      load_spinor<P>(fsite(X + l * xstride, Vh, hb, j, &i), Vh, i, a);
+      site_dot(a, b, v[2 * k], v[2 * k + 1]);
+    }
   }
-  grid_reduce(re, ra, 2 * l, 2 * nl, smem, blockIdx.x, gridDim.x);
-  __syncthreads();
-  grid_reduce(im, ra, 2 * l + 1, 2 * nl, smem, blockIdx.x, gridDim.x);
+  grid_reduce_nr<2 * NL>(v, ra, 2 * l0, 2 * nl, smem, blockIdx.x, gridDim.x, off);
 }
 
-// chi -= sum_l coef_l X_l ; ||chi||^2 -> slot 0
+// chi -= sum_l coef_l X_l ; partials of ||chi||^2 and Re, Im <chi, rho> (rows 0, 1, 2)
 template <int P>
 __global__ void __launch_bounds__(VB) vec_orth_kernel(char* chi, const char* X, long xstride,
-                                                      const double2* coef, int nl, long Vh, long hb, RedArgs ra) {
+                                                      const double2* coef, int nl, const char* rho, long Vh,
+                                                      long hb, RedArgs ra) {
   typedef typename PrecTraits<P>::R R;
-  __shared__ double smem[VB / 32];
-  double acc = 0.0;
+  __shared__ double smem[3 * VB / 32];
+  double acc[3] = {0.0, 0.0, 0.0};
   for (long j = (long)blockIdx.x * blockDim.x + threadIdx.x; j < 2 * Vh; j += (long)gridDim.x * blockDim.x) {
     long i;
     char* cb = (char*)fsite(chi, Vh, hb, j, &i);
-    Spinor<R> v;
+    Spinor<R> v, r;
     load_spinor<P>(cb, Vh, i, v);
     for (int l = 0; l < nl; ++l) {
       Spinor<R> w;
@@ -104,56 +120,39 @@ __global__ void __launch_bounds__(VB) vec_orth_kernel(char* chi, const char* X, 
         for (int a = 0; a < 3; ++a) v.c[s][a] = v.c[s][a] - c * w.c[s][a];
     }
     store_spinor<P>(cb, Vh, i, v);
-    acc += site_norm2(v);
+    load_spinor<P>(fsite(rho, Vh, hb, j, &i), Vh, i, r);  // after the loop: its registers would halve the warps
+    acc[0] += site_norm2(v);
+    site_dot(v, r, acc[1], acc[2]);
   }
-  grid_reduce(acc, ra, 0, 1, smem, blockIdx.x, gridDim.x);
+  const bool off[3] = {false, false, false};
+  grid_reduce_nr<3>(acc, ra, 0, 3, smem, blockIdx.x, gridDim.x, off);
 }
 
-// chi *= inv_b ; <chi, rho> -> slots 0, 1
+// chi *= inv_b ; rho -= c chi ; partials of ||rho||^2 (row 0)
 template <int P>
-__global__ void __launch_bounds__(VB) vec_scale_dot_kernel(char* chi, const char* rho, double inv_b, long Vh,
-                                                           long hb, RedArgs ra) {
-  typedef typename PrecTraits<P>::R R;
-  __shared__ double smem[VB / 32];
-  double re = 0.0, im = 0.0;
-  for (long j = (long)blockIdx.x * blockDim.x + threadIdx.x; j < 2 * Vh; j += (long)gridDim.x * blockDim.x) {
-    long i;
-    char* cb = (char*)fsite(chi, Vh, hb, j, &i);
-    Spinor<R> v, r;
-    load_spinor<P>(cb, Vh, i, v);
-    load_spinor<P>(fsite(rho, Vh, hb, j, &i), Vh, i, r);
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) v.c[s][a] = (R)inv_b * v.c[s][a];
-    site_dot(v, r, re, im);
-    store_spinor<P>(cb, Vh, i, v);
-  }
-  grid_reduce(re, ra, 0, 2, smem, blockIdx.x, gridDim.x);
-  __syncthreads();
-  grid_reduce(im, ra, 1, 2, smem, blockIdx.x, gridDim.x);
-}
-
-// rho -= c chi ; ||rho||^2 -> slot 0
-template <int P>
-__global__ void __launch_bounds__(VB) vec_axpy_norm_kernel(char* rho, const char* chi, double cre, double cim,
-                                                           long Vh, long hb, RedArgs ra) {
+__global__ void __launch_bounds__(VB) vec_step_kernel(char* chi, char* rho, double inv_b, double cre, double cim,
+                                                      long Vh, long hb, RedArgs ra) {
   typedef typename PrecTraits<P>::R R;
   __shared__ double smem[VB / 32];
   double acc = 0.0;
   const cx<R> c{(R)cre, (R)cim};
   for (long j = (long)blockIdx.x * blockDim.x + threadIdx.x; j < 2 * Vh; j += (long)gridDim.x * blockDim.x) {
     long i;
+    char* cb = (char*)fsite(chi, Vh, hb, j, &i);
     char* rb = (char*)fsite(rho, Vh, hb, j, &i);
-    Spinor<R> v, w;
-    load_spinor<P>(rb, Vh, i, v);
-    load_spinor<P>(fsite(chi, Vh, hb, j, &i), Vh, i, w);
+    Spinor<R> v, r;
+    load_spinor<P>(cb, Vh, i, v);
+    load_spinor<P>(rb, Vh, i, r);
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
-      for (int a = 0; a < 3; ++a) v.c[s][a] = v.c[s][a] - c * w.c[s][a];
-    store_spinor<P>(rb, Vh, i, v);
-    acc += site_norm2(v);
+      for (int a = 0; a < 3; ++a) {
+        v.c[s][a] = (R)inv_b * v.c[s][a];
+        r.c[s][a] = r.c[s][a] - c * v.c[s][a];
+      }
+    store_spinor<P>(cb, Vh, i, v);
+    store_spinor<P>(rb, Vh, i, r);
+    acc += site_norm2(r);
   }
   grid_reduce(acc, ra, 0, 1, smem, blockIdx.x, gridDim.x);
 }
@@ -318,7 +317,6 @@ static int gcr_impl(oq_handle h, int lat, const oq_solver_params* prm, const flo
   rc = h->ensure_stage();
   if (rc) return rc;
   double2* coef_host = reinterpret_cast<double2*>(h->stage_host);  // pinned staging of 64 coefficients
-  std::vector<double2> cbuf(64);
 
 #define CK(x)                                   \
   do {                                          \
@@ -338,6 +336,8 @@ static int gcr_impl(oq_handle h, int lat, const oq_solver_params* prm, const flo
   const dim3 rgrid(grid), rblock(VB);
   const dim3 egrid((unsigned)((2 * Vh + VB - 1) / VB)), eblock(VB);
   RedArgs ra = h->red_args(FIN_STORE, 0);
+  RedArgs rp = ra;  // partials, summed by reduce_finish
+  rp.defer = 1;
   // read `n` reduction results (synchronises)
   auto fetch = [&](int n, double* out) -> int {
     CK(cudaMemcpyAsync(h->results_host, h->results, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
@@ -428,43 +428,38 @@ static int gcr_impl(oq_handle h, int lat, const oq_solver_params* prm, const flo
         }
         // chi_k = D phi_k
         RK(dw(P_F32, phik, chik));
-        double bk2 = 0.0;
+        // orthogonalise, with the norm and <chi, rho> of the result
         if (k > 0) {
-          KL((vec_dots_kernel<P_F32><<<dim3(grid, k), rblock, 0, s>>>((const char*)Chi, f32, chik, Vh, hb32, ra, k),
+          KL((vec_dots_kernel<P_F32><<<dim3(grid, (k + NL - 1) / NL), rblock, 0, s>>>((const char*)Chi, f32, chik, Vh,
+                                                                                      hb32, rp, k),
               cudaGetLastError()));
+          KL(reduce_finish(rp, 2 * k, grid, s));
           std::vector<double> d(2 * k);
           RK(fetch(2 * k, d.data()));
           for (int l = 0; l < k; ++l) {
             a[(size_t)l * nkv + k] = std::complex<double>(d[2 * l], d[2 * l + 1]);
-            cbuf[l] = make_double2(d[2 * l], d[2 * l + 1]);
-            coef_host[l] = cbuf[l];
+            coef_host[l] = make_double2(d[2 * l], d[2 * l + 1]);
           }
           CK(cudaMemcpyAsync(coef, coef_host, sizeof(double2) * k, cudaMemcpyHostToDevice, s));
-          KL((vec_orth_kernel<P_F32><<<rgrid, rblock, 0, s>>>(chik, (const char*)Chi, f32, (const double2*)coef, k,
-                                                              Vh, hb32, ra),
-              cudaGetLastError()));
-          RK(fetch(1, &bk2));
-        } else {
-          KL(reduce_norm2(P_F32, chik, Vh, 0, 1, ra, s));
-          KL(reduce_norm2(P_F32, chik + hb32, Vh, 0, 1, (ra.result = h->results + 1, ra), s));
-          ra.result = h->results;
-          double t2[2];
-          RK(fetch(2, t2));
-          bk2 = t2[0] + t2[1];
         }
-        b[k] = sqrt(bk2);
+        KL((vec_orth_kernel<P_F32><<<rgrid, rblock, 0, s>>>(chik, (const char*)Chi, f32, (const double2*)coef, k,
+                                                            (const char*)rho, Vh, hb32, rp),
+            cudaGetLastError()));
+        KL(reduce_finish(rp, 3, grid, s));
+        double t3[3];
+        RK(fetch(3, t3));
+        b[k] = sqrt(t3[0]);
         if (!(b[k] > 0.0) || !isfinite(b[k])) {
           nonfinite = !isfinite(b[k]);
           k_used = k;
           break;
         }
-        KL((vec_scale_dot_kernel<P_F32><<<rgrid, rblock, 0, s>>>(chik, (const char*)rho, 1.0 / b[k], Vh, hb32, ra),
+        // chi_k = chi / b_k, c_k = <chi_k, rho>, rho -= c_k chi_k
+        c[k] = std::complex<double>(t3[1] / b[k], t3[2] / b[k]);
+        KL((vec_step_kernel<P_F32><<<rgrid, rblock, 0, s>>>(chik, (char*)rho, 1.0 / b[k], c[k].real(), c[k].imag(), Vh,
+                                                            hb32, rp),
             cudaGetLastError()));
-        double cd[2];
-        RK(fetch(2, cd));
-        c[k] = std::complex<double>(cd[0], cd[1]);
-        KL((vec_axpy_norm_kernel<P_F32><<<rgrid, rblock, 0, s>>>((char*)rho, chik, cd[0], cd[1], Vh, hb32, ra),
-            cudaGetLastError()));
+        KL(reduce_finish(rp, 1, grid, s));
         double r2 = 0.0;
         RK(fetch(1, &r2));
         status += 1;
