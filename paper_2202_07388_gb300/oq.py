@@ -160,14 +160,35 @@ def _check(code, where):
 
 
 def _ptr(t):
-    return C.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
+
+
+def _stream_getter():
+    """A function that returns the current torch CUDA stream as an integer.
+
+    torch.cuda.current_stream() builds a Stream object for every call (a
+    quarter of the host time of a small operator application); the raw stream
+    of the current device is the same handle.
+    """
+    import torch
+    torch.cuda.current_stream()   # initialises CUDA
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    if raw is None or device is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(device())
+
+
+_current_stream = None
 
 
 def _stream(stream=None):
+    global _current_stream
     if stream is not None:
-        return C.c_void_p(stream)
-    import torch
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return stream
+    if _current_stream is None:
+        _current_stream = _stream_getter()
+    return _current_stream()
 
 
 @dataclass
@@ -316,7 +337,7 @@ class Handle:
 
     @staticmethod
     def halo(from_next, from_prev, sign_next=1.0, sign_prev=1.0):
-        return OqHalo(_ptr(from_next).value, _ptr(from_prev).value, float(sign_next), float(sign_prev))
+        return OqHalo(_ptr(from_next), _ptr(from_prev), float(sign_next), float(sign_prev))
 
     def dw_halo(self, in_dev, out_dev, prec, halo: OqHalo, nrhs=1, dagger=False, lat=0, stream=None):
         _check(lib().oq_dw_apply_halo(self.h, lat, prec, _ptr(in_dev), _ptr(out_dev), nrhs, int(dagger),
