@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(VT) vec_batch_kernel(const VecSys* __restrict_
 #pragma unroll
           for (int s = 0; s < 4; ++s)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) q.c[s][c] = cx<R>{(R)(d.c[s][c].re * inv), (R)(d.c[s][c].im * inv)};
+            for (int c = 0; c < 3; ++c) q.c[s][c] = cx<R>{from64<R>(d.c[s][c].re * inv), from64<R>(d.c[s][c].im * inv)};
         }
 #pragma unroll
         for (int s = 0; s < 4; ++s)

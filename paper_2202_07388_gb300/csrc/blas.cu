@@ -28,7 +28,10 @@ __global__ void __launch_bounds__(RED_BX) norm2_kernel(const char* x, long Vh, l
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) acc += (double)s.c[a][c].re * s.c[a][c].re + (double)s.c[a][c].im * s.c[a][c].im;
+      for (int c = 0; c < 3; ++c) {
+        const double xr = (double)s.c[a][c].re, xi = (double)s.c[a][c].im;
+        acc = fma(xr, xr, fma(xi, xi, acc));
+      }
   }
   grid_reduce(acc, ra, rhs, nrhs, smem, blockIdx.x, gridDim.x);
 }
@@ -50,8 +53,9 @@ __global__ void __launch_bounds__(RED_BX) dot_kernel(const char* x, const char* 
     for (int s = 0; s < 4; ++s)
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        re += (double)a.c[s][c].re * b.c[s][c].re + (double)a.c[s][c].im * b.c[s][c].im;
-        im += (double)a.c[s][c].re * b.c[s][c].im - (double)a.c[s][c].im * b.c[s][c].re;
+        const double ar = (double)a.c[s][c].re, ai = (double)a.c[s][c].im, br = (double)b.c[s][c].re, bi = (double)b.c[s][c].im;
+        re = fma(ar, br, fma(ai, bi, re));
+        im = fma(ar, bi, fma(-ai, br, im));
       }
   }
   grid_reduce(re, ra, 2 * rhs, 2 * nrhs, smem, blockIdx.x, gridDim.x);
@@ -197,8 +201,8 @@ __global__ void __launch_bounds__(256) cg_accx_kernel(char* xd, const char* xs, 
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
       const double re = d.c[k / 3][k % 3].re, im = d.c[k / 3][k % 3].im;
-      const float rh = __double2float_rn(re), ih = __double2float_rn(im);
-      o[k * Vh + i] = make_float4(rh, __double2float_rn(re - (double)rh), ih, __double2float_rn(im - (double)ih));
+      const float rh = narrow(re), ih = narrow(im);
+      o[k * Vh + i] = make_float4(rh, narrow(re - (double)rh), ih, narrow(im - (double)ih));
     }
   }
 }
@@ -254,7 +258,7 @@ __global__ void __launch_bounds__(256) cg_restart_kernel(const char* rd, char* r
 #pragma unroll
       for (int s = 0; s < 4; ++s)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) v.c[s][c] = cx<R>{(R)(d.c[s][c].re * inv), (R)(d.c[s][c].im * inv)};
+        for (int c = 0; c < 3; ++c) v.c[s][c] = cx<R>{from64<R>(d.c[s][c].re * inv), from64<R>(d.c[s][c].im * inv)};
     }
 #pragma unroll
     for (int s = 0; s < 4; ++s)

@@ -387,7 +387,7 @@ __device__ __forceinline__ void store_block(const Geom& g, int p, long i, int b,
 #pragma unroll
   for (int c = 0; c < 9; ++c)
     q32[(9 * b + c) * g.Vh + i] =
-        make_float4((float)r[4 * c], (float)r[4 * c + 1], (float)r[4 * c + 2], (float)r[4 * c + 3]);
+        make_float4(narrow(r[4 * c]), narrow(r[4 * c + 1]), narrow(r[4 * c + 2]), narrow(r[4 * c + 3]));
 }
 
 // A and A^{-1} from the six field strengths c_sw F that a64 holds in its first

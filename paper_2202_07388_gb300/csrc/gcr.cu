@@ -174,7 +174,8 @@ __global__ void __launch_bounds__(VB) vec_diff_norm_kernel(char* out, const char
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         v.c[s][c] = v.c[s][c] - w.c[s][c];
-        acc += (double)v.c[s][c].re * v.c[s][c].re + (double)v.c[s][c].im * v.c[s][c].im;
+        const double xr = (double)v.c[s][c].re, xi = (double)v.c[s][c].im;
+        acc = fma(xr, xr, fma(xi, xi, acc));
       }
     if (out) store_spinor<P>((char*)fsite(out, Vh, hb, j, &i), Vh, i, v);
   }
@@ -195,7 +196,7 @@ __global__ void __launch_bounds__(VB) vec_convert_kernel(char* out, const char* 
 #pragma unroll
   for (int s = 0; s < 4; ++s)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) w.c[s][c] = cx<RO>{(RO)v.c[s][c].re, (RO)v.c[s][c].im};
+    for (int c = 0; c < 3; ++c) w.c[s][c] = cx<RO>{from64<RO>(v.c[s][c].re), from64<RO>(v.c[s][c].im)};
   store_spinor<PO>((char*)fsite(out, Vh, hbo, j, &i), Vh, i, w);
 }
 

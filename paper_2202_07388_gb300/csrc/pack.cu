@@ -60,16 +60,16 @@ __global__ void pack_links_kernel(Geom g, const double2* __restrict__ canon, dou
   if (fmt == LINK_18) {
     float2* d = reinterpret_cast<float2*>(u32) + ((long)(p * 4 + mu) * 9) * g.Vh;
 #pragma unroll
-    for (int k = 0; k < 9; ++k) d[k * g.Vh + i] = make_float2((float)m[k].x, (float)m[k].y);
+    for (int k = 0; k < 9; ++k) d[k * g.Vh + i] = make_float2(narrow(m[k].x), narrow(m[k].y));
   } else {
     float4* d = reinterpret_cast<float4*>(u32) + ((long)(p * 4 + mu) * 3) * g.Vh;
-    d[i] = make_float4((float)m[0].x, (float)m[0].y, (float)m[1].x, (float)m[1].y);
-    d[g.Vh + i] = make_float4((float)m[2].x, (float)m[2].y, (float)m[3].x, (float)m[3].y);
-    d[2 * g.Vh + i] = make_float4((float)m[4].x, (float)m[4].y, (float)m[5].x, (float)m[5].y);
+    d[i] = make_float4(narrow(m[0].x), narrow(m[0].y), narrow(m[1].x), narrow(m[1].y));
+    d[g.Vh + i] = make_float4(narrow(m[2].x), narrow(m[2].y), narrow(m[3].x), narrow(m[3].y));
+    d[2 * g.Vh + i] = make_float4(narrow(m[4].x), narrow(m[4].y), narrow(m[5].x), narrow(m[5].y));
     if (u18) {
       float2* e = u18 + ((long)(p * 4 + mu) * 9) * g.Vh;
 #pragma unroll
-      for (int k = 0; k < 9; ++k) e[k * g.Vh + i] = make_float2((float)m[k].x, (float)m[k].y);
+      for (int k = 0; k < 9; ++k) e[k * g.Vh + i] = make_float2(narrow(m[k].x), narrow(m[k].y));
     }
   }
 }
@@ -123,6 +123,9 @@ cudaError_t sf_mask_links(const Geom& g, double* u64, void* u32, int fmt, void* 
   return cudaGetLastError();
 }
 
+// x * scale; the usual scale of 1 needs no pass through the binary64 pipe
+__device__ __forceinline__ double times(double x, double scale) { return scale == 1.0 ? x : x * scale; }
+
 // one thread per (eo site, parity, rhs).  blockIdx.y = parity index within
 // the subset, blockIdx.z = rhs.
 template <int P>
@@ -144,7 +147,7 @@ __global__ void pack_spinor_kernel(Geom g, const double2* __restrict__ canon, ch
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
     double2 v = src[k];
-    s.c[k / 3][k % 3] = cx<R>{(R)(v.x * scale), (R)(v.y * scale)};
+    s.c[k / 3][k % 3] = cx<R>{from64<R>(times(v.x, scale)), from64<R>(times(v.y, scale))};
   }
   char* dst = out + rhs * out_stride + ((subset == 2) ? (long)p * spinor_half_bytes(g.Vh, P) : 0);
   if constexpr (P == P_BF16 || P == P_F16) {
@@ -156,7 +159,7 @@ __global__ void pack_spinor_kernel(Geom g, const double2* __restrict__ canon, ch
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         double2 v = src[4 * c + k];
-        double re = v.x * scale, im = v.y * scale;
+        double re = times(v.x, scale), im = times(v.y, scale);
         if constexpr (P == P_BF16) {
           __nv_bfloat16 a = __double2bfloat16(re), bb = __double2bfloat16(im);
           w[k] = (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(bb) << 16);
@@ -188,7 +191,7 @@ __global__ void unpack_spinor_kernel(Geom g, const char* __restrict__ in, double
   double2* dst = canon + rhs * canon_stride + (half ? lex_of(g, x) >> 1 : lex_of(g, x)) * 12;
 #pragma unroll
   for (int k = 0; k < 12; ++k)
-    dst[k] = make_double2((double)s.c[k / 3][k % 3].re * inv_scale, (double)s.c[k / 3][k % 3].im * inv_scale);
+    dst[k] = make_double2(times((double)s.c[k / 3][k % 3].re, inv_scale), times((double)s.c[k / 3][k % 3].im, inv_scale));
 }
 
 // Even-site (or odd-site) canonical fields: the site of eo index i sits at
@@ -230,7 +233,7 @@ __global__ void __launch_bounds__(HB) pack_half_kernel(Geom g, const double2* __
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const double2 v = sm[t * HROW + 4 * c + k];
-        const double re = v.x * sc, im = v.y * sc;
+        const double re = times(v.x, sc), im = times(v.y, sc);
         if constexpr (P == P_BF16) {
           __nv_bfloat16 a = __double2bfloat16(re), bb = __double2bfloat16(im);
           w[k] = (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(bb) << 16);
@@ -246,7 +249,7 @@ __global__ void __launch_bounds__(HB) pack_half_kernel(Geom g, const double2* __
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
       const double2 v = sm[t * HROW + k];
-      sp.c[k / 3][k % 3] = cx<R>{(R)(v.x * sc), (R)(v.y * sc)};
+      sp.c[k / 3][k % 3] = cx<R>{from64<R>(times(v.x, sc)), from64<R>(times(v.y, sc))};
     }
     store_spinor<P>(dst, g.Vh, i, sp);
   }
@@ -266,8 +269,8 @@ __global__ void __launch_bounds__(HB) unpack_half_kernel(Geom g, const char* __r
     load_spinor<P>(in + rhs * in_stride, g.Vh, i0 + t, sp);
 #pragma unroll
     for (int k = 0; k < 12; ++k)
-      sm[t * HROW + k] = make_double2((double)sp.c[k / 3][k % 3].re * inv_scale,
-                                      (double)sp.c[k / 3][k % 3].im * inv_scale);
+      sm[t * HROW + k] = make_double2(times((double)sp.c[k / 3][k % 3].re, inv_scale),
+                                      times((double)sp.c[k / 3][k % 3].im, inv_scale));
   }
   __syncthreads();
   double2* dst = canon + rhs * canon_stride + i0 * 12;
@@ -343,8 +346,8 @@ cudaError_t unpack_spinor(const Geom& g, int prec, int subset, const void* in, d
 __global__ void split_f64_kernel(const double* __restrict__ in, float2* __restrict__ out, size_t n) {
   for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
     const double x = in[k];
-    const float hi = __double2float_rn(x);
-    out[k] = make_float2(hi, __double2float_rn(x - (double)hi));
+    const float hi = narrow(x);
+    out[k] = make_float2(hi, narrow(x - (double)hi));
   }
 }
 

@@ -404,7 +404,8 @@ __global__ void __launch_bounds__(256) ptc_loss_kernel(const char* y, const char
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         a.c[s][c] = a.c[s][c] - b.c[s][c];
-        acc += (double)a.c[s][c].re * a.c[s][c].re + (double)a.c[s][c].im * a.c[s][c].im;
+        const double xr = (double)a.c[s][c].re, xi = (double)a.c[s][c].im;
+        acc = fma(xr, xr, fma(xi, xi, acc));
         a.c[s][c] = (float)(2.0 * inv_en2) * a.c[s][c];
       }
     store_spinor<P_F32>(g + p * hb, Vh, i, a);
