@@ -16,8 +16,9 @@
 //      4 steps, ||r|| > alpha ||r_prev||, when ||r|| grew, or when ||r|| fell
 //      below tol = res ||eta|| / n_blocks; every decision is block-uniform;
 //   3. phi_i += x.
-// sap_smem_eo_kernel replaces 2 by MR steps on the block's even-odd Schur
-// complement (see below).  Block reductions are binary64.  Arithmetic and storage binary32.
+// sap_block_eo_kernel replaces 2 by MR steps on the block's even-odd Schur
+// complement (see below).  Arithmetic and storage are binary32, the norms of the
+// adaptive exit tests binary64.
 // sap_block_kernel (the default) keeps a site's links in registers and the
 // block's clover in shared memory; sap_kernel reads them from global memory.
 #include "oq_internal.h"
@@ -379,15 +380,15 @@ __device__ __forceinline__ void sm4_publish(const SapShared& m, int t, const Su3
   sm4_send<3>(m, t, u[3], v);
 }
 
-// the in-block hops along mu of the published field; up / down: the site has
-// a neighbour in the block on that side
+// acc += the in-block hops along mu of the published field, from the positions
+// tu (above) and td (below); up / down: the site has such a neighbour in the
+// block (where not, the position is its own and the weight zero)
 template <int MU>
-__device__ __forceinline__ void sm4_hop(const SapShared& m, int t, int stride, bool up, bool down,
-                                        const Su3<float>& u, Spinor<float>& acc) {
+__device__ __forceinline__ void sm4_hop(const SapShared& m, int tu, int td, bool up, bool down, const Su3<float>& u,
+                                        Spinor<float>& acc) {
   Spinor<float> nb;
-  sm4_load(m.r, m.nsite, up ? t + stride : t, nb);
+  sm4_load(m.r, m.nsite, tu, nb);
   HalfSpinor<float> h, y, z;
-  const int td = down ? t - stride : t;
   cx<float>* c = &z.c[0][0];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -406,10 +407,10 @@ __device__ __forceinline__ void sm4_apply(const SapShared& m, int t, const int (
                                           unsigned down, const Su3<float> (&u)[4], const Spinor<float>& v,
                                           Spinor<float>& p) {
   sm4_clover(m.a, m.nsite, t, v, p);
-  sm4_hop<0>(m, t, stride[0], up & 1, down & 1, u[0], p);
-  sm4_hop<1>(m, t, stride[1], up & 2, down & 2, u[1], p);
-  sm4_hop<2>(m, t, stride[2], up & 4, down & 4, u[2], p);
-  sm4_hop<3>(m, t, stride[3], up & 8, down & 8, u[3], p);
+  sm4_hop<0>(m, up & 1 ? t + stride[0] : t, down & 1 ? t - stride[0] : t, up & 1, down & 1, u[0], p);
+  sm4_hop<1>(m, up & 2 ? t + stride[1] : t, down & 2 ? t - stride[1] : t, up & 2, down & 2, u[1], p);
+  sm4_hop<2>(m, up & 4 ? t + stride[2] : t, down & 4 ? t - stride[2] : t, up & 4, down & 4, u[2], p);
+  sm4_hop<3>(m, up & 8 ? t + stride[3] : t, down & 8 ? t - stride[3] : t, up & 8, down & 8, u[3], p);
 }
 
 // the hops along mu that come from outside the block, from global memory
@@ -604,62 +605,19 @@ __global__ void __launch_bounds__(256, 1) sap_block_kernel(const SapArgs a) {
   if (a.mr_steps && t == 0) atomicAdd(a.mr_steps, (unsigned)steps);
 }
 
-// operands of the even-odd block solver in shared memory
-struct SapSm {
-  float* r;        // [24][nsite] block residual
-  float2* u;       // [mu][9][nsite] forward links, 18 reals
-  float4* a;       // [18][nsite] clover (two blocks: 6 diagonal + 15 complex each)
-  int nsite;
-};
-
-__device__ __forceinline__ void sm_link(const SapSm& m, int mu, int t, Su3<float>& u) {
-#pragma unroll
-  for (int k = 0; k < 9; ++k) {
-    const float2 v = m.u[(mu * 9 + k) * m.nsite + t];
-    u.m[k / 3][k % 3] = cx<float>{v.x, v.y};
-  }
-}
-
-__device__ __forceinline__ void sm_clover(const SapSm& m, int t, const Spinor<float>& in, Spinor<float>& out) {
-  const cx<float>* v = &in.c[0][0];
-  cx<float>* o = &out.c[0][0];
-#pragma unroll
-  for (int b = 0; b < 2; ++b) {
-    float r[36];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      const float4 w = m.a[(9 * b + k) * m.nsite + t];
-      r[4 * k] = w.x;
-      r[4 * k + 1] = w.y;
-      r[4 * k + 2] = w.z;
-      r[4 * k + 3] = w.w;
-    }
-    const cx<float>* x = v + 6 * b;
-    cx<float>* y = o + 6 * b;
-#pragma unroll
-    for (int r0 = 0; r0 < 6; ++r0) y[r0] = r[r0] * x[r0];
-    int k = 0;
-#pragma unroll
-    for (int r0 = 0; r0 < 6; ++r0)
-#pragma unroll
-      for (int c0 = r0 + 1; c0 < 6; ++c0) {
-        const cx<float> off{r[6 + 2 * k], r[7 + 2 * k]};
-        cfma(y[r0], off, x[c0]);
-        cfmac(y[c0], off, x[r0]);
-        ++k;
-      }
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Even-odd reduced block solver (openQCD's choice for SAP, Sec. 3): per block
 //   rhat_e = r_e - D_eo A_oo^{-1} r_o,
 //   MR steps on Dhat_i = A_ee - D_eo A_oo^{-1} D_oe (even block sites),
 //   delta_o = A_oo^{-1} (r_o - D_oe delta_e),
-// D_eo, D_oe the in-block hops.  The shared field holds the even vector at
-// even sites and the odd intermediate at odd sites, so one MR step is two
-// half passes (odd threads, then even threads) separated by a barrier; the
-// staged clover is A at even and A^{-1} at odd sites.
+// D_eo, D_oe the in-block hops.  Links in registers and sends as in
+// sap_block_kernel; the staged clover is A at even and A^{-1} at odd sites.  An
+// MR step is two half passes: the odd threads form A^{-1} D_oe of the published
+// even residual and publish it, the even threads form D_eo of that.  Latency
+// and shared-memory reads bound it: a half pass keeps 4 of an SM's 8 warps
+// busy, and one block fills an SM (255 registers).  (A colour of 24x16^3 in
+// 4^4 blocks, 4 MR steps: 93 us; with links and clover in shared memory and
+// both hops of a link multiplied by their reader it took 128 us.)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void zero_spinor(Spinor<float>& v) {
 #pragma unroll
@@ -675,55 +633,16 @@ __device__ __forceinline__ void zero_spinor(Spinor<float>& v) {
 // whole warps instead of every other lane.
 __device__ __forceinline__ int eo_pos(int n, int par, int half) { return par * half + (n >> 1); }
 
-template <int MU>
-__device__ __forceinline__ void sm_block_hop_eo(const SapSm& m, const int bs[4], int n, int par, int half,
-                                                const int l[4], Spinor<float>& acc) {
-  int stride = 1;
-  for (int nu = 3; nu > MU; --nu) stride *= bs[nu];
-  const int t = eo_pos(n, par, half);
-  if (l[MU] + 1 < bs[MU]) {
-    Spinor<float> nb;
-    load_smem(m.r, m.nsite, eo_pos(n + stride, par ^ 1, half), nb);
-    HalfSpinor<float> h, r;
-    project<MU, -1>(nb, h);
-    Su3<float> u;
-    sm_link(m, MU, t, u);
-    su3_mul(u, h, r);
-    accum_reconstruct<MU, -1>(acc, r, -0.5f);
-  }
-  if (l[MU] > 0) {
-    const int tb = eo_pos(n - stride, par ^ 1, half);
-    Spinor<float> nb;
-    load_smem(m.r, m.nsite, tb, nb);
-    HalfSpinor<float> h, r;
-    project<MU, +1>(nb, h);
-    Su3<float> u;
-    sm_link(m, MU, tb, u);  // U_mu(x - mu): the forward link of the site below
-    su3_dag_mul(u, h, r);
-    accum_reconstruct<MU, +1>(acc, r, -0.5f);
-  }
-}
-
-// acc = D_hop v (in-block hops of the shared field)
-__device__ __forceinline__ void sm_dhop(const SapSm& m, const int bs[4], int n, int par, int half, const int l[4],
-                                        Spinor<float>& acc) {
-  zero_spinor(acc);
-  sm_block_hop_eo<0>(m, bs, n, par, half, l, acc);
-  sm_block_hop_eo<1>(m, bs, n, par, half, l, acc);
-  sm_block_hop_eo<2>(m, bs, n, par, half, l, acc);
-  sm_block_hop_eo<3>(m, bs, n, par, half, l, acc);
-}
-
 template <int FMT>
-__global__ void __launch_bounds__(256) sap_smem_eo_kernel(const SapArgs a) {
+__global__ void __launch_bounds__(256, 1) sap_block_eo_kernel(const SapArgs a) {
   extern __shared__ float4 sm4[];
   const int nsite = a.bs[0] * a.bs[1] * a.bs[2] * a.bs[3];
-  SapSm m;
+  SapShared m;
   m.nsite = nsite;
   m.a = sm4;
-  m.u = reinterpret_cast<float2*>(sm4 + 18 * nsite);
-  m.r = reinterpret_cast<float*>(m.u + 36 * nsite);
-  double* red = reinterpret_cast<double*>(m.r + 24 * nsite);
+  m.r = sm4 + 18 * nsite;
+  m.s = sm4 + 24 * nsite;
+  float* red = reinterpret_cast<float*>(sm4 + 36 * nsite);  // 3 partials per warp (binary64: block_sum1)
   const int t = threadIdx.x;
   const bool act = t < nsite;
   const int half3 = a.nb[3] / 2;
@@ -756,169 +675,200 @@ __global__ void __launch_bounds__(256) sap_smem_eo_kernel(const SapArgs a) {
   const int p = (x[0] + x[1] + x[2] + x[3]) & 1;  // lattice parity (the Schur complement's)
   const long i = eo_index(a.g, x);
   const bool ev = act && p == 0, od = act && p == 1;
-
-  Spinor<float> r;  // block residual (kept for the odd sites' final solve)
-  if (act) {
+  const int stride[4] = {a.bs[1] * a.bs[2] * a.bs[3], a.bs[2] * a.bs[3], a.bs[3], 1};
+  unsigned up = 0, down = 0;
+  int tu[4], td[4];
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-      Su3<float> u;
-      load_link<float, FMT>(a.links, a.g.Vh, p, mu, i, u);
-#pragma unroll
-      for (int k = 0; k < 9; ++k) m.u[(mu * 9 + k) * nsite + t] = make_float2(u.m[k / 3][k % 3].re, u.m[k / 3][k % 3].im);
+  for (int mu = 0; mu < 4; ++mu) {
+    tu[mu] = td[mu] = t;
+    if (l[mu] + 1 < a.bs[mu]) {
+      up |= 1u << mu;
+      tu[mu] = eo_pos(n + stride[mu], par ^ 1, half);
     }
-    const float4* q = reinterpret_cast<const float4*>(p ? a.clov_inv : a.clov) + (long)p * 18 * a.g.Vh;
+    if (l[mu] > 0) {
+      down |= 1u << mu;
+      td[mu] = eo_pos(n - stride[mu], par ^ 1, half);
+    }
+  }
+  const int w = t >> 5, nw = (blockDim.x + 31) >> 5;
+
+  Spinor<float> r, xs;  // r: the residual (odd sites), rhat (even sites)
+  zero_spinor(r);
+  zero_spinor(xs);
+  Su3<float> u[4];
+  // acc += the in-block hops of the published field
+  auto dhop = [&](Spinor<float>& acc) {
+    sm4_hop<0>(m, tu[0], td[0], up & 1, down & 1, u[0], acc);
+    sm4_hop<1>(m, tu[1], td[1], up & 2, down & 2, u[1], acc);
+    sm4_hop<2>(m, tu[2], td[2], up & 4, down & 4, u[2], acc);
+    sm4_hop<3>(m, tu[3], td[3], up & 8, down & 8, u[3], acc);
+  };
+  char* phi = a.phi + (long)p * a.half_bytes;
+  if (act) {
+    const float4* q = reinterpret_cast<const float4*>(p ? a.clov_inv : a.clov) + (long)p * 18 * a.g.Vh + i;
 #pragma unroll
-    for (int k = 0; k < 18; ++k) m.a[k * nsite + t] = __ldg(q + k * a.g.Vh + i);
-    Spinor<float> rh;
-    load_spinor<P_F32>(a.rho + (long)p * a.half_bytes, a.g.Vh, i, rh);
-    r = rh;
-    if (!(a.first && a.colour == 0)) {  // phi is zero before the first half cycle
-      HopArgs ha;
-      ha.g = a.g;
-      ha.links = a.links;
+    for (int k = 0; k < 18; ++k) cp_async16(m.a + k * nsite + t, q + k * a.g.Vh);
+    cp_async_commit();
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) load_link<float, FMT>(a.links, a.g.Vh, p, mu, i, u[mu]);
+    // block residual rho - D phi: the hops from outside the block
+    if (!(a.first && a.colour == 0)) {
       const char* nbf = a.phi + (long)(1 - p) * a.half_bytes;
-      Spinor<float> acc;
-      zero_spinor(acc);
-      hop_dir<P_F32, FMT, 0, false>(ha, nbf, p, i, x, acc, -0.5f);
-      hop_dir<P_F32, FMT, 1, false>(ha, nbf, p, i, x, acc, -0.5f);
-      hop_dir<P_F32, FMT, 2, false>(ha, nbf, p, i, x, acc, -0.5f);
-      hop_dir<P_F32, FMT, 3, false>(ha, nbf, p, i, x, acc, -0.5f);
+      outer_hop<FMT, 3>(a, nbf, p, x, up & 8, down & 8, u[3], r);
+      outer_hop<FMT, 2>(a, nbf, p, x, up & 4, down & 4, u[2], r);
+      outer_hop<FMT, 1>(a, nbf, p, x, up & 2, down & 2, u[1], r);
+      outer_hop<FMT, 0>(a, nbf, p, x, up & 1, down & 1, u[0], r);
+    }
+    if (!a.first) {
       Spinor<float> ph, aph;
-      load_spinor<P_F32>(a.phi + (long)p * a.half_bytes, a.g.Vh, i, ph);
+      load_spinor<P_F32>(phi, a.g.Vh, i, ph);
+      sm4_publish(m, t, u, ph);
       clover_apply<float>(a.clov, a.g.Vh, p, i, ph, aph);
 #pragma unroll
       for (int s = 0; s < 4; ++s)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) r.c[s][c] = rh.c[s][c] - (aph.c[s][c] + acc.c[s][c]);
+        for (int c = 0; c < 3; ++c) r.c[s][c] = r.c[s][c] + aph.c[s][c];
+    } else {
+      // a dropped hop reads its own position with weight zero: that must hold numbers
+      const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) m.r[k * nsite + t] = z;
+#pragma unroll
+      for (int k = 0; k < 12; ++k) m.s[k * nsite + t] = z;
     }
+    cp_async_wait();
   }
-  __syncthreads();  // the staged links and clover are read by the neighbours below
-  // odd sites: w_o = A^{-1} r_o into the shared field
-  if (od) {
-    Spinor<float> w;
-    sm_clover(m, t, r, w);
-    store_smem(m.r, nsite, t, w);
+  if (!a.first) {
+    __syncthreads();  // the published phi
+    if (act) dhop(r);
+    __syncthreads();  // every read of it is done
   }
-  __syncthreads();
-  // even sites: rhat_e = r_e - D_eo w_o (written at the even positions, read
-  // by no one in this phase)
-  Spinor<float> rh;
-  zero_spinor(rh);
-  if (ev) {
-    Spinor<float> acc;
-    sm_dhop(m, a.bs, n, par, half, l, acc);
+  if (act) {
+    Spinor<float> rh;
+    load_spinor<P_F32>(a.rho + (long)p * a.half_bytes, a.g.Vh, i, rh);
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) rh.c[s][c] = r.c[s][c] - acc.c[s][c];
-    store_smem(m.r, nsite, t, rh);
+      for (int c = 0; c < 3; ++c) r.c[s][c] = rh.c[s][c] - r.c[s][c];
   }
-  double n0 = 0.0;
-  if (a.adaptive) {
-    if (ev) n0 = site_norm2(rh);
-    n0 = block_sum1(n0, red);
-  } else {
-    __syncthreads();
+  // odd sites publish A^{-1} r_o; even sites: rhat_e = r_e - D_eo A^{-1} r_o
+  if (od) {
+    Spinor<float> v;
+    sm4_clover(m.a, nsite, t, r, v);
+    sm4_publish(m, t, u, v);
   }
-  double rn_prev = sqrt(n0);
+  __syncthreads();
+  if (ev) {
+    Spinor<float> acc;
+    zero_spinor(acc);
+    dhop(acc);
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) r.c[s][c] = r.c[s][c] - acc.c[s][c];
+    sm4_publish(m, t, u, r);  // at even positions, which no one reads in this phase
+  }
+  double rn_prev = 0.0;
+  if (a.adaptive) rn_prev = sqrt(block_sum1(ev ? site_norm2(r) : 0.0, reinterpret_cast<double*>(red)));
+  __syncthreads();
 
-  Spinor<float> xs;
-  zero_spinor(xs);
   int steps = 0;
   for (int k = 1; k <= a.nmr; ++k) {
     // odd half pass: t_o = A^{-1} D_oe rhat_e
     if (od) {
-      Spinor<float> acc, w;
-      sm_dhop(m, a.bs, n, par, half, l, acc);
-      sm_clover(m, t, acc, w);
-      store_smem(m.r, nsite, t, w);
+      Spinor<float> acc, v;
+      zero_spinor(acc);
+      dhop(acc);
+      sm4_clover(m.a, nsite, t, acc, v);
+      sm4_publish(m, t, u, v);
     }
     __syncthreads();
     // even half pass: q_e = A rhat_e - D_eo t_o, then <q, rhat>, <q, q>
     Spinor<float> pv;
-    float pr_re = 0.f, pr_im = 0.f, pp = 0.f;
+    float d0 = 0.f, d1 = 0.f, d2 = 0.f;
     if (ev) {
-      Spinor<float> own, acc;
-      load_smem(m.r, nsite, t, own);
-      sm_clover(m, t, own, pv);
-      sm_dhop(m, a.bs, n, par, half, l, acc);
-      float ar = 0.f, ai = 0.f, a2 = 0.f;
+      Spinor<float> acc;
+      sm4_clover(m.a, nsite, t, r, pv);
+      zero_spinor(acc);
+      dhop(acc);
 #pragma unroll
       for (int s = 0; s < 4; ++s)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           pv.c[s][c] = pv.c[s][c] - acc.c[s][c];
-          cx<float> q2 = pv.c[s][c], v = own.c[s][c];
-          ar += q2.re * v.re + q2.im * v.im;
-          ai += q2.re * v.im - q2.im * v.re;
-          a2 += q2.re * q2.re + q2.im * q2.im;
+          const cx<float> q = pv.c[s][c], v = r.c[s][c];
+          d0 += q.re * v.re + q.im * v.im;
+          d1 += q.re * v.im - q.im * v.re;
+          d2 += q.re * q.re + q.im * q.im;
         }
-      pr_re = ar;
-      pr_im = ai;
-      pp = a2;
     }
-    block_sum3(pr_re, pr_im, pp, red);  // barrier: every read of this step is done
-    float om_re = 0.f, om_im = 0.f;
-    if (pp > 0.f) {
-      om_re = pr_re / pp;
-      om_im = pr_im / pp;
+    d0 = warp_sum_f(d0);
+    d1 = warp_sum_f(d1);
+    d2 = warp_sum_f(d2);
+    if ((t & 31) == 0) {
+      red[3 * w] = d0;
+      red[3 * w + 1] = d1;
+      red[3 * w + 2] = d2;
     }
-    const cx<float> om{om_re, om_im};
-    double n1 = 0.0;
+    __syncthreads();  // the partial sums
+    d0 = d1 = d2 = 0.f;
+    for (int j = 0; j < nw; ++j) {
+      d0 += red[3 * j];
+      d1 += red[3 * j + 1];
+      d2 += red[3 * j + 2];
+    }
+    cx<float> om{0.f, 0.f};
+    if (d2 > 0.f) om = cx<float>{d0 / d2, d1 / d2};
     if (ev) {
-      Spinor<float> own;
-      load_smem(m.r, nsite, t, own);
 #pragma unroll
       for (int s = 0; s < 4; ++s)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          cfma(xs.c[s][c], om, own.c[s][c]);
-          own.c[s][c] = own.c[s][c] - om * pv.c[s][c];
+          cfma(xs.c[s][c], om, r.c[s][c]);
+          r.c[s][c] = r.c[s][c] - om * pv.c[s][c];
         }
-      store_smem(m.r, nsite, t, own);
-      n1 = site_norm2(own);
+      sm4_publish(m, t, u, r);
     }
     steps = k;
     if (a.adaptive) {
-      n1 = block_sum1(n1, red);
-      const double rn_new = sqrt(n1);
+      const double rn_new = sqrt(block_sum1(ev ? site_norm2(r) : 0.0, reinterpret_cast<double*>(red)));
       if ((k >= 4 && rn_new > (double)a.alpha * rn_prev) || rn_new > rn_prev || rn_new < a.tol) break;
       rn_prev = rn_new;
-    } else {
-      __syncthreads();  // the odd half pass of the next step reads the even residual
     }
+    __syncthreads();  // the odd half pass of the next step reads the even residual
   }
-  // delta_e = x_e into the shared field; delta_o = A^{-1} (r_o - D_oe delta_e)
-  if (ev) store_smem(m.r, nsite, t, xs);
+  // delta_e = x_e published; delta_o = A^{-1} (r_o - D_oe delta_e)
+  if (ev) sm4_publish(m, t, u, xs);
   __syncthreads();
   if (od) {
-    Spinor<float> acc, w;
-    sm_dhop(m, a.bs, n, par, half, l, acc);
+    Spinor<float> acc;
+    zero_spinor(acc);
+    dhop(acc);
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) w.c[s][c] = r.c[s][c] - acc.c[s][c];
-    sm_clover(m, t, w, xs);
+      for (int c = 0; c < 3; ++c) r.c[s][c] = r.c[s][c] - acc.c[s][c];
+    sm4_clover(m.a, nsite, t, r, xs);
   }
   if (act) {
-    char* pp = a.phi + (long)p * a.half_bytes;
-    Spinor<float> ph;
-    load_spinor<P_F32>(pp, a.g.Vh, i, ph);
+    if (!a.first) {
+      Spinor<float> ph;
+      load_spinor<P_F32>(phi, a.g.Vh, i, ph);
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
+      for (int s = 0; s < 4; ++s)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) ph.c[s][c] = ph.c[s][c] + xs.c[s][c];
-    store_spinor<P_F32>(pp, a.g.Vh, i, ph);
+        for (int c = 0; c < 3; ++c) xs.c[s][c] = ph.c[s][c] + xs.c[s][c];
+    }
+    store_spinor<P_F32>(phi, a.g.Vh, i, xs);
   }
   if (a.mr_steps && t == 0) atomicAdd(a.mr_steps, (unsigned)steps);
 }
 
-// operands in shared memory: clover, links and residual (even-odd kernel), or
-// clover, residual and sends (sap_block_kernel); at most 172 KB for 256 sites
-static size_t sap_smem_bytes(const int bs[4], int words) {
+// clover, residual and sends of a block in shared memory; at most 147 KB (256 sites)
+static size_t sap_smem_bytes(const int bs[4]) {
   const int nsite = bs[0] * bs[1] * bs[2] * bs[3];
   const int threads = (nsite + 31) / 32 * 32;
-  return sizeof(float) * words * (size_t)nsite + sizeof(double) * 3 * (threads / 32);
+  return sizeof(float) * (72 + 24 + 48) * (size_t)nsite + sizeof(double) * 3 * (threads / 32);
 }
 
 cudaError_t sap_colour(const Geom& g, const int bs[4], int colour, int fmt, const void* links, const void* clov,
@@ -927,7 +877,7 @@ cudaError_t sap_colour(const Geom& g, const int bs[4], int colour, int fmt, cons
   SapArgs a;
   a.first = cycle == 0;
   // every block is written in the first cycle; the kernels that read phi there need zeros
-  if (cycle == 0 && colour == 0 && (eo || kernel != 0)) {
+  if (cycle == 0 && colour == 0 && !eo && kernel != 0) {
     const cudaError_t e = cudaMemsetAsync(phi, 0, 2 * spinor_half_bytes(g.Vh, P_F32), s);
     if (e != cudaSuccess) return e;
   }
@@ -955,20 +905,20 @@ cudaError_t sap_colour(const Geom& g, const int bs[4], int colour, int fmt, cons
   const size_t smem = sizeof(float) * 24 * nsite + sizeof(double) * 3 * (threads / 32);
   dim3 grid(nblk / 2), block(threads);
   if (eo) {
-    // even-odd reduced block solver: shared-memory operands only
-    const size_t sm2 = sap_smem_bytes(bs, 72 + 72 + 24);
+    // even-odd reduced block solver: one kernel, whatever `kernel` asks for
+    const size_t sm2 = sap_smem_bytes(bs);
     if (sm2 > 227 * 1024 || !clov_inv || bs[3] % 2) return cudaErrorInvalidValue;
     if (fmt == LINK_12) {
-      cudaFuncSetAttribute(sap_smem_eo_kernel<LINK_12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-      sap_smem_eo_kernel<LINK_12><<<grid, block, sm2, s>>>(a);
+      cudaFuncSetAttribute(sap_block_eo_kernel<LINK_12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+      sap_block_eo_kernel<LINK_12><<<grid, block, sm2, s>>>(a);
     } else {
-      cudaFuncSetAttribute(sap_smem_eo_kernel<LINK_18>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-      sap_smem_eo_kernel<LINK_18><<<grid, block, sm2, s>>>(a);
+      cudaFuncSetAttribute(sap_block_eo_kernel<LINK_18>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+      sap_block_eo_kernel<LINK_18><<<grid, block, sm2, s>>>(a);
     }
     return cudaGetLastError();
   }
   if (kernel == 0) {  // the default
-    const size_t sm2 = sap_smem_bytes(bs, 72 + 24 + 48);
+    const size_t sm2 = sap_smem_bytes(bs);
     if (fmt == LINK_12) {
       cudaFuncSetAttribute(sap_block_kernel<LINK_12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
       sap_block_kernel<LINK_12><<<grid, block, sm2, s>>>(a);

@@ -1,4 +1,4 @@
-"""The default Schwarz block kernel at the edges of its block sizes: blocks
+"""The Schwarz block kernels (full and even-odd reduced) at the edges of its block sizes: blocks
 smaller than a warp, not a multiple of a warp, extents of one site (neighbours
 outside on both sides), the largest block; an output buffer that holds NaN
 (the first cycle must not read it); no MR step at all."""
@@ -36,4 +36,27 @@ def test_block_shapes(dims, bs, ncy, nmr, link_fmt):
         assert not got.any()
     else:
         assert rel_err(got, ref) < 1e-5
+    h.close()
+
+
+@pytest.mark.parametrize("dims,bs,ncy,nmr", [((4, 4, 6, 8), (1, 2, 3, 2), 2, 3),
+                                             ((4, 2, 4, 8), (2, 1, 1, 4), 1, 4),
+                                             ((4, 12, 4, 8), (2, 6, 2, 4), 2, 2),
+                                             ((8, 8, 4, 16), (4, 4, 2, 8), 1, 3),
+                                             ((8, 8, 8, 8), (4, 4, 4, 4), 2, 0)])
+@pytest.mark.parametrize("link_fmt", [0, 1])
+def test_even_odd_block_shapes(dims, bs, ncy, nmr, link_fmt):
+    import torch
+    from paper_2202_07388_gb300 import oq
+    u, a, ainv = oracle_case(dims, 0.5, 933, 0.1365, 1.0)
+    rho = synth.make_source(dims, 934)
+    ref = solvers.sap(u, a, rho, bs, ncy, nmr, eo=True, ainv=ainv)
+    h = make_handle(dims, u, 0.1365, 1.0, link_fmt)
+    prho, pphi = h.new_packed(oq.F32), h.new_packed(oq.F32)
+    pphi.view(torch.float32).fill_(float("nan"))
+    h.pack(to_dev(rho), prho, oq.F32)
+    h.sap_apply(prho, pphi, oq.SolverParams(ncy=ncy, nmr=nmr, bs=bs, sap_eo=1))
+    out = to_dev(np.zeros_like(rho))
+    h.unpack(pphi, out, oq.F32)
+    assert rel_err(from_dev(out, rho.shape), ref) < 1e-5
     h.close()
