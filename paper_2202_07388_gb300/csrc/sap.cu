@@ -605,6 +605,250 @@ __global__ void __launch_bounds__(256, 1) sap_block_kernel(const SapArgs a) {
   if (a.mr_steps && t == 0) atomicAdd(a.mr_steps, (unsigned)steps);
 }
 
+__device__ __forceinline__ void zero_spinor(Spinor<float>& v) {
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) v.c[s][c] = cx<float>{0.f, 0.f};
+}
+
+// Two binary32 lanes of one packed instruction, for the even-odd kernel.  A spinor
+// is held as six complex pairs, lanes spin s and s + 2; links as pairs of directions
+// (0, 1) and (2, 3); a site's two clover blocks as one block of pairs.  A packed FMA
+// takes the pipe twice as long as a scalar one, so what it saves is issue: the
+// even-odd kernel, one warp per scheduler in each half pass, gains (93 to 77 us a
+// colour on 24x16^3); sap_block_kernel, two warps and 23 % fewer instructions, takes
+// 252 us instead of 239, waiting for the longer latency, and stays scalar.
+namespace eop {
+typedef float2 F2;
+struct C2 {
+  F2 re, im;
+};
+struct Sp6 {
+  C2 c[6];  // [3 s + colour]
+};
+struct Link2 {
+  C2 m[3][3];
+};
+__device__ __forceinline__ F2 bc2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ F2 ffma2(F2 a, F2 b, F2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ F2 fmul2(F2 a, F2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ F2 fsub2(F2 a, F2 b) { return __ffma2_rn(b, bc2(-1.f), a); }
+__device__ __forceinline__ C2 pair_of(cx<float> a, cx<float> b) { return C2{{a.re, b.re}, {a.im, b.im}}; }
+__device__ __forceinline__ Sp6 pack6(const Spinor<float>& v) {
+  Sp6 o;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) o.c[k] = pair_of(v.c[k / 3][k % 3], v.c[2 + k / 3][k % 3]);
+  return o;
+}
+__device__ __forceinline__ Spinor<float> spinor_of(const Sp6& v) {
+  Spinor<float> o;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    o.c[k / 3][k % 3] = cx<float>{v.c[k].re.x, v.c[k].im.x};
+    o.c[2 + k / 3][k % 3] = cx<float>{v.c[k].re.y, v.c[k].im.y};
+  }
+  return o;
+}
+template <int L>
+__device__ __forceinline__ Su3<float> link_of(const Link2& u) {
+  Su3<float> o;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+      o.m[a][b] = L ? cx<float>{u.m[a][b].re.y, u.m[a][b].im.y} : cx<float>{u.m[a][b].re.x, u.m[a][b].im.x};
+  return o;
+}
+template <int FMT>
+__device__ __forceinline__ void load_link2(const SapArgs& a, int p, int q, long i, Link2& u) {
+  Su3<float> v, w;
+  load_link<float, FMT>(a.links, a.g.Vh, p, 2 * q, i, v);
+  load_link<float, FMT>(a.links, a.g.Vh, p, 2 * q + 1, i, w);
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) u.m[c][d] = pair_of(v.m[c][d], w.m[c][d]);
+}
+__device__ __forceinline__ void sm4_load(const float4* b, int nsite, int t, Sp6& v) {
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const float4 w = b[k * nsite + t];
+    v.c[k] = C2{{w.x, w.y}, {w.z, w.w}};
+  }
+}
+__device__ __forceinline__ void sm4_store(float4* b, int nsite, int t, const Sp6& v) {
+#pragma unroll
+  for (int k = 0; k < 6; ++k) b[k * nsite + t] = make_float4(v.c[k].re.x, v.c[k].re.y, v.c[k].im.x, v.c[k].im.y);
+}
+
+// The staged clover blocks of a site, made pairs in place: slot(q) holds the reals
+// 2q and 2q + 1 of both blocks (6 diagonal, then 15 complex).
+__device__ __forceinline__ int clover_slot(int q) { return (q & 1) ? 9 + q / 2 : q / 2; }
+__device__ __forceinline__ void sm4_clover_pairs(float4* a, int nsite, int t) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const float4 v = a[k * nsite + t], w = a[(9 + k) * nsite + t];
+    a[k * nsite + t] = make_float4(v.x, w.x, v.y, w.y);
+    a[(9 + k) * nsite + t] = make_float4(v.z, w.z, v.w, w.w);
+  }
+}
+// out = A in
+__device__ __forceinline__ void sm4_clover(const float4* a, int nsite, int t, const Sp6& in, Sp6& out) {
+  const F2 m1 = bc2(-1.f);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const float4 w = a[clover_slot(q) * nsite + t];
+    out.c[2 * q] = C2{fmul2({w.x, w.y}, in.c[2 * q].re), fmul2({w.x, w.y}, in.c[2 * q].im)};
+    out.c[2 * q + 1] = C2{fmul2({w.z, w.w}, in.c[2 * q + 1].re), fmul2({w.z, w.w}, in.c[2 * q + 1].im)};
+  }
+  F2 nre[5], nim[5];  // -Re in[0 .. 4], -Im in[1 .. 5]: a packed FMA has no negated operand
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    nre[k] = fmul2(m1, in.c[k].re);
+    nim[k] = fmul2(m1, in.c[k + 1].im);
+  }
+  int q = 3;
+#pragma unroll
+  for (int r = 0; r < 6; ++r)
+#pragma unroll
+    for (int c = r + 1; c < 6; ++c) {
+      const float4 w = a[clover_slot(q) * nsite + t];
+      const F2 ore{w.x, w.y}, oim{w.z, w.w};
+      C2 &y = out.c[r], &z = out.c[c];
+      const C2 &x = in.c[c], &v = in.c[r];
+      y.re = ffma2(oim, nim[c - 1], ffma2(ore, x.re, y.re));
+      y.im = ffma2(oim, x.re, ffma2(ore, x.im, y.im));
+      z.re = ffma2(oim, v.im, ffma2(ore, v.re, z.re));
+      z.im = ffma2(oim, nre[r], ffma2(ore, v.im, z.im));
+      ++q;
+    }
+}
+
+// y = U h or U^dag h for both directions of a pair.  APART: the caller stores the two
+// directions apart, so the last operation of each real is done per lane (a lane of
+// a pair costs a move where four reals of one direction have to be neighbours).
+template <bool DAG, bool APART>
+__device__ __forceinline__ void link2_mul(const Link2& u, const HalfSpinor<float>& h0, const HalfSpinor<float>& h1,
+                                          HalfSpinor<float>& y0, HalfSpinor<float>& y1) {
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      // U: re = p - n, im = s;  U^dag: re = s, im = p - n
+      F2 sum, pos, neg;
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const C2 w = DAG ? u.m[b][a] : u.m[a][b], h = pair_of(h0.c[s][b], h1.c[s][b]);
+        const F2 f = DAG ? h.re : h.im, g = DAG ? h.im : h.re;
+        if (b == 0) {
+          sum = ffma2(w.im, g, fmul2(w.re, f));
+          pos = fmul2(w.re, g);
+          neg = fmul2(w.im, f);
+        } else {
+          pos = ffma2(w.re, g, pos);
+          neg = ffma2(w.im, f, neg);
+          sum = ffma2(w.re, f, sum);
+          if (b < 2 || !APART) sum = ffma2(w.im, g, sum);
+          else sum = F2{fmaf(w.im.x, g.x, sum.x), fmaf(w.im.y, g.y, sum.y)};
+        }
+      }
+      const F2 dif = APART ? F2{pos.x - neg.x, pos.y - neg.y} : fsub2(pos, neg);
+      y0.c[s][a] = DAG ? cx<float>{sum.x, dif.x} : cx<float>{dif.x, sum.x};
+      y1.c[s][a] = DAG ? cx<float>{sum.y, dif.y} : cx<float>{dif.y, sum.y};
+    }
+}
+
+// the sends of a site: U_mu(x)^dag (1 + g_mu) v for its forward neighbours
+template <int Q>
+__device__ __forceinline__ void sm4_send(const SapShared& m, int t, const Link2& u, const Spinor<float>& v) {
+  HalfSpinor<float> h[2], y[2];
+  project<2 * Q, +1>(v, h[0]);
+  project<2 * Q + 1, +1>(v, h[1]);
+  link2_mul<true, true>(u, h[0], h[1], y[0], y[1]);
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    const cx<float>* c = &y[d].c[0][0];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      m.s[((2 * Q + d) * 3 + k) * m.nsite + t] =
+          make_float4(c[2 * k].re, c[2 * k].im, c[2 * k + 1].re, c[2 * k + 1].im);
+  }
+}
+__device__ __forceinline__ void sm4_publish(const SapShared& m, int t, const Link2 (&u)[2], const Sp6& v) {
+  sm4_store(m.r, m.nsite, t, v);
+  const Spinor<float> w = spinor_of(v);
+  sm4_send<0>(m, t, u[0], w);
+  sm4_send<1>(m, t, u[1], w);
+}
+
+// acc += the in-block hops along 2Q and 2Q + 1 of the published field, from the
+// positions tu (above) and td (below); up / down: the site has such a neighbour in
+// the block (where not, the position is its own and the weight zero)
+template <int Q>
+__device__ __forceinline__ void sm4_hops(const SapShared& m, const int (&tu)[4], const int (&td)[4], unsigned up,
+                                         unsigned down, const Link2& u, Spinor<float>& acc) {
+  HalfSpinor<float> h[2], y[2], z[2];
+  Sp6 n;
+  sm4_load(m.r, m.nsite, tu[2 * Q], n);
+  project<2 * Q, -1>(spinor_of(n), h[0]);
+  sm4_load(m.r, m.nsite, tu[2 * Q + 1], n);
+  project<2 * Q + 1, -1>(spinor_of(n), h[1]);
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    cx<float>* c = &z[d].c[0][0];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float4 w = m.s[((2 * Q + d) * 3 + k) * m.nsite + td[2 * Q + d]];
+      c[2 * k] = cx<float>{w.x, w.y};
+      c[2 * k + 1] = cx<float>{w.z, w.w};
+    }
+  }
+  link2_mul<false, false>(u, h[0], h[1], y[0], y[1]);
+  accum_reconstruct<2 * Q, -1>(acc, y[0], up >> (2 * Q) & 1 ? -0.5f : 0.f);
+  accum_reconstruct<2 * Q, +1>(acc, z[0], down >> (2 * Q) & 1 ? -0.5f : 0.f);
+  accum_reconstruct<2 * Q + 1, -1>(acc, y[1], up >> (2 * Q + 1) & 1 ? -0.5f : 0.f);
+  accum_reconstruct<2 * Q + 1, +1>(acc, z[1], down >> (2 * Q + 1) & 1 ? -0.5f : 0.f);
+}
+
+__device__ __forceinline__ double norm2_of(const Sp6& v) { return site_norm2(spinor_of(v)); }
+// a -= b
+__device__ __forceinline__ void sp6_sub(Sp6& a, const Sp6& b) {
+#pragma unroll
+  for (int k = 0; k < 6; ++k) a.c[k] = C2{fsub2(a.c[k].re, b.c[k].re), fsub2(a.c[k].im, b.c[k].im)};
+}
+__device__ __forceinline__ void sp6_zero(Sp6& a) {
+#pragma unroll
+  for (int k = 0; k < 6; ++k) a.c[k] = C2{{0.f, 0.f}, {0.f, 0.f}};
+}
+// a site's part of <p, r> = d0 + i d1 and <p, p> = d2
+__device__ __forceinline__ void mr_dots(const Sp6& p, const Sp6& r, float& d0, float& d1, float& d2) {
+  F2 s{0.f, 0.f}, v = s, w = s, n = s;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    s = ffma2(p.c[k].im, r.c[k].im, ffma2(p.c[k].re, r.c[k].re, s));
+    v = ffma2(p.c[k].re, r.c[k].im, v);
+    w = ffma2(p.c[k].im, r.c[k].re, w);
+    n = ffma2(p.c[k].im, p.c[k].im, ffma2(p.c[k].re, p.c[k].re, n));
+  }
+  d0 = s.x + s.y;
+  d1 = (v.x - w.x) + (v.y - w.y);
+  d2 = n.x + n.y;
+}
+// x += om r, r -= om p
+__device__ __forceinline__ void mr_update(cx<float> om, const Sp6& p, Sp6& x, Sp6& r) {
+  const F2 wr = bc2(om.re), wi = bc2(om.im), nr = bc2(-om.re), ni = bc2(-om.im);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    x.c[k].re = ffma2(ni, r.c[k].im, ffma2(wr, r.c[k].re, x.c[k].re));
+    x.c[k].im = ffma2(wi, r.c[k].re, ffma2(wr, r.c[k].im, x.c[k].im));
+    r.c[k].re = ffma2(wi, p.c[k].im, ffma2(nr, p.c[k].re, r.c[k].re));
+    r.c[k].im = ffma2(ni, p.c[k].re, ffma2(nr, p.c[k].im, r.c[k].im));
+  }
+}
+
+}  // namespace eop
+
 // ---------------------------------------------------------------------------
 // Even-odd reduced block solver (openQCD's choice for SAP, Sec. 3): per block
 //   rhat_e = r_e - D_eo A_oo^{-1} r_o,
@@ -614,18 +858,11 @@ __global__ void __launch_bounds__(256, 1) sap_block_kernel(const SapArgs a) {
 // sap_block_kernel; the staged clover is A at even and A^{-1} at odd sites.  An
 // MR step is two half passes: the odd threads form A^{-1} D_oe of the published
 // even residual and publish it, the even threads form D_eo of that.  Latency
-// and shared-memory reads bound it: a half pass keeps 4 of an SM's 8 warps
-// busy, and one block fills an SM (255 registers).  (A colour of 24x16^3 in
-// 4^4 blocks, 4 MR steps: 93 us; with links and clover in shared memory and
+// and issue of one warp per scheduler bound it: a half pass keeps 4 of an SM's
+// 8 warps busy, and one block fills an SM (255 registers).  (A colour of 24x16^3
+// in 4^4 blocks, 4 MR steps: 77 us; with links and clover in shared memory and
 // both hops of a link multiplied by their reader it took 128 us.)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void zero_spinor(Spinor<float>& v) {
-#pragma unroll
-  for (int s = 0; s < 4; ++s)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) v.c[s][c] = cx<float>{0.f, 0.f};
-}
-
 // The block's sites are held parity-sorted: position k < nsite/2 is the
 // block-local-even site with in-block lexicographic index n = 2k + c, c
 // fixing the parity (bs[3] even, so the sites of one parity alternate along
@@ -692,42 +929,42 @@ __global__ void __launch_bounds__(256, 1) sap_block_eo_kernel(const SapArgs a) {
   }
   const int w = t >> 5, nw = (blockDim.x + 31) >> 5;
 
-  Spinor<float> r, xs;  // r: the residual (odd sites), rhat (even sites)
-  zero_spinor(r);
-  zero_spinor(xs);
-  Su3<float> u[4];
+  eop::Sp6 r, xs;  // r: the residual (odd sites), rhat (even sites)
+  eop::sp6_zero(r);
+  eop::sp6_zero(xs);
+  eop::Link2 u[2];
   // acc += the in-block hops of the published field
   auto dhop = [&](Spinor<float>& acc) {
-    sm4_hop<0>(m, tu[0], td[0], up & 1, down & 1, u[0], acc);
-    sm4_hop<1>(m, tu[1], td[1], up & 2, down & 2, u[1], acc);
-    sm4_hop<2>(m, tu[2], td[2], up & 4, down & 4, u[2], acc);
-    sm4_hop<3>(m, tu[3], td[3], up & 8, down & 8, u[3], acc);
+    eop::sm4_hops<0>(m, tu, td, up, down, u[0], acc);
+    eop::sm4_hops<1>(m, tu, td, up, down, u[1], acc);
   };
   char* phi = a.phi + (long)p * a.half_bytes;
+  Spinor<float> acc;
+  zero_spinor(acc);
   if (act) {
     const float4* q = reinterpret_cast<const float4*>(p ? a.clov_inv : a.clov) + (long)p * 18 * a.g.Vh + i;
 #pragma unroll
     for (int k = 0; k < 18; ++k) cp_async16(m.a + k * nsite + t, q + k * a.g.Vh);
     cp_async_commit();
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) load_link<float, FMT>(a.links, a.g.Vh, p, mu, i, u[mu]);
-    // block residual rho - D phi: the hops from outside the block
+    eop::load_link2<FMT>(a, p, 0, i, u[0]);
+    eop::load_link2<FMT>(a, p, 1, i, u[1]);
+    // block residual rho - D phi; the hops from outside the block first
     if (!(a.first && a.colour == 0)) {
       const char* nbf = a.phi + (long)(1 - p) * a.half_bytes;
-      outer_hop<FMT, 3>(a, nbf, p, x, up & 8, down & 8, u[3], r);
-      outer_hop<FMT, 2>(a, nbf, p, x, up & 4, down & 4, u[2], r);
-      outer_hop<FMT, 1>(a, nbf, p, x, up & 2, down & 2, u[1], r);
-      outer_hop<FMT, 0>(a, nbf, p, x, up & 1, down & 1, u[0], r);
+      outer_hop<FMT, 3>(a, nbf, p, x, up & 8, down & 8, eop::link_of<1>(u[1]), acc);
+      outer_hop<FMT, 2>(a, nbf, p, x, up & 4, down & 4, eop::link_of<0>(u[1]), acc);
+      outer_hop<FMT, 1>(a, nbf, p, x, up & 2, down & 2, eop::link_of<1>(u[0]), acc);
+      outer_hop<FMT, 0>(a, nbf, p, x, up & 1, down & 1, eop::link_of<0>(u[0]), acc);
+    }
+    Spinor<float> v;
+    load_spinor<P_F32>(a.rho + (long)p * a.half_bytes, a.g.Vh, i, v);
+    r = eop::pack6(v);
+    if (!a.first) {
+      load_spinor<P_F32>(phi, a.g.Vh, i, v);
+      xs = eop::pack6(v);
     }
     if (!a.first) {
-      Spinor<float> ph, aph;
-      load_spinor<P_F32>(phi, a.g.Vh, i, ph);
-      sm4_publish(m, t, u, ph);
-      clover_apply<float>(a.clov, a.g.Vh, p, i, ph, aph);
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) r.c[s][c] = r.c[s][c] + aph.c[s][c];
+      eop::sm4_publish(m, t, u, xs);
     } else {
       // a dropped hop reads its own position with weight zero: that must hold numbers
       const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -736,71 +973,59 @@ __global__ void __launch_bounds__(256, 1) sap_block_eo_kernel(const SapArgs a) {
 #pragma unroll
       for (int k = 0; k < 12; ++k) m.s[k * nsite + t] = z;
     }
+    if (!a.first) {
+      v = eop::spinor_of(xs);
+      Spinor<float> aph;
+      clover_apply<float>(a.clov, a.g.Vh, p, i, v, aph);
+      eop::sp6_sub(r, eop::pack6(aph));
+      eop::sp6_zero(xs);
+    }
     cp_async_wait();
+    eop::sm4_clover_pairs(m.a, nsite, t);  // read by this thread alone
   }
   if (!a.first) {
     __syncthreads();  // the published phi
-    if (act) dhop(r);
+    if (act) dhop(acc);
     __syncthreads();  // every read of it is done
   }
-  if (act) {
-    Spinor<float> rh;
-    load_spinor<P_F32>(a.rho + (long)p * a.half_bytes, a.g.Vh, i, rh);
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) r.c[s][c] = rh.c[s][c] - r.c[s][c];
-  }
+  eop::sp6_sub(r, eop::pack6(acc));
   // odd sites publish A^{-1} r_o; even sites: rhat_e = r_e - D_eo A^{-1} r_o
   if (od) {
-    Spinor<float> v;
-    sm4_clover(m.a, nsite, t, r, v);
-    sm4_publish(m, t, u, v);
+    eop::Sp6 v;
+    eop::sm4_clover(m.a, nsite, t, r, v);
+    eop::sm4_publish(m, t, u, v);
   }
   __syncthreads();
   if (ev) {
-    Spinor<float> acc;
     zero_spinor(acc);
     dhop(acc);
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) r.c[s][c] = r.c[s][c] - acc.c[s][c];
-    sm4_publish(m, t, u, r);  // at even positions, which no one reads in this phase
+    eop::sp6_sub(r, eop::pack6(acc));
+    eop::sm4_publish(m, t, u, r);  // at even positions, which no one reads in this phase
   }
   double rn_prev = 0.0;
-  if (a.adaptive) rn_prev = sqrt(block_sum1(ev ? site_norm2(r) : 0.0, reinterpret_cast<double*>(red)));
+  if (a.adaptive) rn_prev = sqrt(block_sum1(ev ? eop::norm2_of(r) : 0.0, reinterpret_cast<double*>(red)));
   __syncthreads();
 
   int steps = 0;
   for (int k = 1; k <= a.nmr; ++k) {
     // odd half pass: t_o = A^{-1} D_oe rhat_e
     if (od) {
-      Spinor<float> acc, v;
       zero_spinor(acc);
       dhop(acc);
-      sm4_clover(m.a, nsite, t, acc, v);
-      sm4_publish(m, t, u, v);
+      eop::Sp6 v;
+      eop::sm4_clover(m.a, nsite, t, eop::pack6(acc), v);
+      eop::sm4_publish(m, t, u, v);
     }
     __syncthreads();
     // even half pass: q_e = A rhat_e - D_eo t_o, then <q, rhat>, <q, q>
-    Spinor<float> pv;
+    eop::Sp6 pv;
     float d0 = 0.f, d1 = 0.f, d2 = 0.f;
     if (ev) {
-      Spinor<float> acc;
-      sm4_clover(m.a, nsite, t, r, pv);
+      eop::sm4_clover(m.a, nsite, t, r, pv);
       zero_spinor(acc);
       dhop(acc);
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          pv.c[s][c] = pv.c[s][c] - acc.c[s][c];
-          const cx<float> q = pv.c[s][c], v = r.c[s][c];
-          d0 += q.re * v.re + q.im * v.im;
-          d1 += q.re * v.im - q.im * v.re;
-          d2 += q.re * q.re + q.im * q.im;
-        }
+      eop::sp6_sub(pv, eop::pack6(acc));
+      eop::mr_dots(pv, r, d0, d1, d2);
     }
     d0 = warp_sum_f(d0);
     d1 = warp_sum_f(d1);
@@ -820,46 +1045,37 @@ __global__ void __launch_bounds__(256, 1) sap_block_eo_kernel(const SapArgs a) {
     cx<float> om{0.f, 0.f};
     if (d2 > 0.f) om = cx<float>{d0 / d2, d1 / d2};
     if (ev) {
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          cfma(xs.c[s][c], om, r.c[s][c]);
-          r.c[s][c] = r.c[s][c] - om * pv.c[s][c];
-        }
-      sm4_publish(m, t, u, r);
+      eop::mr_update(om, pv, xs, r);
+      eop::sm4_publish(m, t, u, r);
     }
     steps = k;
     if (a.adaptive) {
-      const double rn_new = sqrt(block_sum1(ev ? site_norm2(r) : 0.0, reinterpret_cast<double*>(red)));
+      const double rn_new = sqrt(block_sum1(ev ? eop::norm2_of(r) : 0.0, reinterpret_cast<double*>(red)));
       if ((k >= 4 && rn_new > (double)a.alpha * rn_prev) || rn_new > rn_prev || rn_new < a.tol) break;
       rn_prev = rn_new;
     }
     __syncthreads();  // the odd half pass of the next step reads the even residual
   }
   // delta_e = x_e published; delta_o = A^{-1} (r_o - D_oe delta_e)
-  if (ev) sm4_publish(m, t, u, xs);
+  if (ev) eop::sm4_publish(m, t, u, xs);
   __syncthreads();
   if (od) {
-    Spinor<float> acc;
     zero_spinor(acc);
     dhop(acc);
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) r.c[s][c] = r.c[s][c] - acc.c[s][c];
-    sm4_clover(m.a, nsite, t, r, xs);
+    eop::sp6_sub(r, eop::pack6(acc));
+    eop::sm4_clover(m.a, nsite, t, r, xs);
   }
   if (act) {
+    Spinor<float> v = eop::spinor_of(xs);
     if (!a.first) {
       Spinor<float> ph;
       load_spinor<P_F32>(phi, a.g.Vh, i, ph);
 #pragma unroll
       for (int s = 0; s < 4; ++s)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) xs.c[s][c] = ph.c[s][c] + xs.c[s][c];
+        for (int c = 0; c < 3; ++c) v.c[s][c] = ph.c[s][c] + v.c[s][c];
     }
-    store_spinor<P_F32>(phi, a.g.Vh, i, xs);
+    store_spinor<P_F32>(phi, a.g.Vh, i, v);
   }
   if (a.mr_steps && t == 0) atomicAdd(a.mr_steps, (unsigned)steps);
 }
