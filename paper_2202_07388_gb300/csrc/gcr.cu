@@ -248,7 +248,7 @@ extern "C" int oq_sap_apply(oq_handle h, int lat, const oq_solver_params* prm, c
     for (int colour = 0; colour < 2; ++colour) {
       h->launches += 1;
       if (sap_colour(L.g, prm->bs, colour, L.link_fmt, L.u32.p, L.a32.p, L.i32.p, rho_dev, phi_dev, prm->nmr,
-                     prm->adaptive, alpha, mr_tol, nullptr, h->sap_kernel, prm->sap_eo, cy, s) != cudaSuccess)
+                     prm->adaptive, alpha, mr_tol, nullptr, h->sap_kernel, prm->sap_eo, cy, SapBlocked(), s) != cudaSuccess)
         return OQ_ERR_CUDA;
     }
   return OQ_OK;
@@ -356,6 +356,28 @@ static int gcr_impl(oq_handle h, int lat, const oq_solver_params* prm, const flo
     return h->run_hop(h->hop_launch(lat, prec, HOP_DW, 0, EPI_NONE, 1), a, s);
   };
 
+  // The SAP kernels' operands in block order, made once per solve (the links and
+  // clover may change between solves) when it first applies SAP: a launch saves 24
+  // of 228 us on 48x24^3, the copies take 113 us, so they pay from the fifth launch
+  // (18 steps of 8 launches there: 45.7 to 42.5 ms).  oq_sap_apply, which applies
+  // SAP once, reads the packed fields.  Where the device has no room for them SAP reads the packed fields.
+  SapBlocked blk;
+  bool blk_asked = false;
+  auto block_order = [&]() -> int {
+    if (blk_asked || (h->sap_kernel != 0 && !prm->sap_eo)) return OQ_OK;
+    blk_asked = true;
+    if (prm->sap_eo && !L.i32.p) return OQ_OK;  // refused by sap_colour
+    size_t nl, nc;
+    sap_blocked_bytes(L.g, L.link_fmt, &nl, &nc);
+    void* bc = nullptr;
+    if (h->workspace(lat, "gcr_sap", nc + nl, &bc)) return OQ_OK;
+    char* bl = (char*)bc + nc;
+    KL(sap_blocked(L.g, prm->bs, L.link_fmt, L.u32.p, L.a32.p, L.i32.p, prm->sap_eo, bl, bc, s));
+    blk.links = bl;
+    blk.clov = bc;
+    return OQ_OK;
+  };
+
   int ret = OQ_OK;
   for (int r = 0; r < nrhs; ++r) {
     const double* eta_r = eta_dev + (long)r * 2 * Vh * 24;
@@ -399,6 +421,7 @@ static int gcr_impl(oq_handle h, int lat, const oq_solver_params* prm, const flo
         } else if (prm->ncy == 0) {
           CK(cudaMemcpyAsync(phik, rho, f32, cudaMemcpyDeviceToDevice, s));
         } else {
+          RK(block_order());
           double prev = 0.0;
           if (prm->adaptive) {
             CK(cudaMemsetAsync(phik, 0, f32, s));
@@ -411,7 +434,7 @@ static int gcr_impl(oq_handle h, int lat, const oq_solver_params* prm, const flo
             for (int colour = 0; colour < 2; ++colour)
               KL(sap_colour(L.g, prm->bs, colour, L.link_fmt, L.u32.p, L.a32.p, L.i32.p, rho, phik, prm->nmr,
                             prm->adaptive, (float)(prm->alpha > 0.0 ? prm->alpha : 0.9), prm->res * eta_n / nblk,
-                            (unsigned*)mrc, h->sap_kernel, prm->sap_eo, cy, s));
+                            (unsigned*)mrc, h->sap_kernel, prm->sap_eo, cy, blk, s));
             cycles_total += 1;
             if (prm->adaptive) {
               // cycle test on the global SAP residual ||rho - D phi||

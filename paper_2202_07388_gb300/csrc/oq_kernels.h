@@ -64,13 +64,23 @@ int nnprec_forward(struct ::oq_ctx* h, int lat, const void* r, void* y, cudaStre
 // takes the binary32 master weights, synchronises s, OQ_ERR_TIMEOUT on a failed wait
 int nnprec_forward_tc(struct ::oq_ctx* h, int lat, const float* master, const void* r, void* y, cudaStream_t s);
 
+// block-ordered copies of the binary32 links and clover (sap_blocked); null: none
+struct SapBlocked {
+  const void* links = nullptr;
+  const void* clov = nullptr;
+};
 // one SAP half cycle: every block of `colour` (binary32 fields); cycle: the
 // Schwarz cycle's number (in cycle 0 phi counts as zero whatever it holds, and
 // colours 0, 1 set all of it); eo: MR on the blocks' even-odd Schur complements
 // (needs clov_inv and blocks whose operands fit in shared memory, else
-// cudaErrorInvalidValue)
+// cudaErrorInvalidValue); blk: made for the same bs and eo, or empty (kernel 0 and eo only)
 cudaError_t sap_colour(const Geom& g, const int bs[4], int colour, int fmt, const void* links, const void* clov,
                        const void* clov_inv, const void* rho, void* phi, int nmr, int adaptive, float alpha,
-                       double tol, unsigned* mr_steps, int kernel, int eo, int cycle, cudaStream_t s);
+                       double tol, unsigned* mr_steps, int kernel, int eo, int cycle, const SapBlocked& blk,
+                       cudaStream_t s);
+// the block-ordered copies: their sizes, and the pass that makes them
+void sap_blocked_bytes(const Geom& g, int fmt, size_t* links, size_t* clov);
+cudaError_t sap_blocked(const Geom& g, const int bs[4], int fmt, const void* links, const void* clov,
+                        const void* clov_inv, int eo, void* blinks, void* bclov, cudaStream_t s);
 
 }  // namespace oq

@@ -36,6 +36,7 @@ struct SapArgs {
   const void* links;   // binary32 packed links
   const void* clov;    // binary32 packed clover
   const void* clov_inv;  // binary32 packed inverse clover (even-odd block solver)
+  SapBlocked blk;        // copies of a site's own links and clover in block order (null: none)
   const char* rho;     // packed binary32 full field
   char* phi;           // packed binary32 full field, updated in place
   long half_bytes;
@@ -291,10 +292,14 @@ __global__ void __launch_bounds__(256, MINB) sap_kernel(const SapArgs a) {
 // same shared-memory operator and reads only the neighbours outside the block
 // from global memory.  In the first cycle (FIRST) phi is zero on the blocks of
 // this colour (and, with colour 0, everywhere), so those terms are left out.
-// Bound by latency at one block of 8 warps per SM (255 registers, 147 KB): issue
-// 38 % active, a third of the time in staging.  48x24^3, 4^4 blocks, 5 MR steps:
-// 233 us a launch against 338 us with links and residual in shared memory as
-// described above.
+// BLK: own links and clover from the block-ordered copies (sap_blocked_kernel).
+// Bound by latency at one block of 8 warps per SM (255 registers, 147 KB): an MR
+// step runs two thirds of the issue slots (20 us of a launch, 48x24^3 in 4^4
+// blocks), loading a block and the hops from outside it overlap with nothing.
+// 5 MR steps there: 204 us a launch; 338 us with links and residual in shared
+// memory and the operands in packed order.  Two threads per site (512 at 128
+// registers) took 287 against 228 us, both directions' outside operands
+// requested together 243, and an L2 prefetch of the next block 210 against 204.
 // Shared memory: 72 + 24 + 48 floats per block site.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cp_async16(float4* smem, const float4* gmem) {
@@ -304,6 +309,28 @@ __device__ __forceinline__ void cp_async16(float4* smem, const float4* gmem) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
+// where a site's own links and clover lie: packed order (parity p, field stride V,
+// index i) or, with block-ordered copies, the same expression with the block's
+// number, its volume and the thread's position
+struct OwnAt {
+  long p, V, i;
+};
+template <bool BLK>
+__device__ __forceinline__ OwnAt own_at(const SapArgs& a, int nsite, int block, int t, int p, long i) {
+  if (BLK) return OwnAt{block, nsite, t};
+  return OwnAt{p, a.g.Vh, i};
+}
+// coordinates of the n-th block of the colour, and its number among all blocks
+__device__ __forceinline__ int colour_block(const SapArgs& a, int n, int (&bc)[4]) {
+  const int half3 = a.nb[3] / 2;
+  int row = n / half3;
+  bc[2] = row % a.nb[2];
+  row /= a.nb[2];
+  bc[1] = row % a.nb[1];
+  bc[0] = row / a.nb[1];
+  bc[3] = 2 * (n % half3) + ((a.colour + bc[0] + bc[1] + bc[2]) & 1);
+  return ((bc[0] * a.nb[1] + bc[1]) * a.nb[2] + bc[2]) * a.nb[3] + bc[3];
+}
 struct SapShared {
   float4* a;  // [18][nsite] clover (two blocks: 6 diagonal + 15 complex each)
   float4* r;  // [6][nsite] residual, two complex components per chunk
@@ -440,7 +467,7 @@ __device__ __forceinline__ void outer_hop(const SapArgs& a, const char* nbf, int
   }
 }
 
-template <int FMT>
+template <int FMT, bool BLK>
 __global__ void __launch_bounds__(256, 1) sap_block_kernel(const SapArgs a) {
   extern __shared__ float4 sm4[];
   const int nsite = a.bs[0] * a.bs[1] * a.bs[2] * a.bs[3];
@@ -452,14 +479,8 @@ __global__ void __launch_bounds__(256, 1) sap_block_kernel(const SapArgs a) {
   float* red = reinterpret_cast<float*>(sm4 + 36 * nsite);  // 3 partials per warp (binary64: block_sum1)
   const int t = threadIdx.x;
   const bool act = t < nsite;
-  const int half3 = a.nb[3] / 2;
-  int row = blockIdx.x / half3;
-  const int mb = blockIdx.x % half3;
-  const int bc2 = row % a.nb[2];
-  row /= a.nb[2];
-  const int bc1 = row % a.nb[1];
-  const int bc0 = row / a.nb[1];
-  const int bc3 = 2 * mb + ((a.colour + bc0 + bc1 + bc2) & 1);
+  int bc[4];
+  const int block = colour_block(a, blockIdx.x, bc);
   const int stride[4] = {a.bs[1] * a.bs[2] * a.bs[3], a.bs[2] * a.bs[3], a.bs[3], 1};
   int l[4], x[4];
   {
@@ -471,12 +492,13 @@ __global__ void __launch_bounds__(256, 1) sap_block_kernel(const SapArgs a) {
     l[1] = tt % a.bs[1];
     l[0] = tt / a.bs[1];
   }
-  x[0] = bc0 * a.bs[0] + l[0];
-  x[1] = bc1 * a.bs[1] + l[1];
-  x[2] = bc2 * a.bs[2] + l[2];
-  x[3] = bc3 * a.bs[3] + l[3];
+  x[0] = bc[0] * a.bs[0] + l[0];
+  x[1] = bc[1] * a.bs[1] + l[1];
+  x[2] = bc[2] * a.bs[2] + l[2];
+  x[3] = bc[3] * a.bs[3] + l[3];
   const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
   const long i = eo_index(a.g, x);
+  const OwnAt own = own_at<BLK>(a, nsite, block, t, p, i);
   unsigned up = 0, down = 0;
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
@@ -493,12 +515,13 @@ __global__ void __launch_bounds__(256, 1) sap_block_kernel(const SapArgs a) {
     for (int c = 0; c < 3; ++c) r.c[s][c] = xs.c[s][c] = cx<float>{0.f, 0.f};
   char* phi = a.phi + (long)p * a.half_bytes;
   if (act) {
-    const float4* q = reinterpret_cast<const float4*>(a.clov) + (long)p * 18 * a.g.Vh + i;
+    const float4* q = reinterpret_cast<const float4*>(BLK ? a.blk.clov : a.clov) + own.p * 18 * own.V + own.i;
 #pragma unroll
-    for (int k = 0; k < 18; ++k) cp_async16(m.a + k * nsite + t, q + k * a.g.Vh);
+    for (int k = 0; k < 18; ++k) cp_async16(m.a + k * nsite + t, q + k * own.V);
     cp_async_commit();
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu) load_link<float, FMT>(a.links, a.g.Vh, p, mu, i, u[mu]);
+    for (int mu = 0; mu < 4; ++mu)
+      load_link<float, FMT>(BLK ? a.blk.links : a.links, own.V, (int)own.p, mu, own.i, u[mu]);
     // 1. block residual rho - D phi: the hops from outside the block
     if (!(a.first && a.colour == 0)) {
       const char* nbf = a.phi + (long)(1 - p) * a.half_bytes;
@@ -660,11 +683,12 @@ __device__ __forceinline__ Su3<float> link_of(const Link2& u) {
       o.m[a][b] = L ? cx<float>{u.m[a][b].re.y, u.m[a][b].im.y} : cx<float>{u.m[a][b].re.x, u.m[a][b].im.x};
   return o;
 }
-template <int FMT>
-__device__ __forceinline__ void load_link2(const SapArgs& a, int p, int q, long i, Link2& u) {
+template <int FMT, bool BLK>
+__device__ __forceinline__ void load_link2(const SapArgs& a, const OwnAt& own, int q, Link2& u) {
+  const void* b = BLK ? a.blk.links : a.links;
   Su3<float> v, w;
-  load_link<float, FMT>(a.links, a.g.Vh, p, 2 * q, i, v);
-  load_link<float, FMT>(a.links, a.g.Vh, p, 2 * q + 1, i, w);
+  load_link<float, FMT>(b, own.V, (int)own.p, 2 * q, own.i, v);
+  load_link<float, FMT>(b, own.V, (int)own.p, 2 * q + 1, own.i, w);
 #pragma unroll
   for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -869,8 +893,19 @@ __device__ __forceinline__ void mr_update(cx<float> om, const Sp6& p, Sp6& x, Sp
 // x3), positions from nsite/2 on the local-odd sites.  A half pass then runs
 // whole warps instead of every other lane.
 __device__ __forceinline__ int eo_pos(int n, int par, int half) { return par * half + (n >> 1); }
+// coordinates in the block and in-block index of the k-th site of a parity
+__device__ __forceinline__ int eo_site(const SapArgs& a, int k, int par, int (&l)[4]) {
+  int rr = (2 * k) / a.bs[3];  // the row (l0, l1, l2) of in-block index 2k + c
+  l[2] = rr % a.bs[2];
+  rr /= a.bs[2];
+  l[1] = rr % a.bs[1];
+  l[0] = rr / a.bs[1];
+  const int c = (par + l[0] + l[1] + l[2]) & 1;
+  l[3] = (2 * k) % a.bs[3] + c;
+  return 2 * k + c;
+}
 
-template <int FMT>
+template <int FMT, bool BLK>
 __global__ void __launch_bounds__(256, 1) sap_block_eo_kernel(const SapArgs a) {
   extern __shared__ float4 sm4[];
   const int nsite = a.bs[0] * a.bs[1] * a.bs[2] * a.bs[3];
@@ -882,35 +917,23 @@ __global__ void __launch_bounds__(256, 1) sap_block_eo_kernel(const SapArgs a) {
   float* red = reinterpret_cast<float*>(sm4 + 36 * nsite);  // 3 partials per warp (binary64: block_sum1)
   const int t = threadIdx.x;
   const bool act = t < nsite;
-  const int half3 = a.nb[3] / 2;
-  int row = blockIdx.x / half3;
-  const int mb = blockIdx.x % half3;
-  const int bc2 = row % a.nb[2];
-  row /= a.nb[2];
-  const int bc1 = row % a.nb[1];
-  const int bc0 = row / a.nb[1];
-  const int bc3 = 2 * mb + ((a.colour + bc0 + bc1 + bc2) & 1);
+  int bc[4];
+  const int block = colour_block(a, blockIdx.x, bc);
   // thread t holds the site at parity-sorted position t (see eo_pos)
   const int half = nsite >> 1;
   const int par = (act && t >= half) ? 1 : 0;  // block-local parity
   int l[4], x[4], n;
   {
     const int k = act ? t - par * half : 0;
-    int rr = (2 * k) / a.bs[3];  // the row (l0, l1, l2) of in-block index 2k + c
-    l[2] = rr % a.bs[2];
-    rr /= a.bs[2];
-    l[1] = rr % a.bs[1];
-    l[0] = rr / a.bs[1];
-    const int c = (par + l[0] + l[1] + l[2]) & 1;
-    l[3] = (2 * k) % a.bs[3] + c;
-    n = 2 * k + c;
+    n = eo_site(a, k, par, l);
   }
-  x[0] = bc0 * a.bs[0] + l[0];
-  x[1] = bc1 * a.bs[1] + l[1];
-  x[2] = bc2 * a.bs[2] + l[2];
-  x[3] = bc3 * a.bs[3] + l[3];
+  x[0] = bc[0] * a.bs[0] + l[0];
+  x[1] = bc[1] * a.bs[1] + l[1];
+  x[2] = bc[2] * a.bs[2] + l[2];
+  x[3] = bc[3] * a.bs[3] + l[3];
   const int p = (x[0] + x[1] + x[2] + x[3]) & 1;  // lattice parity (the Schur complement's)
   const long i = eo_index(a.g, x);
+  const OwnAt own = own_at<BLK>(a, nsite, block, t, p, i);
   const bool ev = act && p == 0, od = act && p == 1;
   const int stride[4] = {a.bs[1] * a.bs[2] * a.bs[3], a.bs[2] * a.bs[3], a.bs[3], 1};
   unsigned up = 0, down = 0;
@@ -942,12 +965,13 @@ __global__ void __launch_bounds__(256, 1) sap_block_eo_kernel(const SapArgs a) {
   Spinor<float> acc;
   zero_spinor(acc);
   if (act) {
-    const float4* q = reinterpret_cast<const float4*>(p ? a.clov_inv : a.clov) + (long)p * 18 * a.g.Vh + i;
+    const float4* q = reinterpret_cast<const float4*>(BLK ? a.blk.clov : p ? a.clov_inv : a.clov) +
+                      own.p * 18 * own.V + own.i;
 #pragma unroll
-    for (int k = 0; k < 18; ++k) cp_async16(m.a + k * nsite + t, q + k * a.g.Vh);
+    for (int k = 0; k < 18; ++k) cp_async16(m.a + k * nsite + t, q + k * own.V);
     cp_async_commit();
-    eop::load_link2<FMT>(a, p, 0, i, u[0]);
-    eop::load_link2<FMT>(a, p, 1, i, u[1]);
+    eop::load_link2<FMT, BLK>(a, own, 0, u[0]);
+    eop::load_link2<FMT, BLK>(a, own, 1, u[1]);
     // block residual rho - D phi; the hops from outside the block first
     if (!(a.first && a.colour == 0)) {
       const char* nbf = a.phi + (long)(1 - p) * a.half_bytes;
@@ -1080,6 +1104,87 @@ __global__ void __launch_bounds__(256, 1) sap_block_eo_kernel(const SapArgs a) {
   if (a.mr_steps && t == 0) atomicAdd(a.mr_steps, (unsigned)steps);
 }
 
+// ---------------------------------------------------------------------------
+// Block-ordered copies of the links and the clover: [block][chunk][position], the
+// order in which the block kernels' threads read them.  In packed order a block of
+// 4^4 sites reads runs of 32 bytes (two sites of a parity along x3) whose 64-byte
+// DRAM neighbours belong to the other colour: a launch fetched twice its bytes
+// (382 MB of DRAM reads for 191 MB on 48x24^3).  EO: A at lattice-even and A^{-1}
+// at lattice-odd sites, positions sorted by the block-local parity.
+// One CTA per block, one thread per site; 113 us on 48x24^3, where a colour takes
+// 204 us from the copies and 228 us from the packed fields.
+// ---------------------------------------------------------------------------
+template <int EO>
+__global__ void __launch_bounds__(256) sap_blocked_kernel(const SapArgs a, int link_chunks, int link_words,
+                                                          char* links, float4* clov) {
+  const int nsite = a.bs[0] * a.bs[1] * a.bs[2] * a.bs[3];
+  const int t = threadIdx.x;
+  if (t >= nsite) return;
+  int l[4], x[4];
+  if (EO) {
+    const int half = nsite >> 1, par = t >= half;
+    eo_site(a, t - par * half, par, l);
+  } else {
+    int tt = t;
+    l[3] = tt % a.bs[3];
+    tt /= a.bs[3];
+    l[2] = tt % a.bs[2];
+    tt /= a.bs[2];
+    l[1] = tt % a.bs[1];
+    l[0] = tt / a.bs[1];
+  }
+  const int block = blockIdx.x;
+  int bb = block;
+#pragma unroll
+  for (int mu = 3; mu >= 0; --mu) {
+    x[mu] = (bb % a.nb[mu]) * a.bs[mu] + l[mu];
+    bb /= a.nb[mu];
+  }
+  const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
+  const long i = eo_index(a.g, x), Vh = a.g.Vh;
+  const float4* q = reinterpret_cast<const float4*>(EO && p ? a.clov_inv : a.clov) + (long)p * 18 * Vh + i;
+  float4* d = clov + (long)block * 18 * nsite + t;
+#pragma unroll 6
+  for (int k = 0; k < 18; ++k) d[k * nsite] = q[k * Vh];
+  if (link_words == 4) {
+    const float4* f = reinterpret_cast<const float4*>(a.links) + (long)p * link_chunks * Vh + i;
+    float4* o = reinterpret_cast<float4*>(links) + (long)block * link_chunks * nsite + t;
+#pragma unroll 6
+    for (int k = 0; k < link_chunks; ++k) o[k * nsite] = f[k * Vh];
+  } else {
+    const float2* f = reinterpret_cast<const float2*>(a.links) + (long)p * link_chunks * Vh + i;
+    float2* o = reinterpret_cast<float2*>(links) + (long)block * link_chunks * nsite + t;
+#pragma unroll 6
+    for (int k = 0; k < link_chunks; ++k) o[k * nsite] = f[k * Vh];
+  }
+}
+
+void sap_blocked_bytes(const Geom& g, int fmt, size_t* links, size_t* clov) {
+  *links = (size_t)(fmt == LINK_12 ? 12 * sizeof(float4) : 36 * sizeof(float2)) * 2 * g.Vh;
+  *clov = 18 * sizeof(float4) * 2 * (size_t)g.Vh;
+}
+
+cudaError_t sap_blocked(const Geom& g, const int bs[4], int fmt, const void* links, const void* clov,
+                        const void* clov_inv, int eo, void* blinks, void* bclov, cudaStream_t s) {
+  SapArgs a = {};
+  a.g = g;
+  int nblk = 1, nsite = 1;
+  for (int mu = 0; mu < 4; ++mu) {
+    a.bs[mu] = bs[mu];
+    a.nb[mu] = g.L[mu] / bs[mu];
+    nblk *= a.nb[mu];
+    nsite *= bs[mu];
+  }
+  a.links = links;
+  a.clov = clov;
+  a.clov_inv = clov_inv;
+  const int chunks = fmt == LINK_12 ? 12 : 36, words = fmt == LINK_12 ? 4 : 2;
+  const dim3 block((nsite + 31) / 32 * 32);
+  if (eo) sap_blocked_kernel<1><<<nblk, block, 0, s>>>(a, chunks, words, (char*)blinks, (float4*)bclov);
+  else sap_blocked_kernel<0><<<nblk, block, 0, s>>>(a, chunks, words, (char*)blinks, (float4*)bclov);
+  return cudaGetLastError();
+}
+
 // clover, residual and sends of a block in shared memory; at most 147 KB (256 sites)
 static size_t sap_smem_bytes(const int bs[4]) {
   const int nsite = bs[0] * bs[1] * bs[2] * bs[3];
@@ -1089,8 +1194,10 @@ static size_t sap_smem_bytes(const int bs[4]) {
 
 cudaError_t sap_colour(const Geom& g, const int bs[4], int colour, int fmt, const void* links, const void* clov,
                        const void* clov_inv, const void* rho, void* phi, int nmr, int adaptive, float alpha,
-                       double tol, unsigned* mr_steps, int kernel, int eo, int cycle, cudaStream_t s) {
+                       double tol, unsigned* mr_steps, int kernel, int eo, int cycle, const SapBlocked& blk,
+                       cudaStream_t s) {
   SapArgs a;
+  a.blk = blk;
   a.first = cycle == 0;
   // every block is written in the first cycle; the kernels that read phi there need zeros
   if (cycle == 0 && colour == 0 && !eo && kernel != 0) {
@@ -1120,28 +1227,25 @@ cudaError_t sap_colour(const Geom& g, const int bs[4], int colour, int fmt, cons
   const int threads = (nsite + 31) / 32 * 32;
   const size_t smem = sizeof(float) * 24 * nsite + sizeof(double) * 3 * (threads / 32);
   dim3 grid(nblk / 2), block(threads);
+  const bool ord = blk.links != nullptr;
+  auto launch = [&](void (*k)(SapArgs), size_t bytes) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    k<<<grid, block, bytes, s>>>(a);
+  };
   if (eo) {
     // even-odd reduced block solver: one kernel, whatever `kernel` asks for
     const size_t sm2 = sap_smem_bytes(bs);
     if (sm2 > 227 * 1024 || !clov_inv || bs[3] % 2) return cudaErrorInvalidValue;
-    if (fmt == LINK_12) {
-      cudaFuncSetAttribute(sap_block_eo_kernel<LINK_12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-      sap_block_eo_kernel<LINK_12><<<grid, block, sm2, s>>>(a);
-    } else {
-      cudaFuncSetAttribute(sap_block_eo_kernel<LINK_18>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-      sap_block_eo_kernel<LINK_18><<<grid, block, sm2, s>>>(a);
-    }
+    launch(fmt == LINK_12 ? (ord ? sap_block_eo_kernel<LINK_12, true> : sap_block_eo_kernel<LINK_12, false>)
+                          : (ord ? sap_block_eo_kernel<LINK_18, true> : sap_block_eo_kernel<LINK_18, false>),
+           sm2);
     return cudaGetLastError();
   }
   if (kernel == 0) {  // the default
     const size_t sm2 = sap_smem_bytes(bs);
-    if (fmt == LINK_12) {
-      cudaFuncSetAttribute(sap_block_kernel<LINK_12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-      sap_block_kernel<LINK_12><<<grid, block, sm2, s>>>(a);
-    } else {
-      cudaFuncSetAttribute(sap_block_kernel<LINK_18>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
-      sap_block_kernel<LINK_18><<<grid, block, sm2, s>>>(a);
-    }
+    launch(fmt == LINK_12 ? (ord ? sap_block_kernel<LINK_12, true> : sap_block_kernel<LINK_12, false>)
+                          : (ord ? sap_block_kernel<LINK_18, true> : sap_block_kernel<LINK_18, false>),
+           sm2);
     return cudaGetLastError();
   }
   if (kernel == 2) {

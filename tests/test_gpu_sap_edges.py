@@ -60,3 +60,31 @@ def test_even_odd_block_shapes(dims, bs, ncy, nmr, link_fmt):
     h.unpack(pphi, out, oq.F32)
     assert rel_err(from_dev(out, rho.shape), ref) < 1e-5
     h.close()
+
+
+@pytest.mark.parametrize("dims,bs,ncy,nmr", [((4, 4, 6, 8), (1, 2, 3, 2), 2, 3),
+                                             ((4, 12, 4, 8), (2, 6, 2, 4), 2, 2),
+                                             ((8, 8, 8, 8), (4, 4, 4, 4), 1, 4)])
+@pytest.mark.parametrize("link_fmt", [0, 1])
+@pytest.mark.parametrize("eo", [0, 1])
+def test_block_ordered_operands(dims, bs, ncy, nmr, link_fmt, eo):
+    """The solver's SAP reads block-ordered links and clover.  One Krylov vector:
+    psi = phi <D phi, eta> / <D phi, D phi> with phi = SAP eta.  The binary32
+    errors of phi and D phi enter psi, the latter through the coefficient: the
+    bound of the single application above, doubled.  A second solve with another
+    right-hand side finds the same operands."""
+    import torch
+    from oracle import dirac
+    from paper_2202_07388_gb300 import oq
+    u, a, ainv = oracle_case(dims, 0.5, 935, 0.1365, 1.0)
+    h = make_handle(dims, u, 0.1365, 1.0, link_fmt)
+    for seed in (936, 937):
+        eta = synth.make_source(dims, seed)
+        phi = solvers.sap(u, a, eta, bs, ncy, nmr, eo=bool(eo), ainv=ainv)
+        chi = dirac.dw(u, a, phi, -1.0)
+        ref = phi * (np.vdot(chi, eta) / np.vdot(chi, chi))
+        psi = to_dev(np.zeros_like(eta))
+        h.sap_gcr(to_dev(eta), psi, oq.SolverParams(nkv=1, nmx=1, res=1e-12, ncy=ncy, nmr=nmr, bs=bs, sap_eo=eo,
+                                                    sdtype=oq.F32))
+        assert rel_err(from_dev(psi, eta.shape), ref) < 2e-5
+    h.close()
