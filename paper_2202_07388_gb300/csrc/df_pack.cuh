@@ -62,7 +62,9 @@ __device__ __forceinline__ D2 dfma(D2 a, D2 b, D2 c) {
   return fast_two_sum(s.hi, add(s.lo, add(c.lo, e)));
 }
 
-// lazy dot product (DfAcc) with a factor shared by the two lanes
+// A dot product accumulated lazily: s is the running sum of the high products (each
+// added by a two-sum), e collects the two-sum errors and the low parts; one
+// renormalisation at the end.  One factor is shared by the two lanes.
 struct Acc {
   F2 s, e;
 };

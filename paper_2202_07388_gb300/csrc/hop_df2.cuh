@@ -34,7 +34,7 @@ __device__ __forceinline__ void st(float4* b0, float4* b1, bool l0, bool l1, lon
   if (l1) b1[k * Vh + i] = make_float4(z.re.hi.y, z.re.lo.y, z.im.hi.y, z.im.lo.y);
 }
 
-// y = K x for clover block b of site i (parity p): clover_apply<dfloat>'s
+// y = K x for clover block b of site i (parity p):
 // row-by-row lazy dot products, the block's reals loaded once for both lanes
 __device__ __forceinline__ void clover_block(const void* base, long Vh, int p, long i, int b, const C2 (&x)[6],
                                              C2 (&y)[6]) {

@@ -509,12 +509,15 @@ static cudaError_t launch_one(const HopLaunch& L, const HopArgs& a, cudaStream_t
   const unsigned ntile = (unsigned)((a.nrhs + L.by - 1) / L.by);
   dim3 grid((MODE == HOP_DW ? 2u * nb : nb) * ntile, 1u, 1u);
   size_t smem = (EPI == EPI_NONE) ? 0 : sizeof(double) * (L.bx / 32) * L.by;
-  if (L.sys) {
-    dim3 bblock(L.bx, 1, 1);
-    if (P == P_DF64 && L.bx > 64) return cudaErrorInvalidValue;
-    hop_batch_kernel<P, FMT, MODE, DAG, EPI>
-        <<<L.ntiles, bblock, (EPI == EPI_NONE) ? 0 : sizeof(double) * (L.bx / 32), s>>>(L.sys, L.tiles);
-    return cudaGetLastError();
+  if (L.sys) {  // the binary32-arithmetic types run batches in hop_pair_batch_kernel
+    if constexpr (P == P_F64 || P == P_DF64) {
+      dim3 bblock(L.bx, 1, 1);
+      if (P == P_DF64 && L.bx > 64) return cudaErrorInvalidValue;
+      hop_batch_kernel<P, FMT, MODE, DAG, EPI>
+          <<<L.ntiles, bblock, (EPI == EPI_NONE) ? 0 : sizeof(double) * (L.bx / 32), s>>>(L.sys, L.tiles);
+      return cudaGetLastError();
+    }
+    return cudaErrorInvalidValue;
   }
   if constexpr (P == P_DF64) {
     if (L.regcap) {
