@@ -638,7 +638,7 @@ __device__ __forceinline__ void zero_spinor(Spinor<float>& v) {
 // is held as six complex pairs, lanes spin s and s + 2; links as pairs of directions
 // (0, 1) and (2, 3); a site's two clover blocks as one block of pairs.  A packed FMA
 // takes the pipe twice as long as a scalar one, so what it saves is issue: the
-// even-odd kernel, one warp per scheduler in each half pass, gains (93 to 77 us a
+// even-odd kernel, one warp per scheduler in each half pass, gained (93 to 77 us a
 // colour on 24x16^3); sap_block_kernel, two warps and 23 % fewer instructions, takes
 // 252 us instead of 239, waiting for the longer latency, and stays scalar.
 namespace eop {
