@@ -290,13 +290,13 @@ __global__ void __launch_bounds__(256, MINB) sap_kernel(const SapArgs a) {
 //
 // The block residual rho - D phi takes the in-block part of D phi through the
 // same shared-memory operator and reads only the neighbours outside the block
-// from global memory.  In the first cycle (FIRST) phi is zero on the blocks of
+// from global memory.  In the first cycle phi is zero on the blocks of
 // this colour (and, with colour 0, everywhere), so those terms are left out.
 // BLK: own links and clover from the block-ordered copies (sap_blocked_kernel).
 // Bound by latency at one block of 8 warps per SM (255 registers, 147 KB): an MR
 // step runs two thirds of the issue slots (20 us of a launch, 48x24^3 in 4^4
 // blocks), loading a block and the hops from outside it overlap with nothing.
-// 5 MR steps there: 204 us a launch; 338 us with links and residual in shared
+// 5 MR steps there: 201 us a launch; 338 us with links and residual in shared
 // memory and the operands in packed order.  Two threads per site (512 at 128
 // registers) took 287 against 228 us, both directions' outside operands
 // requested together 243, and an L2 prefetch of the next block 210 against 204.

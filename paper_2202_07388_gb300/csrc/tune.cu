@@ -51,6 +51,14 @@ cudaError_t tune_fill(void* p, size_t bytes, int prec, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// The launch of 64 x 1 threads, one right-hand side each, no cap, is two threads
+// per site for the binary32-arithmetic types (hop_pair.cuh), so that a launch that
+// oq_tune_get reported comes back from oq_tune_set.
+bool pair_shape(const LatCtx& L, int prec, const TuneVal& v) {
+  return (prec == P_F32 || prec == P_BF16 || prec == P_F16) && !L.halo_t && v.bx == 64 && v.by == 1 && v.nr == 1 &&
+         v.regcap == 0;
+}
+
 std::vector<TuneVal> candidates(int prec, int nrhs) {
   std::vector<TuneVal> c;
   const int bxs[] = {32, 64, 128, 256};
@@ -64,13 +72,6 @@ std::vector<TuneVal> candidates(int prec, int nrhs) {
       v.by = by;
       c.push_back(v);
     }
-  // two threads per site (binary32 arithmetic types)
-  if (prec == P_F32 || prec == P_BF16 || prec == P_F16) {
-    TuneVal v;
-    v.bx = 64;
-    v.pair = true;
-    c.push_back(v);
-  }
   // double-float: the register-capped kernel (<= 128 threads per CTA)
   if (prec == P_DF64) {
     const size_t n0 = c.size();
@@ -243,7 +244,7 @@ extern "C" int oq_autotune(oq_handle h, int lat, int prec, int nrhs, void* strea
         l.by = c.by;
         l.nr = c.nr;
         l.regcap = c.regcap;
-        l.pair = c.pair;
+        l.pair = c.pair = pair_shape(L, prec, c);
         l.link_fmt = fmt;
         const HopArgs b = h->with_links(l, a);
         for (int w = 0; w < 2; ++w)
@@ -311,6 +312,7 @@ extern "C" int oq_tune_set(oq_handle h, int lat, int prec, int mode, int nrhs, i
   v.regcap = regcap;
   v.link_fmt = link_fmt;
   v.ms = 0.f;
+  v.pair = pair_shape(L, prec, v);
   if (!valid_shape(L, prec, nrhs, v)) return OQ_ERR_ARG;
   // the pinned launch serves every epilogue of the mode
   const int epis[] = {EPI_NORM, EPI_CG, EPI_RESID64};

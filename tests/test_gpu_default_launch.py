@@ -30,7 +30,7 @@ def test_default_against_pinned(dims, nrhs, prec, link_fmt):
     for pinned in (False, True):
         for mode in (0, 1, 2):
             if pinned:
-                h.tune_set(prec, mode, nrhs, 64, 1, nr=1)
+                h.tune_set(prec, mode, nrhs, 128, 1, nr=1)
         h.dw(a, c if pinned else b, prec, nrhs=nrhs, dagger=True)
         psi = torch.zeros_like(eta)
         rc, st = h.cgne_even(eta, psi, prm, nrhs=nrhs)
@@ -41,4 +41,26 @@ def test_default_against_pinned(dims, nrhs, prec, link_fmt):
     assert d < 16 * 2.0 ** -24 + (eps if prec != 1 else 0.0)
     # two solutions of residual 1e-9, condition number of Dhat^dag Dhat below 1e3
     assert (sol[0] - sol[1]).norm() / sol[1].norm() < 2e-6
+    h.close()
+
+
+@pytest.mark.parametrize("prec", [1, 2, 3])
+def test_reported_launch_comes_back(prec):
+    """oq_tune_set with what oq_tune_get reported gives the tuner's launch: the same bits."""
+    import torch
+    from paper_2202_07388_gb300 import oq, synth
+    from tests.gpu_cases import to_dev
+    dims = (4, 6, 10, 6)
+    h = oq.Handle(dims)
+    h.gauge_upload(to_dev(synth.make_gauge(dims, 0.5, 943)), 1)
+    h.clover_build(0.13, 1.0)
+    x = torch.randn(1, 4 * 6 * 10 * 6, 24, dtype=torch.float64, device="cuda")
+    a, b, c = (h.new_packed(prec) for _ in range(3))
+    h.pack(x, a, prec)
+    h.autotune(prec, 1)
+    h.dw(a, b, prec)
+    bx, by, _, fmt, nr, cap = h.tune_get(prec, 0, 1)
+    h.tune_set(prec, 0, 1, bx, by, nr=nr, regcap=cap, link_fmt=oq.LINK_12 if fmt == "12-real" else oq.LINK_18)
+    h.dw(a, c, prec)
+    assert torch.equal(b, c)
     h.close()
