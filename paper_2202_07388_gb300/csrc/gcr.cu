@@ -200,7 +200,18 @@ __global__ void __launch_bounds__(VB) vec_convert_kernel(char* out, const char* 
   store_spinor<PO>((char*)fsite(out, Vh, hbo, j, &i), Vh, i, w);
 }
 
-// psi (F64) += sum_l beta_l Phi_l (F32)
+// binary32 to binary64 by integer operations (exact; the conversion instruction
+// runs on the binary64 pipe), values that are not normal by the instruction
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), m = b & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+  return (double)x;
+}
+
+// psi (F64) += sum_l beta_l Phi_l (F32).  Bound by the binary64 pipe: 48 FMAs per
+// site and vector (16 vectors on 48x24^3: 848 us; 1111 us with 24 conversions and
+// the products added by separate operations, 96 in all).
 __global__ void __launch_bounds__(VB) vec_psi_update_kernel(char* psi, const char* Phi, long pstride,
                                                             const double2* beta, int nl, long Vh, long hb64,
                                                             long hb32) {
@@ -217,7 +228,12 @@ __global__ void __launch_bounds__(VB) vec_psi_update_kernel(char* psi, const cha
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
-      for (int a = 0; a < 3; ++a) v.c[s][a] = v.c[s][a] + c * cx<double>{(double)w.c[s][a].re, (double)w.c[s][a].im};
+      for (int a = 0; a < 3; ++a) {
+        const double re = widen(w.c[s][a].re), im = widen(w.c[s][a].im);
+        cx<double>& z = v.c[s][a];
+        z.re = fma(c.re, re, fma(-c.im, im, z.re));
+        z.im = fma(c.re, im, fma(c.im, re, z.im));
+      }
   }
   store_spinor<P_F64>(pb, Vh, i, v);
 }
