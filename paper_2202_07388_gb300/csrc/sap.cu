@@ -883,7 +883,7 @@ __device__ __forceinline__ void mr_update(cx<float> om, const Sp6& p, Sp6& x, Sp
 // even residual and publish it, the even threads form D_eo of that.  Latency
 // and issue of one warp per scheduler bound it: a half pass keeps 4 of an SM's
 // 8 warps busy, and one block fills an SM (255 registers).  (A colour of 24x16^3
-// in 4^4 blocks, 4 MR steps: 64 us; with links and clover in shared memory and
+// in 4^4 blocks, 4 MR steps: 77 us; with links and clover in shared memory and
 // both hops of a link multiplied by their reader it took 128 us.)
 // ---------------------------------------------------------------------------
 // The block's sites are held parity-sorted: position k < nsite/2 is the
@@ -951,12 +951,15 @@ __global__ void __launch_bounds__(256, 1) sap_block_eo_kernel(const SapArgs a) {
   }
   const int w = t >> 5, nw = (blockDim.x + 31) >> 5;
 
-  // r: the residual (odd sites), rhat (even sites); xs: the solution (even sites),
-  // what is published (odd sites)
-  eop::Sp6 r, xs;
+  eop::Sp6 r, xs;  // r: the residual (odd sites), rhat (even sites)
   eop::sp6_zero(r);
   eop::sp6_zero(xs);
   eop::Link2 u[2];
+  // acc += the in-block hops of the published field
+  auto dhop = [&](Spinor<float>& acc) {
+    eop::sm4_hops<0>(m, tu, td, up, down, u[0], acc);
+    eop::sm4_hops<1>(m, tu, td, up, down, u[1], acc);
+  };
   char* phi = a.phi + (long)p * a.half_bytes;
   Spinor<float> acc;
   zero_spinor(acc);
@@ -983,101 +986,107 @@ __global__ void __launch_bounds__(256, 1) sap_block_eo_kernel(const SapArgs a) {
       load_spinor<P_F32>(phi, a.g.Vh, i, v);
       xs = eop::pack6(v);
     }
-    if (a.first) {
+    if (!a.first) {
+      eop::sm4_publish(m, t, u, xs);
+    } else {
       // a dropped hop reads its own position with weight zero: that must hold numbers
       const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int k = 0; k < 6; ++k) m.r[k * nsite + t] = z;
 #pragma unroll
       for (int k = 0; k < 12; ++k) m.s[k * nsite + t] = z;
-    } else {
+    }
+    if (!a.first) {
+      v = eop::spinor_of(xs);
       Spinor<float> aph;
       clover_apply<float>(a.clov, a.g.Vh, p, i, v, aph);
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) acc.c[s][c] = acc.c[s][c] + aph.c[s][c];
+      eop::sp6_sub(r, eop::pack6(aph));
+      eop::sp6_zero(xs);
     }
     cp_async_wait();
     eop::sm4_clover_pairs(m.a, nsite, t);  // read by this thread alone
   }
-  // The half passes, in one copy of the code (its length costs more than the
-  // selections: 77 to 64 us): publish, hops of the published field, clover.
-  //  -1:       phi published by all (not in the first cycle); r -= D phi; odd: A^{-1} r
-  //   0:       odd publish A^{-1} r_o; even: rhat = r_e - D_eo A^{-1} r_o
-  //   2k - 1:  even publish rhat; odd: A^{-1} D_oe rhat
-  //   2k:      odd publish that; even: q = A rhat - D_eo of it, the MR step
-  //   last:    even publish delta_e; odd: delta_o = A^{-1} (r_o - D_oe delta_e)
-  // A parity's published field is next written two half passes after it is read,
-  // so one barrier a half pass is enough but for -1, where both parities read.
+  if (!a.first) {
+    __syncthreads();  // the published phi
+    if (act) dhop(acc);
+    __syncthreads();  // every read of it is done
+  }
+  eop::sp6_sub(r, eop::pack6(acc));
+  // odd sites publish A^{-1} r_o; even sites: rhat_e = r_e - D_eo A^{-1} r_o
+  if (od) {
+    eop::Sp6 v;
+    eop::sm4_clover(m.a, nsite, t, r, v);
+    eop::sm4_publish(m, t, u, v);
+  }
+  __syncthreads();
+  if (ev) {
+    zero_spinor(acc);
+    dhop(acc);
+    eop::sp6_sub(r, eop::pack6(acc));
+    eop::sm4_publish(m, t, u, r);  // at even positions, which no one reads in this phase
+  }
   double rn_prev = 0.0;
+  if (a.adaptive) rn_prev = sqrt(block_sum1(ev ? eop::norm2_of(r) : 0.0, reinterpret_cast<double*>(red)));
+  __syncthreads();
+
   int steps = 0;
-  const int last = 2 * a.nmr + 1;
-  for (int j = -1;;) {
-    const bool odd_pub = !(j & 1), both = j < 0 && !a.first;
-    if (both ? act : j < 0 ? false : odd_pub ? od : ev) {
+  for (int k = 1; k <= a.nmr; ++k) {
+    // odd half pass: t_o = A^{-1} D_oe rhat_e
+    if (od) {
+      zero_spinor(acc);
+      dhop(acc);
       eop::Sp6 v;
-      const bool sol = od || j < 0 || j == last;
-#pragma unroll
-      for (int k = 0; k < 6; ++k) v.c[k] = sol ? xs.c[k] : r.c[k];
+      eop::sm4_clover(m.a, nsite, t, eop::pack6(acc), v);
       eop::sm4_publish(m, t, u, v);
     }
     __syncthreads();
-    if (j >= 0) zero_spinor(acc);  // before: the hops from outside the block
-    const bool recv = both ? act : j < 0 ? false : odd_pub ? ev : od;
-    if (recv) {
-      eop::sm4_hops<0>(m, tu, td, up, down, u[0], acc);
-      eop::sm4_hops<1>(m, tu, td, up, down, u[1], acc);
-    }
-    if (both) __syncthreads();  // every read of phi is done
-    eop::Sp6 y = eop::pack6(acc);
-    if (j < 0 || (recv && (j == 0 || j == last))) eop::sp6_sub(r, y);
-    if (j < 0) eop::sp6_zero(xs);
-    const bool step = odd_pub && j > 0;
+    // even half pass: q_e = A rhat_e - D_eo t_o, then <q, rhat>, <q, q>
     eop::Sp6 pv;
-    if (step ? ev : (j & 1) ? od : false) {
-#pragma unroll
-      for (int k = 0; k < 6; ++k) pv.c[k] = (j < 0 || j == last || step) ? r.c[k] : y.c[k];
-      eop::Sp6 o;
-      eop::sm4_clover(m.a, nsite, t, pv, o);
-      if (od) xs = o;
-      else pv = o;
+    float d0 = 0.f, d1 = 0.f, d2 = 0.f;
+    if (ev) {
+      eop::sm4_clover(m.a, nsite, t, r, pv);
+      zero_spinor(acc);
+      dhop(acc);
+      eop::sp6_sub(pv, eop::pack6(acc));
+      eop::mr_dots(pv, r, d0, d1, d2);
     }
-    if (j == last) break;
-    bool done = false;
-    if (step) {
-      float d0 = 0.f, d1 = 0.f, d2 = 0.f;
-      if (ev) {
-        eop::sp6_sub(pv, y);
-        eop::mr_dots(pv, r, d0, d1, d2);
-      }
-      d0 = warp_sum_f(d0);
-      d1 = warp_sum_f(d1);
-      d2 = warp_sum_f(d2);
-      if ((t & 31) == 0) {
-        red[3 * w] = d0;
-        red[3 * w + 1] = d1;
-        red[3 * w + 2] = d2;
-      }
-      __syncthreads();  // the partial sums
-      d0 = d1 = d2 = 0.f;
-      for (int q = 0; q < nw; ++q) {
-        d0 += red[3 * q];
-        d1 += red[3 * q + 1];
-        d2 += red[3 * q + 2];
-      }
-      cx<float> om{0.f, 0.f};
-      if (d2 > 0.f) om = cx<float>{d0 / d2, d1 / d2};
-      if (ev) eop::mr_update(om, pv, xs, r);
-      steps = j >> 1;
+    d0 = warp_sum_f(d0);
+    d1 = warp_sum_f(d1);
+    d2 = warp_sum_f(d2);
+    if ((t & 31) == 0) {
+      red[3 * w] = d0;
+      red[3 * w + 1] = d1;
+      red[3 * w + 2] = d2;
     }
-    if (a.adaptive && j >= 0 && odd_pub) {
+    __syncthreads();  // the partial sums
+    d0 = d1 = d2 = 0.f;
+    for (int j = 0; j < nw; ++j) {
+      d0 += red[3 * j];
+      d1 += red[3 * j + 1];
+      d2 += red[3 * j + 2];
+    }
+    cx<float> om{0.f, 0.f};
+    if (d2 > 0.f) om = cx<float>{d0 / d2, d1 / d2};
+    if (ev) {
+      eop::mr_update(om, pv, xs, r);
+      eop::sm4_publish(m, t, u, r);
+    }
+    steps = k;
+    if (a.adaptive) {
       const double rn_new = sqrt(block_sum1(ev ? eop::norm2_of(r) : 0.0, reinterpret_cast<double*>(red)));
-      done = step && ((steps >= 4 && rn_new > (double)a.alpha * rn_prev) || rn_new > rn_prev || rn_new < a.tol);
+      if ((k >= 4 && rn_new > (double)a.alpha * rn_prev) || rn_new > rn_prev || rn_new < a.tol) break;
       rn_prev = rn_new;
-      __syncthreads();  // the sums are read
     }
-    j = done ? last : j + 1;
+    __syncthreads();  // the odd half pass of the next step reads the even residual
+  }
+  // delta_e = x_e published; delta_o = A^{-1} (r_o - D_oe delta_e)
+  if (ev) eop::sm4_publish(m, t, u, xs);
+  __syncthreads();
+  if (od) {
+    zero_spinor(acc);
+    dhop(acc);
+    eop::sp6_sub(r, eop::pack6(acc));
+    eop::sm4_clover(m.a, nsite, t, r, xs);
   }
   if (act) {
     Spinor<float> v = eop::spinor_of(xs);
