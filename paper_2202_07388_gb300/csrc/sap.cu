@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(256, MINB) sap_kernel(const SapArgs a) {
 // Bound by latency at one block of 8 warps per SM (255 registers, 147 KB): an MR
 // step runs two thirds of the issue slots (20 us of a launch, 48x24^3 in 4^4
 // blocks), loading a block and the hops from outside it overlap with nothing.
-// 5 MR steps there: 201 us a launch; 338 us with links and residual in shared
+// 5 MR steps there: 204 us a launch; 338 us with links and residual in shared
 // memory and the operands in packed order.  Two threads per site (512 at 128
 // registers) took 287 against 228 us, both directions' outside operands
 // requested together 243, and an L2 prefetch of the next block 210 against 204.
@@ -536,39 +536,40 @@ __global__ void __launch_bounds__(256, 1) sap_block_kernel(const SapArgs a) {
     for (int s = 0; s < 4; ++s)
 #pragma unroll
       for (int c = 0; c < 3; ++c) r.c[s][c] = rh.c[s][c] - r.c[s][c];
-    if (!a.first) {  // r: the block's phi, xs: what the part of D phi inside the block is taken from
-      xs = r;
-      load_spinor<P_F32>(phi, a.g.Vh, i, r);
+    if (!a.first) {
+      load_spinor<P_F32>(phi, a.g.Vh, i, xs);  // the block's phi
+      sm4_publish(m, t, u, xs);
     }
-    cp_async_wait();  // the staged clover: each thread reads its own
+    cp_async_wait();
   }
-  double rn_prev = 0.0;
-  if (a.adaptive && a.first) rn_prev = sqrt(block_sum1(act ? site_norm2(r) : 0.0, reinterpret_cast<double*>(red)));
-
-  // 2. MR on D_i; step 0 applies D_i to phi (one copy of that code: the kernel's
-  // straight-line code is longer than the instruction caches near the SM)
-  int steps = 0;
-  for (int k = a.first ? 1 : 0; k <= a.nmr; ++k) {
-    if (act) sm4_publish(m, t, u, r);
-    __syncthreads();
-    Spinor<float> pv = r;
-    float d0 = 0.f, d1 = 0.f, d2 = 0.f;  // <p, r>, <p, p>
+  __syncthreads();  // the staged clover (each site reads its own) and the published phi
+  if (!a.first) {
+    // the part of D phi inside the block
     if (act) {
-      sm4_apply(m, t, stride, up, down, u, r, pv);
-    }
-    if (k == 0) {
+      Spinor<float> pv;
+      sm4_apply(m, t, stride, up, down, u, xs, pv);
 #pragma unroll
       for (int s = 0; s < 4; ++s)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          r.c[s][c] = xs.c[s][c] - pv.c[s][c];
+          r.c[s][c] = r.c[s][c] - pv.c[s][c];
           xs.c[s][c] = cx<float>{0.f, 0.f};
         }
-      if (a.adaptive) rn_prev = sqrt(block_sum1(act ? site_norm2(r) : 0.0, reinterpret_cast<double*>(red)));
-      __syncthreads();  // every read of the published phi is done
-      continue;
     }
+    __syncthreads();  // every read of the published phi is done
+  }
+  double rn_prev = 0.0;
+  if (a.adaptive) rn_prev = sqrt(block_sum1(act ? site_norm2(r) : 0.0, reinterpret_cast<double*>(red)));
+
+  // 2. MR on D_i
+  int steps = 0;
+  for (int k = 1; k <= a.nmr; ++k) {
+    if (act) sm4_publish(m, t, u, r);
+    __syncthreads();
+    Spinor<float> pv;
+    float d0 = 0.f, d1 = 0.f, d2 = 0.f;  // <p, r>, <p, p>
     if (act) {
+      sm4_apply(m, t, stride, up, down, u, r, pv);
 #pragma unroll
       for (int s = 0; s < 4; ++s)
 #pragma unroll
