@@ -88,3 +88,25 @@ def test_block_ordered_operands(dims, bs, ncy, nmr, link_fmt, eo):
                                                     sdtype=oq.F32))
         assert rel_err(from_dev(psi, eta.shape), ref) < 2e-5
     h.close()
+
+
+def test_solution_update_from_zero_components():
+    """A point source: phi is exactly zero away from it, and the update of the
+    binary64 solution must leave those components zero."""
+    from oracle import dirac
+    from paper_2202_07388_gb300 import oq
+    dims, bs = (8, 8, 8, 8), (4, 4, 4, 4)
+    u, a, ainv = oracle_case(dims, 0.5, 938, 0.1365, 1.0)
+    h = make_handle(dims, u, 0.1365, 1.0, 1)
+    eta = np.zeros_like(synth.make_source(dims, 939))
+    eta[0, 0, 0, 0, 0, 0] = 1.0
+    phi = solvers.sap(u, a, eta, bs, 1, 1)
+    chi = dirac.dw(u, a, phi, -1.0)
+    ref = phi * (np.vdot(chi, eta) / np.vdot(chi, chi))
+    psi = to_dev(np.zeros_like(eta))
+    h.sap_gcr(to_dev(eta), psi, oq.SolverParams(nkv=1, nmx=1, res=1e-12, ncy=1, nmr=1, bs=bs, sdtype=oq.F32))
+    got = from_dev(psi, eta.shape)
+    far = ref == 0
+    assert far.sum() > ref.size // 2 and not got[far].any()
+    assert rel_err(got, ref) < 2e-5  # as test_block_ordered_operands
+    h.close()
