@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(VT) vec_batch_kernel(const VecSys* __restrict_
     if constexpr (OP == VOP_RESTART || OP == VOP_RESTART_DF) {
       const unsigned nblk = (unsigned)((v.Vh + VT - 1) / VT);
       grid_reduce(acc, v.red, 0, 1, smem, (unsigned)tl.y, nblk);
+      __syncthreads();  // the first warp has read this tile's sums before another warp writes the next tile's
     }
   }
 }

@@ -78,3 +78,43 @@ def test_batch_rejects_mixed_link_formats():
     rc, _ = h.cgne_batch([0, 1], [eta, eta], psi, oq.SolverParams(sdtype=1), check=False)
     assert rc == oq.ERR_ARG
     h.close()
+
+
+@pytest.mark.parametrize("prec", [1, 3])
+def test_more_tiles_than_ctas(prec):
+    """Two systems of 864 vector tiles each: the restart's CTAs (8 per SM) take
+    more than one tile, and its norms still start every inner solve: the batch
+    follows the single solves and repeats bit for bit."""
+    import torch
+    from paper_2202_07388_gb300 import oq
+    dims = (32, 24, 24, 24)
+    vol = 32 * 24 ** 3
+    h = oq.Handle([dims, dims])
+    u = torch.zeros(vol, 4, 3, 3, dtype=torch.complex128, device="cuda")
+    u[...] = torch.eye(3, dtype=torch.complex128, device="cuda")
+    for lat in (0, 1):
+        h.gauge_upload(torch.view_as_real(u).contiguous(), oq.LINK_18, lat=lat)
+        h.clover_build(0.10, 1.0, lat=lat)
+    g = torch.Generator(device="cuda").manual_seed(480)
+    etas = []
+    for _ in range(2):
+        e = torch.randn(vol, 24, dtype=torch.float64, device="cuda", generator=g)
+        x = torch.arange(vol, device="cuda")
+        odd = (x + x // 24 + x // 24 ** 2 + x // 24 ** 3) % 2 == 1
+        e[odd] = 0.0
+        etas.append(e)
+    prm = oq.SolverParams(res=1e-10, nmx=400, sdtype=prec)
+    out = []
+    for _ in range(2):
+        psis = [torch.zeros_like(e) for e in etas]
+        rc, st = h.cgne_batch([0, 1], etas, psis, prm)
+        assert rc == oq.OK and all(s["converged"] for s in st)
+        out.append((psis, st))
+    for k in range(2):
+        assert torch.equal(out[0][0][k], out[1][0][k])
+        psi = torch.zeros_like(etas[k])
+        rc, st1 = h.cgne(etas[k], psi, prm, lat=k)
+        assert rc == oq.OK and abs(st1[0]["steps"] - out[0][1][k]["steps"]) <= 2
+        # two solutions of residual 1e-10; free field, A = 5: |Dhat - 5| <= 16 / 5, so cond(Dhat^dag Dhat) <= 21
+        assert (psi - out[0][0][k]).norm() <= 2e-8 * psi.norm()
+    h.close()
