@@ -111,8 +111,9 @@ size_t face_bytes(const LatCtx& L, int prec) {
 // read the same links)
 const void* links_of(const LatCtx& L, int prec) { return prec == P_F64 ? L.u64.p : L.u32.p; }
 
-// a stencil launch on a sub-domain: the tuned CTA shape with one rhs per
-// thread (the halo hops live in the one-rhs kernel) on the uploaded links
+// a stencil launch with faces (a sub-domain, or a whole lattice whose caller
+// passes them): the tuned CTA shape with one rhs and one site per thread (the
+// halo hops live in hop_kernel) on the uploaded links
 HopLaunch halo_launch(oq_handle h, int lat, int prec, int mode, int dagger, int nrhs) {
   HopLaunch l = h->hop_launch(lat, prec, mode, dagger, EPI_NONE, nrhs);
   if (l.nr != 1) {
@@ -120,6 +121,7 @@ HopLaunch halo_launch(oq_handle h, int lat, int prec, int mode, int dagger, int 
     if (l.bx * l.by > 256) l.by = 1;
   }
   l.regcap = 0;
+  l.pair = false;
   l.link_fmt = h->lats[lat].link_fmt;
   return l;
 }

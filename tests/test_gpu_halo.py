@@ -173,3 +173,43 @@ def test_sub_domain_refuses_whole_lattice_calls():
     assert lib().oq_gauge_upload_halo(w.h, 0, _ptr(to_dev(u)), oq.LINK_12, _stream()) == oq.ERR_STATE
     h.close()
     w.close()
+
+
+@pytest.mark.parametrize("tuned", [False, True])
+@pytest.mark.parametrize("prec", [0, 1, 2, 3])
+def test_faces_on_a_whole_lattice(prec, tuned):
+    """The calls that take faces on a lattice that is not split, its own faces
+    handed back to it: the lattice's operator, whatever launch the lattice has
+    by default or from the tuner."""
+    oq = _oq()
+    dims = (6, 4, 4, 6)
+    u, a, ainv = oracle_case(dims, 0.5, 7, KAPPA, CSW)
+    h = make_handle(dims, u, KAPPA, CSW, oq.LINK_12)
+    for nrhs in (1, 3):
+        if tuned:
+            h.autotune(prec, nrhs)
+        psi = synth.make_source(dims, 75, nrhs=nrhs)
+        x, y = h.new_packed(prec, nrhs=nrhs), h.new_packed(prec, nrhs=nrhs)
+        h.pack(to_dev(psi), x, prec, nrhs=nrhs)
+        fp, fn = h.new_faces(prec, nrhs, parities=2), h.new_faces(prec, nrhs, parities=2)
+        h.face_pack(x, fp, fn, prec, oq.FULL, nrhs=nrhs)
+        h.dw_halo(x, y, prec, oq.Handle.halo(fp, fn, -1.0, -1.0), nrhs=nrhs)
+        out = to_dev(np.zeros_like(psi))
+        h.unpack(y, out, prec, nrhs=nrhs)
+        got = from_dev(out, psi.shape)
+        for k in range(nrhs):
+            assert rel_err(got[k], dirac.dw(u, a, psi[k])) < TOL[prec]
+        ev = np.stack([dirac.even_part(p) for p in psi])
+        xe, to, ye = (h.new_packed(prec, oq.EVEN, nrhs=nrhs) for _ in range(3))
+        h.pack(to_dev(ev), xe, prec, oq.EVEN, nrhs=nrhs)
+        fp, fn = h.new_faces(prec, nrhs), h.new_faces(prec, nrhs)
+        h.face_pack(xe, fp, fn, prec, oq.EVEN, nrhs=nrhs)
+        h.dhat_pass(1, xe, None, to, prec, halo=oq.Handle.halo(fp, fn, -1.0, -1.0), nrhs=nrhs)
+        h.face_pack(to, fp, fn, prec, oq.ODD, nrhs=nrhs)
+        h.dhat_pass(2, to, xe, ye, prec, halo=oq.Handle.halo(fp, fn, -1.0, -1.0), nrhs=nrhs)
+        out = to_dev(np.zeros_like(ev))
+        h.unpack(ye, out, prec, oq.EVEN, nrhs=nrhs)
+        got = from_dev(out, ev.shape)
+        for k in range(nrhs):
+            assert rel_err(got[k], dirac.dw_hat(u, a, ainv, ev[k])) < TOL[prec]
+    h.close()
