@@ -271,8 +271,8 @@ int oq_dw_hat_apply_noalloc(oq_handle h, int lat, int prec, const void* in_dev, 
  * thread nr (1; or 2, 4 for F32/BF16/F16 storage with nrhs >= nr: the links,
  * clover blocks and indices of a site are loaded once for nr right-hand sides
  * and the arithmetic runs on packed pairs of them; bx*by <= 128), two threads
- * per site for the same types (bx = 64, by = 1, nr = 1, regcap 0; on time-split
- * sub-domains those numbers mean one thread per site), a register
+ * per site for the same types (bx = 64, by = 0, nr = 1, regcap 0; whole lattices
+ * only), a register
  * cap (regcap 0/1) of the nr > 1 kernels and of the OQ_DF64 kernel (bx*by <=
  * 128; regcap 1: at most 128 registers per thread, 2: at most 168), for the
  * nr > 1 kernels regcap 2: the cap of 1 with each hop's neighbour spinors and

@@ -79,7 +79,7 @@ struct TuneVal {
   int nr = 1;            // right-hand sides per thread
   int regcap = 0;        // register-capped multi-rhs variant
   int link_fmt = -1;     // binary32 link format (-1: the uploaded one)
-  bool pair = false;     // two threads per site (bx = 64, by = nr = 1; chosen by the tuner)
+  bool pair = false;     // two threads per site (bx = 64, by = nr = 1; reported and pinned as by = 0)
   float ms = 0.f;        // tuner's time per launch (0 if set by hand)
 };
 

@@ -1,8 +1,8 @@
 // Autotuner for the stencil launch shape: for one (lattice, precision,
 // number of right-hand sides) it times every admissible launch of the full
 // Dw and of both Dhat passes with CUDA events on scratch fields: CTA shapes
-// (bx sites x by rows, bx a multiple of 32), one or several (2, 4)
-// right-hand sides per thread with or without a register cap, and both
+// (bx sites x by rows, bx a multiple of 32), two threads per site, one or several
+// (2, 4) right-hand sides per thread with or without a register cap, and both
 // binary32 link formats when the handle holds both.  The fastest launch per
 // mode is kept in the handle and used by every later launch of that mode;
 // pass 2 is also timed with its norm and CG-update epilogues (on scratch
@@ -51,14 +51,6 @@ cudaError_t tune_fill(void* p, size_t bytes, int prec, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// The launch of 64 x 1 threads, one right-hand side each, no cap, is two threads
-// per site for the binary32-arithmetic types (hop_pair.cuh), so that a launch that
-// oq_tune_get reported comes back from oq_tune_set.
-bool pair_shape(const LatCtx& L, int prec, const TuneVal& v) {
-  return (prec == P_F32 || prec == P_BF16 || prec == P_F16) && !L.halo_t && v.bx == 64 && v.by == 1 && v.nr == 1 &&
-         v.regcap == 0;
-}
-
 std::vector<TuneVal> candidates(int prec, int nrhs) {
   std::vector<TuneVal> c;
   const int bxs[] = {32, 64, 128, 256};
@@ -98,8 +90,13 @@ std::vector<TuneVal> candidates(int prec, int nrhs) {
           c.push_back(v);
         }
   }
-  // several right-hand sides per thread (binary32 arithmetic types)
+  // two threads per site, then several right-hand sides per thread (binary32 arithmetic types)
   if (prec == P_F32 || prec == P_BF16 || prec == P_F16) {
+    TuneVal two;
+    two.bx = 64;
+    two.by = 1;
+    two.pair = true;
+    c.push_back(two);
     const int nrs[] = {2, 4};
     for (int nr : nrs) {
       if (nr > nrhs) continue;
@@ -121,7 +118,10 @@ std::vector<TuneVal> candidates(int prec, int nrhs) {
 
 bool valid_shape(const LatCtx& L, int prec, int nrhs, const TuneVal& v) {
   if (v.bx < 32 || v.bx % 32 != 0 || v.by < 1 || v.by > nrhs) return false;
-  if (v.nr == 1) {
+  if (v.pair) {
+    if ((prec != P_F32 && prec != P_BF16 && prec != P_F16) || L.halo_t) return false;
+    if (v.bx != 64 || v.by != 1 || v.nr != 1 || v.regcap != 0) return false;
+  } else if (v.nr == 1) {
     if (v.bx * v.by > 256) return false;
     if (v.regcap != 0 && !(prec == P_DF64 && (v.regcap == 1 || v.regcap == 2) && v.bx * v.by <= 128))
       return false;
@@ -244,7 +244,7 @@ extern "C" int oq_autotune(oq_handle h, int lat, int prec, int nrhs, void* strea
         l.by = c.by;
         l.nr = c.nr;
         l.regcap = c.regcap;
-        l.pair = c.pair = pair_shape(L, prec, c);
+        l.pair = c.pair;
         l.link_fmt = fmt;
         const HopArgs b = h->with_links(l, a);
         for (int w = 0; w < 2; ++w)
@@ -285,7 +285,7 @@ extern "C" int oq_tune_get_epi(oq_handle h, int lat, int prec, int mode, int epi
   if (it == h->tuned.end()) return OQ_ERR_STATE;
   const TuneVal& v = it->second;
   *bx = v.bx;
-  *by = v.by;
+  *by = v.pair ? 0 : v.by;
   *ms = v.ms;
   if (link_fmt) *link_fmt = v.link_fmt >= 0 ? v.link_fmt : h->lats[lat].link_fmt;
   if (nr) *nr = v.nr;
@@ -307,12 +307,12 @@ extern "C" int oq_tune_set(oq_handle h, int lat, int prec, int mode, int nrhs, i
   if (!L.has_gauge) return OQ_ERR_STATE;
   TuneVal v;
   v.bx = bx;
-  v.by = by;
+  v.pair = by == 0;  // two threads per site
+  v.by = v.pair ? 1 : by;
   v.nr = nr;
   v.regcap = regcap;
   v.link_fmt = link_fmt;
   v.ms = 0.f;
-  v.pair = pair_shape(L, prec, v);
   if (!valid_shape(L, prec, nrhs, v)) return OQ_ERR_ARG;
   // the pinned launch serves every epilogue of the mode
   const int epis[] = {EPI_NORM, EPI_CG, EPI_RESID64};

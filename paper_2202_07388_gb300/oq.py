@@ -456,7 +456,8 @@ class Handle:
     # tuning ------------------------------------------------------------
     def autotune(self, prec, nrhs=1, lat=0, stream=None):
         """Tune the stencil launches of (lat, prec, nrhs); returns per mode (0 Dw, 1 Dhat pass 1,
-        2 Dhat pass 2) the chosen (bx, by, ms, link format, rhs per thread, register cap)."""
+        2 Dhat pass 2) the chosen (bx, by, ms, link format, rhs per thread, register cap);
+        by 0: two threads per site."""
         _check(lib().oq_autotune(self.h, lat, prec, nrhs, _stream(stream)), "oq_autotune")
         return {mode: self.tune_get(prec, mode, nrhs, lat) for mode in (0, 1, 2)}
 
@@ -473,6 +474,7 @@ class Handle:
         return (bx.value, by.value, ms.value, "12-real" if fmt.value == LINK_12 else "18-real", nr.value, cap.value)
 
     def tune_set(self, prec, mode, nrhs, bx, by, nr=1, regcap=0, link_fmt=-1, lat=0, check=True):
+        """Pin a launch (bx = 64, by = 0: two threads per site, F32 / BF16 / F16)."""
         rc = lib().oq_tune_set(self.h, lat, prec, mode, nrhs, bx, by, nr, regcap, link_fmt)
         if check:
             _check(rc, "oq_tune_set")

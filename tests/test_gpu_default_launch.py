@@ -44,23 +44,91 @@ def test_default_against_pinned(dims, nrhs, prec, link_fmt):
     h.close()
 
 
-@pytest.mark.parametrize("prec", [1, 2, 3])
-def test_reported_launch_comes_back(prec):
-    """oq_tune_set with what oq_tune_get reported gives the tuner's launch: the same bits."""
+def _operator(prec, link_fmt, nrhs, dims, pins):
+    """Dw, Dhat and a short CGNE solve with `pins` (bx, by) for every mode, "tuned" or None
+    (the default launch)."""
     import torch
     from paper_2202_07388_gb300 import oq, synth
     from tests.gpu_cases import to_dev
-    dims = (4, 6, 10, 6)
     h = oq.Handle(dims)
-    h.gauge_upload(to_dev(synth.make_gauge(dims, 0.5, 943)), 1)
+    h.gauge_upload(to_dev(synth.make_gauge(dims, 0.5, 943)), link_fmt)
     h.clover_build(0.13, 1.0)
-    x = torch.randn(1, 4 * 6 * 10 * 6, 24, dtype=torch.float64, device="cuda")
-    a, b, c = (h.new_packed(prec) for _ in range(3))
-    h.pack(x, a, prec)
-    h.autotune(prec, 1)
-    h.dw(a, b, prec)
-    bx, by, _, fmt, nr, cap = h.tune_get(prec, 0, 1)
-    h.tune_set(prec, 0, 1, bx, by, nr=nr, regcap=cap, link_fmt=oq.LINK_12 if fmt == "12-real" else oq.LINK_18)
-    h.dw(a, c, prec)
-    assert torch.equal(b, c)
+    g = torch.Generator(device="cuda").manual_seed(944)
+    vol = dims[0] * dims[1] * dims[2] * dims[3]
+    x = torch.randn(nrhs, vol, 24, dtype=torch.float64, device="cuda", generator=g)
+    eta = torch.randn(nrhs, vol // 2, 24, dtype=torch.float64, device="cuda", generator=g)
+    a, b = h.new_packed(prec, nrhs=nrhs), h.new_packed(prec, nrhs=nrhs)
+    e, f = h.new_packed(prec, oq.EVEN, nrhs=nrhs), h.new_packed(prec, oq.EVEN, nrhs=nrhs)
+    h.pack(x, a, prec, nrhs=nrhs)
+    h.pack(x, e, prec, oq.EVEN, nrhs=nrhs)
+    if pins == "tuned":
+        h.autotune(prec, nrhs)
+    elif pins is not None:
+        for mode in (0, 1, 2):
+            h.tune_set(prec, mode, nrhs, *pins)
+            assert h.tune_get(prec, mode, nrhs)[:2] == pins
+    h.dw(a, b, prec, nrhs=nrhs)
+    h.dw_hat(e, f, prec, nrhs=nrhs)
+    psi = torch.zeros_like(eta)
+    rc, st = h.cgne_even(eta, psi, oq.SolverParams(res=1e-9, nmx=400, sdtype=prec), nrhs=nrhs)
+    assert rc == oq.OK and all(s["converged"] for s in st)
+    return h, (a, b, e, f, eta, psi)
+
+
+@pytest.mark.parametrize("prec", [1, 2, 3])
+@pytest.mark.parametrize("link_fmt", [0, 1])
+@pytest.mark.parametrize("nrhs", [1, 3])
+def test_one_and_two_threads_per_site_have_names(prec, link_fmt, nrhs):
+    """(64, 1) is one thread per site, the arithmetic of (128, 1) in other CTAs; (64, 0) is two
+    threads per site, the default for one right-hand side (its reductions in CTAs of the same
+    sites): the operators and a solve have the same bits."""
+    import torch
+    dims = (4, 6, 10, 6)
+    r = {k: _operator(prec, link_fmt, nrhs, dims, k) for k in ((64, 1), (128, 1), (64, 0), None)}
+    for k in (1, 3):   # Dw, Dhat
+        assert torch.equal(r[(64, 1)][1][k], r[(128, 1)][1][k])
+        if nrhs == 1:
+            assert torch.equal(r[(64, 0)][1][k], r[None][1][k])
+    if prec == 1:   # the hops are added in another order (a 16-bit type's rounding may hide it)
+        assert not torch.equal(r[(64, 0)][1][1], r[(64, 1)][1][1])
+    if nrhs == 1:
+        assert torch.equal(r[(64, 0)][1][5], r[None][1][5])
+    for h, _ in r.values():
+        h.close()
+
+
+@pytest.mark.parametrize("prec", [1, 2, 3])
+@pytest.mark.parametrize("nrhs", [1, 3])
+def test_reported_launch_comes_back(prec, nrhs):
+    """oq_tune_set with what oq_tune_get reported gives the tuner's launches: the same bits."""
+    import torch
+    from paper_2202_07388_gb300 import oq
+    h, (a, b, e, f, eta, psi) = _operator(prec, 1, nrhs, (4, 6, 10, 6), "tuned")
+    c, d = torch.empty_like(b), torch.empty_like(f)
+    for mode in (0, 1, 2):
+        bx, by, _, fmt, nr, cap = h.tune_get(prec, mode, nrhs)
+        h.tune_set(prec, mode, nrhs, bx, by, nr=nr, regcap=cap,
+                   link_fmt=oq.LINK_12 if fmt == "12-real" else oq.LINK_18)
+    h.dw(a, c, prec, nrhs=nrhs)
+    h.dw_hat(e, d, prec, nrhs=nrhs)
+    assert torch.equal(b, c) and torch.equal(f, d)
     h.close()
+
+
+def test_two_threads_per_site_refused_elsewhere():
+    from paper_2202_07388_gb300 import oq, synth
+    from tests.gpu_cases import to_dev
+    dims = (4, 6, 4, 6)
+    u = synth.make_gauge(dims, 0.5, 945)
+    h = oq.Handle(dims)
+    h.gauge_upload(to_dev(u), oq.LINK_12)
+    for kw in (dict(bx=128, by=0), dict(bx=64, by=0, nr=2), dict(bx=64, by=0, regcap=1), dict(bx=64, by=-1)):
+        assert h.tune_set(oq.F32, 0, 4, check=False, **kw) == oq.ERR_ARG, kw
+    for prec in (oq.F64, oq.DF64):
+        assert h.tune_set(prec, 0, 1, 64, 0, check=False) == oq.ERR_ARG
+    h.close()
+    s = oq.Handle((2,) + dims[1:], bc_t=oq.BC_HALO)
+    s.gauge_upload_halo(to_dev(u), oq.LINK_12)   # 2 slices and one beyond each face
+    assert s.tune_set(oq.F32, 0, 1, 64, 0, check=False) == oq.ERR_ARG
+    assert s.tune_set(oq.F32, 0, 1, 64, 1, check=False) == oq.OK
+    s.close()
