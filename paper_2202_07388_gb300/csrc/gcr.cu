@@ -64,6 +64,20 @@ __device__ __forceinline__ void site_dot(const Spinor<R>& a, const Spinor<R>& b,
   }
 }
 
+// ||v||^2 of one site by binary64 products
+template <typename R>
+__device__ __forceinline__ double site_norm2_64(const Spinor<R>& v) {
+  double acc = 0.0;
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double xr = (double)v.c[s][c].re, xi = (double)v.c[s][c].im;
+      acc = fma(xr, xr, fma(xi, xi, acc));
+    }
+  return acc;
+}
+
 // The dots <X_l, y> of NL consecutive fields per CTA row (blockIdx.y), y read
 // once for them: partials of rows 2 l, 2 l + 1 (re, im).  (One field per CTA
 // read y from L2 for each of them: 15 dots on 48x24^3 took 340 us, 304 now.)
@@ -97,8 +111,11 @@ __global__ void __launch_bounds__(VB) vec_dots_kernel(const char* X, long xstrid
   grid_reduce_nr<2 * NL>(v, ra, 2 * l0, 2 * nl, smem, blockIdx.x, gridDim.x, off);
 }
 
-// chi -= sum_l coef_l X_l ; partials of ||chi||^2 and Re, Im <chi, rho> (rows 0, 1, 2)
-template <int P>
+// chi -= sum_l coef_l X_l ; partials of ||chi||^2 and Re, Im <chi, rho> (rows 0, 1, 2).
+// FIRST: the first vector of a cycle (nl = 0), whose norm is summed from binary64
+// products; that of an orthogonalised one from binary32 sums per site (a kernel
+// of its own: the conversions would take a quarter of the other's warps).
+template <int P, bool FIRST>
 __global__ void __launch_bounds__(VB) vec_orth_kernel(char* chi, const char* X, long xstride,
                                                       const double2* coef, int nl, const char* rho, long Vh,
                                                       long hb, RedArgs ra) {
@@ -110,7 +127,7 @@ __global__ void __launch_bounds__(VB) vec_orth_kernel(char* chi, const char* X, 
     char* cb = (char*)fsite(chi, Vh, hb, j, &i);
     Spinor<R> v, r;
     load_spinor<P>(cb, Vh, i, v);
-    for (int l = 0; l < nl; ++l) {
+    for (int l = 0; !FIRST && l < nl; ++l) {
       Spinor<R> w;
       load_spinor<P>(fsite(X + l * xstride, Vh, hb, j, &i), Vh, i, w);
       const cx<R> c{(R)coef[l].x, (R)coef[l].y};
@@ -119,9 +136,9 @@ __global__ void __launch_bounds__(VB) vec_orth_kernel(char* chi, const char* X, 
 #pragma unroll
         for (int a = 0; a < 3; ++a) v.c[s][a] = v.c[s][a] - c * w.c[s][a];
     }
-    store_spinor<P>(cb, Vh, i, v);
+    if (!FIRST) store_spinor<P>(cb, Vh, i, v);
     load_spinor<P>(fsite(rho, Vh, hb, j, &i), Vh, i, r);  // after the loop: its registers would halve the warps
-    acc[0] += site_norm2(v);
+    acc[0] += FIRST ? site_norm2_64(v) : site_norm2(v);
     site_dot(v, r, acc[1], acc[2]);
   }
   const bool off[3] = {false, false, false};
@@ -482,8 +499,9 @@ static int gcr_impl(oq_handle h, int lat, const oq_solver_params* prm, const flo
           }
           CK(cudaMemcpyAsync(coef, coef_host, sizeof(double2) * k, cudaMemcpyHostToDevice, s));
         }
-        KL((vec_orth_kernel<P_F32><<<rgrid, rblock, 0, s>>>(chik, (const char*)Chi, f32, (const double2*)coef, k,
-                                                            (const char*)rho, Vh, hb32, rp),
+        auto* orth = k == 0 ? vec_orth_kernel<P_F32, true> : vec_orth_kernel<P_F32, false>;
+        KL((orth<<<rgrid, rblock, 0, s>>>((char*)chik, (const char*)Chi, f32, (const double2*)coef, k,
+                                          (const char*)rho, Vh, hb32, rp),
             cudaGetLastError()));
         KL(reduce_finish(rp, 3, grid, s));
         double t3[3];

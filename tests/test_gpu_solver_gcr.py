@@ -230,3 +230,31 @@ def test_sap_eo_needs_even_bs3():
     with pytest.raises(oq.OqError):
         h.sap_apply(prho, pphi, oq.SolverParams(ncy=1, nmr=2, bs=(2, 2, 2, 3), sap_eo=1))
     h.sap_apply(prho, pphi, oq.SolverParams(ncy=1, nmr=2, bs=(2, 2, 2, 3)))
+
+
+def test_first_krylov_norm_in_binary64():
+    """One GCR step without a preconditioner on a right-hand side of one 1 per
+    site: psi = (<D eta, eta> / ||D eta||^2) eta.  With one component per site
+    the dot is a sum of exact terms, so what is left is the norm of the first
+    Krylov vector: summed from binary64 products (2^-53 a term; binary32 sums
+    of 24 squares per site are off by 2e-9 of beta here)."""
+    oq = _oq()
+    dims = (4, 4, 4, 4)
+    u, a, ainv = oracle_case(dims, 0.5, 31, 0.1365, 1.0)
+    h = make_handle(dims, u, 0.1365, 1.0, oq.LINK_12)
+    eta = np.zeros(dims + (4, 3), complex)
+    eta[..., 1, 2] = 1.0
+    x, y = h.new_packed(oq.F32), h.new_packed(oq.F32)
+    h.pack(to_dev(eta), x, oq.F32)
+    h.dw(x, y, oq.F32)   # chi_0, with the solver's launch
+    chi = to_dev(np.zeros_like(eta))
+    h.unpack(y, chi, oq.F32)
+    chi = from_dev(chi, eta.shape)
+    beta = np.vdot(chi, eta) / np.vdot(chi, chi).real
+    psi = to_dev(np.zeros_like(eta))
+    rc, st = h.sap_gcr(to_dev(eta), psi, oq.SolverParams(res=1e-10, nmx=1, nkv=4, ncy=0, sdtype=oq.F32))
+    assert rc == oq.ERR_NOCONV and st[0]["steps"] == 1
+    got = from_dev(psi, eta.shape)
+    assert not np.any(got[..., 0, :]) and not np.any(got[..., 2:, :])
+    assert np.max(np.abs(got[..., 1, 2] - beta)) < 1e-13 * abs(beta)
+    h.close()
