@@ -509,8 +509,9 @@ __device__ __forceinline__ void su3_dag_mul(const Su3<R>& u, const HalfSpinor<R>
 // clover blocks
 // ---------------------------------------------------------------------------
 // Multiply the two Hermitian 6x6 blocks of site i (parity p) onto psi:
-// out = A psi.  Block b acts on spins 2b, 2b+1 (index 3*spin_local+colour).
-template <typename R>
+// out = A psi (ADD: out += A psi).  Block b acts on spins 2b, 2b+1 (index
+// 3*spin_local+colour).
+template <typename R, bool ADD = false>
 __device__ __forceinline__ void clover_apply(const void* base, long Vh, int p, long i,
                                              const Spinor<R>& in, Spinor<R>& out) {
   const cx<R>* v = &in.c[0][0];
@@ -552,7 +553,10 @@ __device__ __forceinline__ void clover_apply(const void* base, long Vh, int p, l
     const cx<R>* x = v + 6 * b;
     cx<R>* y = o + 6 * b;
 #pragma unroll
-    for (int r0 = 0; r0 < 6; ++r0) y[r0] = d[r0] * x[r0];
+    for (int r0 = 0; r0 < 6; ++r0) {
+      if constexpr (ADD) y[r0] = cx<R>{fma(d[r0], x[r0].re, y[r0].re), fma(d[r0], x[r0].im, y[r0].im)};
+      else y[r0] = d[r0] * x[r0];
+    }
     int k = 0;
 #pragma unroll
     for (int r0 = 0; r0 < 6; ++r0)
