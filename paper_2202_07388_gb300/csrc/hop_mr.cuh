@@ -403,10 +403,14 @@ __device__ __forceinline__ void blk_from(const float4 (&w)[9], Blk& k) {
   for (int c = 0; c < 15; ++c) k.off[c] = cx<float>{r[6 + 2 * c], r[7 + 2 * c]};
 }
 
-// y = K x for one block (x, y: the 6 components 3*spin_local + colour)
+// y = K x for one block (x, y: the 6 components 3*spin_local + colour); ADD: y += K x
+template <bool ADD = false>
 __device__ __forceinline__ void blk_apply(const Blk& k, const C2* x, C2* y) {
 #pragma unroll
-  for (int r = 0; r < 6; ++r) y[r] = {mul(bc(k.d[r]), x[r].re), mul(bc(k.d[r]), x[r].im)};
+  for (int r = 0; r < 6; ++r) {
+    if constexpr (ADD) y[r] = {ffma(bc(k.d[r]), x[r].re, y[r].re), ffma(bc(k.d[r]), x[r].im, y[r].im)};
+    else y[r] = {mul(bc(k.d[r]), x[r].re), mul(bc(k.d[r]), x[r].im)};
+  }
   int n = 0;
 #pragma unroll
   for (int r = 0; r < 6; ++r)
@@ -443,9 +447,8 @@ __device__ __forceinline__ void coords(const Geom& g, int p, uint32_t i, int x[4
 // clover blocks the same way after the last hop (stg: 2 stages of
 // NR * chunks + 3 slots).  Staged pass 2 and Dw first copy in2 (into
 // NR * chunks / 2 extra slots of each stage) and the two clover blocks (into
-// the stages' hop slots) and form A in2 from there before the hops, the
-// summation order of the unstaged kernel; hop 0's operands are copied once
-// block 0 has been read.
+// the stages' hop slots) and form A in2 from there before the hops; hop 0's
+// operands are copied once block 0 has been read.
 template <int P, int FMT, int MODE, bool DAG, int EPI, int NR, bool PF>
 __device__ __forceinline__ void site(const HopArgs& a, uint32_t i, int rhs0, int p, const bool (&live)[NR],
                                      float (&red)[NR], const Stage& stg) {
@@ -550,7 +553,10 @@ __device__ __forceinline__ void site(const HopArgs& a, uint32_t i, int rhs0, int
   // The weighted hops accumulate onto acc: for pass 2 and Dw onto A in2,
   // formed first while few registers are live (the site-local spinors stay
   // in their loaded chunks until their clover block is multiplied), for
-  // pass 1 onto zero, then multiplied by A^{-1}.
+  // pass 1 onto zero, then multiplied by A^{-1}.  LAST: pass 2 and Dw of the
+  // unstaged F32 kernels, whose stored result shows the order, sum the hops and
+  // add A in2 onto them (see below).
+  constexpr bool LAST = !PF && MODE != HOP_P1 && P == P_F32;
   const F2 w = bc(MODE == HOP_P2 ? 0.5f : -0.5f);
   Sp2 acc[NP];
   if constexpr (LOC) {
@@ -584,7 +590,7 @@ __device__ __forceinline__ void site(const HopArgs& a, uint32_t i, int rhs0, int
         for (int r = 0; r < 6; ++r) acc[q].c[2 * b + r / 3][r % 3] = yv[r];
       }
     }
-  } else if constexpr (MODE == HOP_P1) {
+  } else if constexpr (MODE == HOP_P1 || LAST) {
 #pragma unroll
     for (int q = 0; q < NP; ++q)
 #pragma unroll
@@ -617,6 +623,7 @@ __device__ __forceinline__ void site(const HopArgs& a, uint32_t i, int rhs0, int
     }
   }
   const F2 wf = mul(w, sf), wb = mul(w, sb);
+  Blk kb;  // LAST: clover block 0, requested before the last direction's hops
 
   auto hop = [&](auto mu_c) {
     constexpr int MU = decltype(mu_c)::value;
@@ -683,10 +690,39 @@ __device__ __forceinline__ void site(const HopArgs& a, uint32_t i, int rhs0, int
     hop(std::integral_constant<int, 0>{});
     hop(std::integral_constant<int, 1>{});
     hop(std::integral_constant<int, 2>{});
+    if constexpr (LAST) load_blk(a.clov, Vh, p, 0, i, kb);
     hop(std::integral_constant<int, 3>{});
   }
 
   Sp2 (&res)[NP] = acc;
+  if constexpr (LAST) {
+    // res = w H in + A in2, one clover block (spins 2b, 2b + 1) at a time, by
+    // FMAs onto the hops: hops added onto A in2, the larger of the two, round at
+    // its size every time (error of Dw with a diagonal A 7.8e-8; 4.5e-8 in this
+    // order, 5.1e-8 with A in2 summed apart, 8x6x4x10).  It costs the overlap of
+    // the clover with the first hops: 4 rhs on 32x16^3, Dw 56.6 against 51.6 us,
+    // Dhat 58.2 against 57.9 us; 12 rhs on 48x24^3, 739 against 686 and 688
+    // against 672 us (without block 0 ahead of the last hops 748 and 718 us).
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      if (b == 1) load_blk(a.clov, Vh, p, 1, i, kb);
+#pragma unroll
+      for (int q = 0; q < NP; ++q) {
+        const int r0 = rhs0 + 2 * q < a.nrhs ? rhs0 + 2 * q : a.nrhs - 1;
+        const int r1 = rhs0 + 2 * q + 1 < a.nrhs ? rhs0 + 2 * q + 1 : a.nrhs - 1;
+        const float4* l0 = reinterpret_cast<const float4*>((const char*)a.in2 + (long)r0 * a.in2_stride + par_out);
+        const float4* l1 = reinterpret_cast<const float4*>((const char*)a.in2 + (long)r1 * a.in2_stride + par_out);
+        C2 xv[6];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const float4 z0 = __ldg(l0 + ((3 * b + c) * Vh + i)), z1 = __ldg(l1 + ((3 * b + c) * Vh + i));
+          xv[2 * c] = {make_float2(z0.x, z1.x), make_float2(z0.y, z1.y)};
+          xv[2 * c + 1] = {make_float2(z0.z, z1.z), make_float2(z0.w, z1.w)};
+        }
+        blk_apply<true>(kb, xv, &res[q].c[2 * b][0]);
+      }
+    }
+  }
   if constexpr (MODE == HOP_P1 && PF) {
     // res = A^{-1} (w H in): block 0 was staged with the last hop, block 1
     // is staged while block 0 is applied

@@ -57,3 +57,16 @@ def test_binary64_rounds_once(dims, dagger):
         x, s, g = (getattr(v, part).reshape(-1) for v in (c, hop, got))
         for k in range(0, x.size, 3):
             assert g[k] == float(c0 * Fraction(x[k]) + Fraction(s[k])), k
+
+
+@pytest.mark.parametrize("nrhs,pin", [(2, (64, 1, 2, 1)), (3, (32, 1, 2, 0)), (4, (64, 1, 4, 1)), (12, None)])
+@pytest.mark.parametrize("dagger", [False, True])
+def test_binary32_several_rhs_round_once(nrhs, pin, dagger):
+    """binary32, several right-hand sides per thread (the launch without a pin on
+    this lattice): c0 x by an FMA onto the hops, one rounding."""
+    dims = (8, 8, 8, 16)
+    psi = _field(dims, nrhs)
+    c, got = _dw(dims, psi, 1, dagger, pin)
+    want = np.float32(1.0 / (2.0 * KAPPA)).astype(np.float64) * c + _hops(dims, psi, dagger)   # exact: 34 bits
+    assert np.array_equal(got.astype(np.complex64), want.astype(np.complex64))
+    assert np.array_equal(got, got.astype(np.complex64))
