@@ -271,13 +271,27 @@ struct oq_ctx {
   // Two threads per site by default (hop_pair.cuh; binary32-arithmetic types):
   // every launch with one right-hand side (F32 Dhat on 48x24^3: 105 against
   // 120 us with one thread per site, on 32x24x16x16 34 against 43 us, equal on
-  // 32x16^3); with several, the plain passes of up to 2^15 site-rhs (2 rhs F32
-  // on 16x16x12x12: 16 against 19 us; 4 rhs F16 on the same: 21 against 17 us)
-  // and those with a reduction below 2^18 (CG, 4 rhs F16 on 16^4: 29 against 32
-  // us with two rhs per thread; 12 rhs on 32x16^3: 122 against 98 us).
-  static bool pair_pays(int prec, int epi, long work, int nrhs) {
+  // 32x16^3); with several, while the launch is small enough for its latency to
+  // count, against two rhs per thread (work: site-rhs of one parity; Dw launches
+  // twice as many, which the limits of the 16-bit types count).  Measured from
+  // 8^4 to 32x16^3 with 2 to 12 rhs, us of Dw / Dhat, two threads a site against
+  // two rhs a thread:
+  //  - passes with a reduction below 2^18 (CG step, F32: 221,184 182 against 196,
+  //    262,144 214 against 210; F16: 147,456 141 against 160, 262,144 231 against 209);
+  //  - F32 below 2^17 (36,864: 8.2 / 9.5 against 10.0 / 15.8; 98,304: 21.6 / 23.3
+  //    against 26.4 / 23.3; 131,072: 31.3 / 33.3 against 33.5 / 30.9);
+  //  - 16-bit types on 18-real links below 2^17 launched (Dhat, 73,728: 15.2 against
+  //    16.5; 131,072: 24.9 against 24.3; Dw, 55,296: 10.7 against 10.5);
+  //  - on 12-real links, staged (below), up to 3 * 2^14 launched (24,576: 6.2 / 8.5
+  //    against 6.6 / 10.9; Dw, 36,864: 8.1 against 7.2; Dhat, 41,472: 12.2 against
+  //    12.9, 55,296: 14.3 against 13.1).
+  static bool pair_pays(int prec, int mode, int epi, long work, int nrhs, int link_fmt) {
     if (prec != oq::P_F32 && prec != oq::P_BF16 && prec != oq::P_F16) return false;
-    return nrhs == 1 || work <= (1L << 15) || (epi != oq::EPI_NONE && work < (1L << 18));
+    if (nrhs == 1) return true;
+    if (epi != oq::EPI_NONE) return work < (1L << 18);
+    if (prec == oq::P_F32) return work < (1L << 17);
+    const long launched = mode == oq::HOP_DW ? 2 * work : work;
+    return link_fmt == oq::LINK_12 ? launched <= (3L << 14) : launched < (1L << 17);
   }
 
   oq::HopLaunch hop_launch(int lat, int prec, int mode, int dagger, int epi, int nrhs) {
@@ -296,7 +310,7 @@ struct oq_ctx {
       l.regcap = it->second.regcap;
       l.pair = it->second.pair;
       if (it->second.link_fmt >= 0) l.link_fmt = it->second.link_fmt;
-    } else if (pair_pays(prec, epi, lats[lat].g.Vh * nrhs, nrhs) && !lats[lat].halo_t) {
+    } else if (pair_pays(prec, mode, epi, lats[lat].g.Vh * nrhs, nrhs, l.link_fmt) && !lats[lat].halo_t) {
       l.bx = 64;
       l.by = 1;
       l.pair = true;

@@ -97,6 +97,41 @@ def test_one_and_two_threads_per_site_have_names(prec, link_fmt, nrhs):
         h.close()
 
 
+@pytest.mark.parametrize("prec,link_fmt,nrhs,dw_pair,dhat_pair", [
+    (1, 1, 15, True, True), (1, 1, 16, False, False),       # F32: 2^17 site-rhs of a parity
+    (3, 1, 3, True, True), (3, 1, 4, False, True),          # 16 bits, 12-real: 3 * 2^14 launched
+    (2, 1, 6, False, True), (2, 1, 7, False, False),
+    (3, 0, 7, True, True), (2, 0, 8, False, True),          # 18-real: 2^17 launched
+    (3, 0, 15, False, True), (3, 0, 16, False, False)])
+def test_default_on_both_sides_of_its_limits(prec, link_fmt, nrhs, dw_pair, dhat_pair):
+    """The launch without the tuner is two threads per site below the limits and two
+    right-hand sides per thread above: the bits of that launch, pinned."""
+    import torch
+    from paper_2202_07388_gb300 import oq, synth
+    from tests.gpu_cases import to_dev
+    dims = (8, 8, 16, 16)
+    h = oq.Handle(dims)
+    h.gauge_upload(to_dev(synth.make_gauge(dims, 0.5, 946)), link_fmt)
+    h.clover_build(0.13, 1.0)
+    x = torch.randn(nrhs, 8 * 8 * 16 * 16, 24, dtype=torch.float64, device="cuda")
+    a, e = h.new_packed(prec, nrhs=nrhs), h.new_packed(prec, oq.EVEN, nrhs=nrhs)
+    h.pack(x, a, prec, nrhs=nrhs)
+    h.pack(x, e, prec, oq.EVEN, nrhs=nrhs)
+    out = {}
+    for pin in (None, (64, 0, 1, 0), (64, 1, 2, 3 if prec != 1 and link_fmt == 1 else 1)):
+        if pin:
+            for mode in (0, 1, 2):
+                h.tune_set(prec, mode, nrhs, *pin[:2], nr=pin[2], regcap=pin[3])
+        b, f = torch.empty_like(a), torch.empty_like(e)
+        h.dw(a, b, prec, nrhs=nrhs)
+        h.dw_hat(e, f, prec, nrhs=nrhs)
+        out["default" if not pin else pin[1] == 0] = b, f
+    for k, pair in enumerate((dw_pair, dhat_pair)):
+        assert torch.equal(out["default"][k], out[pair][k])
+        assert not torch.equal(out["default"][k], out[not pair][k])
+    h.close()
+
+
 @pytest.mark.parametrize("prec", [1, 2, 3])
 @pytest.mark.parametrize("nrhs", [1, 3])
 def test_reported_launch_comes_back(prec, nrhs):
