@@ -377,13 +377,6 @@ struct oq_ctx {
     *per_rhs = sites * spin;
   }
 
-  // all right-hand sides live
-  double hop_bytes(const oq::HopLaunch& l, const oq::HopArgs& a) {
-    double f = 0.0, r = 0.0;
-    hop_bytes_parts(l, a, &f, &r);
-    return f + r * a.nrhs;
-  }
-
   // the binary32 link copy that matches the launch's link format
   oq::HopArgs with_links(const oq::HopLaunch& l, const oq::HopArgs& a) {
     oq::HopArgs b = a;

@@ -46,11 +46,16 @@ __device__ __forceinline__ D2 dadd(D2 x, D2 y) {
   const D2 s = two_sum(x.hi, y.hi);
   return fast_two_sum(s.hi, add(s.lo, add(x.lo, y.lo)));
 }
+// x + y without the final renormalisation: the two-sum of the high parts
+// and the low parts added to its error (8 operations instead of dadd's 11).
+// The low part may exceed ulp(hi)/2 by a few ulp; a product or another lazy sum
+// takes such a value as it is, and dnorm restores the normal form.
 __device__ __forceinline__ D2 add_lazy(D2 x, D2 y) {
   const D2 s = two_sum(x.hi, y.hi);
   return D2{s.hi, add(s.lo, add(x.lo, y.lo))};
 }
 __device__ __forceinline__ D2 dnorm(D2 x) { return fast_two_sum(x.hi, x.lo); }
+// x * 2^k for a power of two s = 2^k: exact, both parts scaled
 __device__ __forceinline__ D2 dscale(D2 x, float s) { return D2{mul(x.hi, bc(s)), mul(x.lo, bc(s))}; }
 // a * b + c (both factors per lane)
 __device__ __forceinline__ D2 dfma(D2 a, D2 b, D2 c) {
@@ -87,7 +92,7 @@ __device__ __forceinline__ void acc_add(Acc& a, dfloat x, D2 y) {
 }
 __device__ __forceinline__ D2 acc_get(const Acc& a) { return fast_two_sum(a.s, a.e); }
 
-// z * i^c (selects and sign flips, as rot_ic)
+// z * i^c for c in 0..3: a swap of the parts for odd c and sign flips, all by selects
 __device__ __forceinline__ C2 rot_ic(const C2& z, int c) {
   const bool sw = c & 1;
   D2 re = sw ? z.im : z.re, im = sw ? z.re : z.im;
@@ -95,7 +100,7 @@ __device__ __forceinline__ C2 rot_ic(const C2& z, int c) {
   if (c >= 2) im = dneg(im);
   return C2{re, im};
 }
-// the same with a factor per lane
+// acc_first, acc_add with both factors per lane
 __device__ __forceinline__ void acc_first(Acc& a, D2 x, D2 y) {
   a.s = mul(x.hi, y.hi);
   F2 e = fma2(x.hi, y.hi, neg(a.s));

@@ -2,7 +2,8 @@
 //
 // The reset steps of the mixed-precision CGNE recompute the residual in
 // double-float arithmetic (an unevaluated sum hi + lo of two binary32
-// numbers; oq_device.cuh), one right-hand side per thread in hop_impl.cuh.
+// numbers; oq_device.cuh), one right-hand side per thread in hop_impl.cuh (whose
+// lanes are spins).
 // Here a thread carries two right-hand sides: every binary32 operation of
 // the double-float formulas acts on the pair at once as one packed two-lane
 // instruction (FADD2 / FMUL2 / FFMA2 of sm_100-class GPUs), in the same order
@@ -10,8 +11,8 @@
 // one-rhs kernel.  The links and clover blocks of a site are loaded once for
 // both.  A packed instruction occupies the binary32 pipe as long as two
 // scalar ones (the same flop rate); what it saves is issue slots and the
-// loads, index arithmetic and link handling per right-hand side, which bound
-// the one-rhs kernel (binary32 pipe ~55 % busy at ~75 % issue).
+// loads, index arithmetic and link handling per right-hand side, at the price of
+// its registers (255; the one-rhs kernel runs 12 warps per SM).
 //
 // Passes and epilogues: Dw (HOP_DW), Dhat pass 1 (HOP_P1), pass 2
 // (HOP_P2), with the plain store or the binary64-residual epilogue of a reset
@@ -73,7 +74,8 @@ __device__ __forceinline__ void clover_block(const void* base, long Vh, int p, l
   }
 }
 
-// The 8 hops as one runtime loop (hop_loop_df for two lanes): the spin
+// The 8 hops as one runtime loop (dfs::hop_loop with the two right-hand sides
+// as lanes instead of the two spins of a half spinor): the spin
 // projection is formed colour by colour from the neighbour's chunks, and each
 // colour row of U h is reconstructed onto acc as soon as it is formed, so
 // neither the neighbour spinor nor the transported half spinor is held whole.

@@ -52,33 +52,7 @@ __device__ __forceinline__ C2 csub(C2 a, C2 b) { return {sub(a.re, b.re), sub(a.
 __device__ __forceinline__ C2 cadd_i(C2 a, C2 b) { return {sub(a.re, b.im), add(a.im, b.re)}; }
 __device__ __forceinline__ C2 csub_i(C2 a, C2 b) { return {add(a.re, b.im), sub(a.im, b.re)}; }
 
-// spinor of site j, 32-bit offsets (chunk c at c*Vh + j)
-template <int P>
-__device__ __forceinline__ void load_sp(const char* base, uint32_t Vh, uint32_t j, Spinor<float>& s) {
-  cx<float>* f = &s.c[0][0];
-  if constexpr (P == P_F32) {
-    const float4* b = reinterpret_cast<const float4*>(base);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      const float4 v = __ldg(b + (c * Vh + j));
-      f[2 * c] = cx<float>{v.x, v.y};
-      f[2 * c + 1] = cx<float>{v.z, v.w};
-    }
-  } else {
-    const uint4* b = reinterpret_cast<const uint4*>(base);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const uint4 v = __ldg(b + (c * Vh + j));
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float2 z = (P == P_BF16) ? unpack_bf16x2(w[k]) : unpack_f16x2(w[k]);
-        f[4 * c + k] = cx<float>{z.x, z.y};
-      }
-    }
-  }
-}
-
+// store the spinor of site i, 32-bit offsets (chunk c at c*Vh + i)
 template <int P>
 __device__ __forceinline__ void store_sp(char* base, uint32_t Vh, uint32_t i, const Spinor<float>& s) {
   const cx<float>* f = &s.c[0][0];
@@ -835,10 +809,6 @@ template <int P, int NR, int MODE>
 constexpr int mr_stage_slots() {
   constexpr int sc = P == P_F32 ? 6 : 3;
   return (2 * (NR * sc + 3 + (MODE == HOP_P1 ? 0 : NR * sc / 2))) | 1;
-}
-template <int P, int NR, int MODE>
-constexpr size_t mr_stage_bytes(int nthr) {
-  return (size_t)mr_stage_slots<P, NR, MODE>() * 16 * nthr;
 }
 // the per-thread slots of a launch (staged: CAP = 2, 3)
 template <int P, int NR, int MODE, int CAP>

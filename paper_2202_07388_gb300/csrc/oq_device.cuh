@@ -98,17 +98,6 @@ __device__ __forceinline__ dfloat fma(dfloat a, dfloat b, dfloat c) {
   const dfloat s = df_two_sum(c.hi, p);
   return df_fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(c.lo, e)));
 }
-// x + y without the final renormalisation: the two-sum of the high parts
-// and the low parts added to its error (8 operations instead of 11).  The
-// low part may exceed ulp(hi)/2 by a few ulp; a product or another lazy sum
-// takes such a value as it is, and df_norm restores the normal form.
-__device__ __forceinline__ dfloat df_add_lazy(dfloat x, dfloat y) {
-  const dfloat s = df_two_sum(x.hi, y.hi);
-  return dfloat(s.hi, __fadd_rn(s.lo, __fadd_rn(x.lo, y.lo)));
-}
-__device__ __forceinline__ dfloat df_norm(dfloat x) { return df_fast_two_sum(x.hi, x.lo); }
-// x * 2^k for a power of two s = 2^k: exact, both parts scaled
-__device__ __forceinline__ dfloat df_scale(dfloat x, float s) { return dfloat(x.hi * s, x.lo * s); }
 using ::fma;  // keep the float / double overloads visible next to the dfloat one
 enum LinkFmt : int { LINK_18 = 0, LINK_12 = 1 };
 
@@ -168,8 +157,6 @@ __device__ __forceinline__ cx<R> cmulc(cx<R> a, cx<R> b) {
 }
 template <typename R>
 __device__ __forceinline__ cx<R> times_i(cx<R> a) { return {-a.im, a.re}; }
-template <typename R>
-__device__ __forceinline__ cx<R> times_mi(cx<R> a) { return {a.im, -a.re}; }
 // acc += a * b
 template <typename R>
 __device__ __forceinline__ void cfma(cx<R>& acc, cx<R> a, cx<R> b) {
