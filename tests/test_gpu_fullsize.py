@@ -99,3 +99,30 @@ def test_c3_dhat_f16_12rhs_sampled_sites():
             err = np.linalg.norm(got[k][x] - ref) / np.linalg.norm(ref)
             assert err < 5e-3, (k, x, err)
     h.close()
+
+
+def test_production_solve_residual_of_every_rhs():
+    """48 x 24^3, 12 right-hand sides, F16 storage, tuned launches: the residual of
+    every one, recomputed with the binary64 operator (its own kernels and links)."""
+    import torch
+    from paper_2202_07388_gb300 import oq
+    dims, nrhs = (48, 24, 24, 24), 12
+    vol = 48 * 24 ** 3
+    h = make_handle(dims, synth.make_gauge(dims, 0.5, 4), 0.135, 1.0, oq.LINK_12)
+    h.autotune(oq.F16, nrhs)
+    g = torch.Generator(device="cuda").manual_seed(35)
+    eta = torch.randn(nrhs, vol, 24, dtype=torch.float64, device="cuda", generator=g)
+    eta[:, torch.from_numpy(dirac.parity_mask(dims).reshape(-1)).cuda()] = 0.0
+    psi = torch.zeros_like(eta)
+    rc, st = h.cgne(eta, psi, oq.SolverParams(res=1e-10, nmx=5000, sdtype=oq.F16), nrhs=nrhs)
+    assert rc == oq.OK
+    e, x, t, y = (h.new_packed(oq.F64, oq.EVEN, nrhs=nrhs) for _ in range(4))
+    h.pack(eta, e, oq.F64, oq.EVEN, nrhs=nrhs)
+    h.pack(psi, x, oq.F64, oq.EVEN, nrhs=nrhs)
+    h.dw_hat(x, t, oq.F64, nrhs=nrhs)
+    h.dw_hat(t, y, oq.F64, nrhs=nrhs, dagger=True)
+    e, y = (v.view(torch.float64).view(nrhs, -1) for v in (e, y))
+    rel = ((e - y).norm(dim=1) / e.norm(dim=1)).cpu().numpy()
+    for k in range(nrhs):
+        check_residual(rel[k], st[k]["true_rel_res"])
+    h.close()
