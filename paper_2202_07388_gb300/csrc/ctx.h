@@ -317,12 +317,17 @@ struct oq_ctx {
     } else if (prec == oq::P_DF64 && !lats[lat].halo_t) {
       // the double-float site is latency- and issue-bound: 12 warps per SM at
       // 168 registers (Dhat, 12 rhs on 48x24^3: 4.0 ms against 6.5 ms
-      // uncapped in 32 x 6 CTAs, 4 rhs on 32x16^3: 304 against 370 us), 16
-      // with some spilling where a launch fills few waves (1 rhs on 32x16^3:
-      // 113 against 121 us)
+      // uncapped in 32 x 6 CTAs, 4 rhs on 32x16^3: 304 against 370 us).  The
+      // cap of 128 registers (16 warps, some spilling) pays only where it puts
+      // a launch of more than 3 CTAs per SM into one wave of 4 (Dhat, 1 rhs on
+      // 32x16^3, 512 CTAs: 107 against 116 us; 2 rhs on 16^4: 102 against 103;
+      // Dw on 16^4, 512 CTAs: 48.1 against 49.1) and costs elsewhere (Dhat on 8^4:
+      // 40.9 against 32.8 us; 16^4, 256 CTAs: 60.8 against 48.8; 4 rhs on
+      // 16x12^3, 432 CTAs: 73.7 against 65.0; 2 rhs on 32x16^3: 178 against 173)
       l.bx = 128;
       l.by = 1;
-      l.regcap = lats[lat].g.Vh * nrhs < (1L << 17) ? 1 : 2;
+      const long ctas = (lats[lat].g.Vh + 127) / 128 * nrhs * (mode == oq::HOP_DW ? 2 : 1);
+      l.regcap = ctas > 3 * 152 && ctas <= 4 * 152 ? 1 : 2;
     } else if (nrhs == 1) {
       l.bx = 128;
       l.by = 1;

@@ -167,3 +167,32 @@ def test_two_threads_per_site_refused_elsewhere():
     assert s.tune_set(oq.F32, 0, 1, 64, 0, check=False) == oq.ERR_ARG
     assert s.tune_set(oq.F32, 0, 1, 64, 1, check=False) == oq.OK
     s.close()
+
+
+@pytest.mark.parametrize("dims,nrhs", [((2, 2, 2, 2), 1), ((4, 6, 10, 6), 3), ((16, 16, 16, 16), 1),
+                                       ((16, 16, 16, 16), 2), ((16, 16, 16, 18), 2)])
+def test_default_double_float_launch(dims, nrhs):
+    """OQ_DF64 without the tuner: 168 registers, or 128 where that makes one wave of the
+    launch (16^4: Dw with 1, the passes of Dhat with 2 right-hand sides); the caps do not
+    change a bit of the uncapped kernel's result."""
+    import torch
+    from paper_2202_07388_gb300 import oq, synth
+    from tests.gpu_cases import to_dev
+    h = oq.Handle(dims)
+    h.gauge_upload(to_dev(synth.make_gauge(dims, 0.5, 947)), oq.LINK_18)
+    h.clover_build(0.13, 1.0)
+    x = torch.randn(nrhs, dims[0] * dims[1] * dims[2] * dims[3], 24, dtype=torch.float64, device="cuda")
+    a, e = h.new_packed(oq.DF64, nrhs=nrhs), h.new_packed(oq.DF64, oq.EVEN, nrhs=nrhs)
+    h.pack(x, a, oq.DF64, nrhs=nrhs)
+    h.pack(x, e, oq.DF64, oq.EVEN, nrhs=nrhs)
+    out = []
+    for pinned in (False, True):
+        if pinned:
+            for mode in (0, 1, 2):
+                h.tune_set(oq.DF64, mode, nrhs, 128, 1, regcap=0)
+        b, f = torch.empty_like(a), torch.empty_like(e)
+        h.dw(a, b, oq.DF64, nrhs=nrhs)
+        h.dw_hat(e, f, oq.DF64, nrhs=nrhs)
+        out.append((b, f))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    h.close()
