@@ -106,19 +106,25 @@ enum LinkFmt : int { LINK_18 = 0, LINK_12 = 1 };
 // on the binary64 pipe (2 lanes per SM and clock on GB300), which bounds kernels
 // that build or read binary64 fields; the integer pipe has 64 lanes.  Bit for bit
 // the conversion (round to nearest even); values outside the normal binary32
-// range take the instruction.  (Packing two F32 fields on 32^4: 125 against 188
+// range take the instruction.  (Packing 12 F32 fields on 48x24^3: 395 against 693
 // us, with the multiplication by a scale of 1 left out.  The other direction
-// gains nothing: unpacking them took 287 us that way, 258 us by the instruction.)
+// gained nothing in an unpacking kernel bound by its stores: 287 us that way,
+// 258 us by the instruction, 2 fields on 32^4.)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float narrow(double x) {
+// narrow_bits: the integer form alone; sets slow (and returns no result) where the
+// value needs the instruction.
+__device__ __forceinline__ float narrow_bits(double x, bool& slow) {
   const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x), m = hi & 0x7fffffffu;
-  if (m - 0x38100000u < 0x0fe00000u) {  // exponents of normal binary32 values
-    const uint32_t q = ((m - 0x38000000u) << 3) | (lo >> 29);
-    const uint32_t up = ((lo & 0x1fffffffu) + 0x0fffffffu + (q & 1u)) >> 29;  // to nearest, ties to even
-    return __uint_as_float((q + up) | (hi & 0x80000000u));
-  }
-  if (m == 0u && lo == 0u) return __uint_as_float(hi & 0x80000000u);
-  return __double2float_rn(x);
+  const bool zero = (m | lo) == 0u;
+  slow = slow || !(zero || m - 0x38100000u < 0x0fe00000u);  // the exponents of normal binary32 values
+  const uint32_t q = ((m - 0x38000000u) << 3) | (lo >> 29);
+  const uint32_t up = ((lo & 0x1fffffffu) + 0x0fffffffu + (q & 1u)) >> 29;  // to nearest, ties to even
+  return __uint_as_float((zero ? 0u : q + up) | (hi & 0x80000000u));
+}
+__device__ __forceinline__ float narrow(double x) {
+  bool slow = false;
+  const float r = narrow_bits(x, slow);
+  return slow ? __double2float_rn(x) : r;
 }
 // a binary64 value in the arithmetic type R
 template <typename R>

@@ -123,75 +123,82 @@ cudaError_t sf_mask_links(const Geom& g, double* u64, void* u32, int fmt, void* 
   return cudaGetLastError();
 }
 
-// x * scale; the usual scale of 1 needs no pass through the binary64 pipe
-__device__ __forceinline__ double times(double x, double scale) { return scale == 1.0 ? x : x * scale; }
+// The site's 24 reals in the arithmetic type: at(k) gives complex component k
+// (scaled).  Binary32: by integer operations, and over again by the conversion
+// instruction if one of them needs it.  One branch a site: with one a value, F32
+// fields took 4.5 against 2.9 us on 8^4, and 742 against 395 us for 12 fields of
+// zeros on 48x24^3 (418 of other values; by the instruction 693).
+template <typename R, typename F>
+__device__ __forceinline__ void site_from64(Spinor<R>& s, F at) {
+  if constexpr (std::is_same<R, float>::value) {
+    bool slow = false;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const double2 v = at(k);
+      s.c[k / 3][k % 3] = cx<R>{narrow_bits(v.x, slow), narrow_bits(v.y, slow)};
+    }
+    if (!slow) return;
+  }
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    const double2 v = at(k);
+    s.c[k / 3][k % 3] = cx<R>{R(v.x), R(v.y)};
+  }
+}
+
+// four complex values as 16-bit pairs, rounded from binary64 directly (no
+// intermediate binary32 rounding)
+template <int P, typename F>
+__device__ __forceinline__ uint4 chunk16(F at) {
+  uint32_t w[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double2 v = at(k);
+    if constexpr (P == P_BF16) {
+      const __nv_bfloat16 a = __double2bfloat16(v.x), b = __double2bfloat16(v.y);
+      w[k] = (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+    } else {
+      const __half a = __double2half(v.x), b = __double2half(v.y);
+      w[k] = (uint32_t)__half_as_ushort(a) | ((uint32_t)__half_as_ushort(b) << 16);
+    }
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
 
 // one thread per (eo site, parity, rhs).  blockIdx.y = parity index within
-// the subset, blockIdx.z = rhs.
-template <int P>
+// the subset, blockIdx.z = rhs.  UNIT: scale 1 and not a Schroedinger-functional
+// lattice (whose field vanishes at x0 = 0: scale 0 there): no multiplications on
+// the binary64 pipe.
+template <int P, bool UNIT>
 __global__ void pack_spinor_kernel(Geom g, const double2* __restrict__ canon, char* __restrict__ out,
-                                   int subset, long canon_stride, long out_stride, double scale, int half) {
-  typedef typename PrecTraits<P>::R R;
+                                   int subset, long canon_stride, long out_stride, double scale) {
   const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= g.Vh) return;
   const int p = (subset == 2) ? (int)blockIdx.y : subset;
   const int rhs = blockIdx.z;
   int x[4];
   eo_coords(g, p, i, x);
-  // half: the canonical field holds one parity only, site lex / 2 (the sites
-  // of one parity alternate along x3, L3 even)
-  const double2* src = canon + rhs * canon_stride + (half ? lex_of(g, x) >> 1 : lex_of(g, x)) * 12;
-  // Schroedinger-functional lattices: the field vanishes at x0 = 0
-  if (g.bc_t == 0.f && x[0] == 0) scale = 0.0;
-  Spinor<R> s;
-#pragma unroll
-  for (int k = 0; k < 12; ++k) {
-    double2 v = src[k];
-    s.c[k / 3][k % 3] = cx<R>{from64<R>(times(v.x, scale)), from64<R>(times(v.y, scale))};
-  }
+  const double2* src = canon + rhs * canon_stride + lex_of(g, x) * 12;
+  if (!UNIT && g.bc_t == 0.f && x[0] == 0) scale = 0.0;
+  auto at = [&](int k) {
+    const double2 v = src[k];
+    return UNIT ? v : make_double2(v.x * scale, v.y * scale);
+  };
   char* dst = out + rhs * out_stride + ((subset == 2) ? (long)p * spinor_half_bytes(g.Vh, P) : 0);
   if constexpr (P == P_BF16 || P == P_F16) {
-    // round binary64 -> 16-bit directly (no intermediate binary32 rounding)
     uint4* b = reinterpret_cast<uint4*>(dst);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      uint32_t w[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        double2 v = src[4 * c + k];
-        double re = times(v.x, scale), im = times(v.y, scale);
-        if constexpr (P == P_BF16) {
-          __nv_bfloat16 a = __double2bfloat16(re), bb = __double2bfloat16(im);
-          w[k] = (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(bb) << 16);
-        } else {
-          __half a = __double2half(re), bb = __double2half(im);
-          w[k] = (uint32_t)__half_as_ushort(a) | ((uint32_t)__half_as_ushort(bb) << 16);
-        }
-      }
-      b[c * g.Vh + i] = make_uint4(w[0], w[1], w[2], w[3]);
-    }
+    for (int c = 0; c < 3; ++c) b[c * g.Vh + i] = chunk16<P>([&](int k) { return at(4 * c + k); });
   } else {
+    Spinor<typename PrecTraits<P>::R> s;
+    site_from64(s, at);
     store_spinor<P>(dst, g.Vh, i, s);
   }
 }
 
-template <int P>
-__global__ void unpack_spinor_kernel(Geom g, const char* __restrict__ in, double2* __restrict__ canon,
-                                     int subset, long in_stride, long canon_stride, double inv_scale, int half) {
-  typedef typename PrecTraits<P>::R R;
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= g.Vh) return;
-  const int p = (subset == 2) ? (int)blockIdx.y : subset;
-  const int rhs = blockIdx.z;
-  int x[4];
-  eo_coords(g, p, i, x);
-  const char* src = in + rhs * in_stride + ((subset == 2) ? (long)p * spinor_half_bytes(g.Vh, P) : 0);
-  Spinor<R> s;
-  load_spinor<P>(src, g.Vh, i, s);
-  double2* dst = canon + rhs * canon_stride + (half ? lex_of(g, x) >> 1 : lex_of(g, x)) * 12;
-#pragma unroll
-  for (int k = 0; k < 12; ++k)
-    dst[k] = make_double2(times((double)s.c[k / 3][k % 3].re, inv_scale), times((double)s.c[k / 3][k % 3].im, inv_scale));
+template <bool UNIT, typename R>
+__device__ __forceinline__ double unscaled(R x, double inv_scale) {
+  return UNIT ? (double)x : (double)x * inv_scale;
 }
 
 // Even-site (or odd-site) canonical fields: the site of eo index i sits at
@@ -204,11 +211,10 @@ __global__ void unpack_spinor_kernel(Geom g, const char* __restrict__ in, double
 // conflicts.  blockDim.x = 128.
 constexpr int HB = 128, HROW = 13;
 
-template <int P>
+template <int P, bool UNIT>
 __global__ void __launch_bounds__(HB) pack_half_kernel(Geom g, const double2* __restrict__ canon,
                                                        char* __restrict__ out, int p, long canon_stride,
                                                        long out_stride, double scale) {
-  typedef typename PrecTraits<P>::R R;
   __shared__ double2 sm[HB * HROW];
   const int t = threadIdx.x, rhs = blockIdx.z;
   const long i0 = (long)blockIdx.x * HB;
@@ -218,124 +224,120 @@ __global__ void __launch_bounds__(HB) pack_half_kernel(Geom g, const double2* __
   __syncthreads();
   if (t >= nsite) return;
   const long i = i0 + t;
-  double sc = scale;
-  if (g.bc_t == 0.f) {  // Schroedinger-functional lattices: the field vanishes at x0 = 0
+  if (!UNIT && g.bc_t == 0.f) {  // Schroedinger-functional lattices: the field vanishes at x0 = 0
     int x[4];
     eo_coords(g, p, i, x);
-    if (x[0] == 0) sc = 0.0;
+    if (x[0] == 0) scale = 0.0;
   }
+  auto at = [&](int k) {
+    const double2 v = sm[t * HROW + k];
+    return UNIT ? v : make_double2(v.x * scale, v.y * scale);
+  };
   char* dst = out + rhs * out_stride;
   if constexpr (P == P_BF16 || P == P_F16) {
     uint4* b = reinterpret_cast<uint4*>(dst);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      uint32_t w[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const double2 v = sm[t * HROW + 4 * c + k];
-        const double re = times(v.x, sc), im = times(v.y, sc);
-        if constexpr (P == P_BF16) {
-          __nv_bfloat16 a = __double2bfloat16(re), bb = __double2bfloat16(im);
-          w[k] = (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(bb) << 16);
-        } else {
-          __half a = __double2half(re), bb = __double2half(im);
-          w[k] = (uint32_t)__half_as_ushort(a) | ((uint32_t)__half_as_ushort(bb) << 16);
-        }
-      }
-      b[c * g.Vh + i] = make_uint4(w[0], w[1], w[2], w[3]);
-    }
+    for (int c = 0; c < 3; ++c) b[c * g.Vh + i] = chunk16<P>([&](int k) { return at(4 * c + k); });
   } else {
-    Spinor<R> sp;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      const double2 v = sm[t * HROW + k];
-      sp.c[k / 3][k % 3] = cx<R>{from64<R>(times(v.x, sc)), from64<R>(times(v.y, sc))};
-    }
+    Spinor<typename PrecTraits<P>::R> sp;
+    site_from64(sp, at);
     store_spinor<P>(dst, g.Vh, i, sp);
   }
 }
 
-template <int P>
-__global__ void __launch_bounds__(HB) unpack_half_kernel(Geom g, const char* __restrict__ in,
-                                                         double2* __restrict__ canon, long in_stride,
-                                                         long canon_stride, double inv_scale) {
-  typedef typename PrecTraits<P>::R R;
+// Packed sites to a canonical field of one parity (HALF) or of both (blockIdx.y),
+// through shared memory as above: a site's 192 bytes are written by 12
+// neighbouring threads.  (Each thread writing its own site's, pieces of 16 bytes
+// 384 bytes apart: 12 full fields on 48x24^3 F64 654, F32 1070, F16 1130 us; 560, 446
+// and 322 this way.)  UNIT: scale 1, no multiplication on the binary64 pipe (a
+// choice per value is a branch before each store: F64 on 8^4 3.5 against 2.0 us).
+template <int P, bool UNIT, bool HALF>
+__global__ void __launch_bounds__(HB) unpack_kernel(Geom g, const char* __restrict__ in, double2* __restrict__ canon,
+                                                    int subset, long in_stride, long canon_stride, double inv_scale) {
   __shared__ double2 sm[HB * HROW];
-  const int t = threadIdx.x, rhs = blockIdx.z;
+  __shared__ int at[HB];  // the site's position in the canonical field
+  const int t = threadIdx.x, rhs = blockIdx.z, p = subset == 2 ? (int)blockIdx.y : subset;
   const long i0 = (long)blockIdx.x * HB;
   const int nsite = (int)(g.Vh - i0 < HB ? g.Vh - i0 : HB);
+  const char* src = in + rhs * in_stride + ((subset == 2) ? (long)p * spinor_half_bytes(g.Vh, P) : 0);
   if (t < nsite) {
-    Spinor<R> sp;
-    load_spinor<P>(in + rhs * in_stride, g.Vh, i0 + t, sp);
+    const long i = i0 + t;
+    if (!HALF) {
+      int x[4];
+      eo_coords(g, p, i, x);
+      at[t] = (int)(2 * i) + (x[3] & 1);  // lex: the eo index is lex >> 1
+    }
+    Spinor<typename PrecTraits<P>::R> sp;
+    load_spinor<P>(src, g.Vh, i, sp);
 #pragma unroll
-    for (int k = 0; k < 12; ++k)
-      sm[t * HROW + k] = make_double2(times((double)sp.c[k / 3][k % 3].re, inv_scale),
-                                      times((double)sp.c[k / 3][k % 3].im, inv_scale));
+    for (int k = 0; k < 12; ++k) {
+      const double re = (double)sp.c[k / 3][k % 3].re, im = (double)sp.c[k / 3][k % 3].im;
+      sm[t * HROW + k] = UNIT ? make_double2(re, im) : make_double2(re * inv_scale, im * inv_scale);
+    }
   }
   __syncthreads();
-  double2* dst = canon + rhs * canon_stride + i0 * 12;
-  for (int e = t; e < nsite * 12; e += HB) dst[e] = sm[(e / 12) * HROW + e % 12];
+  double2* dst = canon + rhs * canon_stride;
+  for (int e = t; e < nsite * 12; e += HB) {
+    const long site = HALF ? i0 + e / 12 : (long)at[e / 12];
+    dst[site * 12 + e % 12] = sm[(e / 12) * HROW + e % 12];
+  }
+}
+
+template <int P, bool UNIT>
+static void pack_launch(const Geom& g, int subset, const double2* canon, char* out, double scale, int nrhs,
+                        long canon_stride, long out_stride, cudaStream_t s, int half) {
+  if (half) {
+    const dim3 hb(HB), hg((unsigned)((g.Vh + HB - 1) / HB), 1, nrhs);
+    pack_half_kernel<P, UNIT><<<hg, hb, 0, s>>>(g, canon, out, subset, canon_stride, out_stride, scale);
+  } else {
+    const dim3 block(128), grid((unsigned)((g.Vh + 127) / 128), subset == 2 ? 2 : 1, nrhs);
+    pack_spinor_kernel<P, UNIT><<<grid, block, 0, s>>>(g, canon, out, subset, canon_stride, out_stride, scale);
+  }
 }
 
 cudaError_t pack_spinor(const Geom& g, int prec, int subset, const double* canon, void* out, double scale,
                         int nrhs, long canon_stride_d2, long out_stride_bytes, cudaStream_t s, int half) {
   if (half && subset == 2) return cudaErrorInvalidValue;
-  if (half) {
-    dim3 hb(HB), hg((unsigned)((g.Vh + HB - 1) / HB), 1, nrhs);
-    const double2* c = reinterpret_cast<const double2*>(canon);
-    char* o = reinterpret_cast<char*>(out);
-    switch (prec) {
-      case P_F64: pack_half_kernel<P_F64><<<hg, hb, 0, s>>>(g, c, o, subset, canon_stride_d2, out_stride_bytes, scale); break;
-      case P_F32: pack_half_kernel<P_F32><<<hg, hb, 0, s>>>(g, c, o, subset, canon_stride_d2, out_stride_bytes, scale); break;
-      case P_BF16: pack_half_kernel<P_BF16><<<hg, hb, 0, s>>>(g, c, o, subset, canon_stride_d2, out_stride_bytes, scale); break;
-      case P_F16: pack_half_kernel<P_F16><<<hg, hb, 0, s>>>(g, c, o, subset, canon_stride_d2, out_stride_bytes, scale); break;
-      case P_DF64: pack_half_kernel<P_DF64><<<hg, hb, 0, s>>>(g, c, o, subset, canon_stride_d2, out_stride_bytes, scale); break;
-      default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-  }
-  dim3 block(128), grid((unsigned)((g.Vh + 127) / 128), subset == 2 ? 2 : 1, nrhs);
   const double2* c = reinterpret_cast<const double2*>(canon);
   char* o = reinterpret_cast<char*>(out);
+  auto launch = [&](auto* unit, auto* scaled) {
+    (scale == 1.0 && g.bc_t != 0.f ? unit : scaled)(g, subset, c, o, scale, nrhs, canon_stride_d2, out_stride_bytes, s,
+                                                    half);
+  };
   switch (prec) {
-    case P_F64: pack_spinor_kernel<P_F64><<<grid, block, 0, s>>>(g, c, o, subset, canon_stride_d2, out_stride_bytes, scale, half); break;
-    case P_F32: pack_spinor_kernel<P_F32><<<grid, block, 0, s>>>(g, c, o, subset, canon_stride_d2, out_stride_bytes, scale, half); break;
-    case P_BF16: pack_spinor_kernel<P_BF16><<<grid, block, 0, s>>>(g, c, o, subset, canon_stride_d2, out_stride_bytes, scale, half); break;
-    case P_F16: pack_spinor_kernel<P_F16><<<grid, block, 0, s>>>(g, c, o, subset, canon_stride_d2, out_stride_bytes, scale, half); break;
-    case P_DF64: pack_spinor_kernel<P_DF64><<<grid, block, 0, s>>>(g, c, o, subset, canon_stride_d2, out_stride_bytes, scale, half); break;
+    case P_F64: launch(pack_launch<P_F64, true>, pack_launch<P_F64, false>); break;
+    case P_F32: launch(pack_launch<P_F32, true>, pack_launch<P_F32, false>); break;
+    case P_BF16: launch(pack_launch<P_BF16, true>, pack_launch<P_BF16, false>); break;
+    case P_F16: launch(pack_launch<P_F16, true>, pack_launch<P_F16, false>); break;
+    case P_DF64: launch(pack_launch<P_DF64, true>, pack_launch<P_DF64, false>); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
 
+template <int P, bool UNIT>
+static void unpack_launch(const Geom& g, int subset, const char* in, double2* canon, double inv_scale, int nrhs,
+                          long in_stride, long canon_stride, cudaStream_t s, int half) {
+  const dim3 grid((unsigned)((g.Vh + HB - 1) / HB), subset == 2 ? 2 : 1, nrhs);
+  auto* k = half ? unpack_kernel<P, UNIT, true> : unpack_kernel<P, UNIT, false>;
+  k<<<grid, HB, 0, s>>>(g, in, canon, subset, in_stride, canon_stride, inv_scale);
+}
+
 cudaError_t unpack_spinor(const Geom& g, int prec, int subset, const void* in, double* canon, double scale,
                           int nrhs, long in_stride_bytes, long canon_stride_d2, cudaStream_t s, int half) {
   if (half && subset == 2) return cudaErrorInvalidValue;
-  if (half) {
-    dim3 hb(HB), hg((unsigned)((g.Vh + HB - 1) / HB), 1, nrhs);
-    double2* c = reinterpret_cast<double2*>(canon);
-    const char* i = reinterpret_cast<const char*>(in);
-    const double inv = 1.0 / scale;
-    switch (prec) {
-      case P_F64: unpack_half_kernel<P_F64><<<hg, hb, 0, s>>>(g, i, c, in_stride_bytes, canon_stride_d2, inv); break;
-      case P_F32: unpack_half_kernel<P_F32><<<hg, hb, 0, s>>>(g, i, c, in_stride_bytes, canon_stride_d2, inv); break;
-      case P_BF16: unpack_half_kernel<P_BF16><<<hg, hb, 0, s>>>(g, i, c, in_stride_bytes, canon_stride_d2, inv); break;
-      case P_F16: unpack_half_kernel<P_F16><<<hg, hb, 0, s>>>(g, i, c, in_stride_bytes, canon_stride_d2, inv); break;
-      case P_DF64: unpack_half_kernel<P_DF64><<<hg, hb, 0, s>>>(g, i, c, in_stride_bytes, canon_stride_d2, inv); break;
-      default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-  }
-  dim3 block(128), grid((unsigned)((g.Vh + 127) / 128), subset == 2 ? 2 : 1, nrhs);
   double2* c = reinterpret_cast<double2*>(canon);
   const char* i = reinterpret_cast<const char*>(in);
   const double inv = 1.0 / scale;
+  auto launch = [&](auto* unit, auto* scaled) {
+    (inv == 1.0 ? unit : scaled)(g, subset, i, c, inv, nrhs, in_stride_bytes, canon_stride_d2, s, half);
+  };
   switch (prec) {
-    case P_F64: unpack_spinor_kernel<P_F64><<<grid, block, 0, s>>>(g, i, c, subset, in_stride_bytes, canon_stride_d2, inv, half); break;
-    case P_F32: unpack_spinor_kernel<P_F32><<<grid, block, 0, s>>>(g, i, c, subset, in_stride_bytes, canon_stride_d2, inv, half); break;
-    case P_BF16: unpack_spinor_kernel<P_BF16><<<grid, block, 0, s>>>(g, i, c, subset, in_stride_bytes, canon_stride_d2, inv, half); break;
-    case P_F16: unpack_spinor_kernel<P_F16><<<grid, block, 0, s>>>(g, i, c, subset, in_stride_bytes, canon_stride_d2, inv, half); break;
-    case P_DF64: unpack_spinor_kernel<P_DF64><<<grid, block, 0, s>>>(g, i, c, subset, in_stride_bytes, canon_stride_d2, inv, half); break;
+    case P_F64: launch(unpack_launch<P_F64, true>, unpack_launch<P_F64, false>); break;
+    case P_F32: launch(unpack_launch<P_F32, true>, unpack_launch<P_F32, false>); break;
+    case P_BF16: launch(unpack_launch<P_BF16, true>, unpack_launch<P_BF16, false>); break;
+    case P_F16: launch(unpack_launch<P_F16, true>, unpack_launch<P_F16, false>); break;
+    case P_DF64: launch(unpack_launch<P_DF64, true>, unpack_launch<P_DF64, false>); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -1,5 +1,5 @@
-"""Packing and unpacking of binary32 fields bit for bit against the conversions
-of the host (round to nearest even): ties, values that round up to the next
+"""Packing and unpacking of fields bit for bit against the conversions of the host
+(round to nearest even; binary64, binary32 and binary16): ties, values that round up to the next
 exponent or to infinity, binary32 subnormals, zeros of both signs, infinities
 and NaN, with scale 1 and a power of two."""
 import numpy as np
@@ -23,11 +23,11 @@ def _specials():
 
 @pytest.mark.parametrize("scale", [1.0, 0.25])
 @pytest.mark.parametrize("half", [False, True])
-def test_binary32_pack_and_unpack_bits(scale, half):
+@pytest.mark.parametrize("dims", [(4, 4, 6, 8), (2, 2, 2, 2), (2, 6, 10, 6)])   # 384, 8, 360 sites of a parity
+def test_binary32_pack_and_unpack_bits(scale, half, dims):
     import torch
     from paper_2202_07388_gb300 import oq
-    dims = (4, 4, 6, 8)
-    vol = 768
+    vol = int(np.prod(dims))
     x = np.resize(_specials(), (vol, 24))
     h = oq.Handle(dims)
     sub = oq.EVEN if half else oq.FULL
@@ -50,4 +50,38 @@ def test_binary32_pack_and_unpack_bits(scale, half):
     b = back.cpu().numpy()
     ok = ~np.isnan(exp)
     assert np.array_equal(b.view(np.uint64)[ok], exp.view(np.uint64)[ok]) and np.isnan(b[~ok]).all()
+    h.close()
+
+
+@pytest.mark.parametrize("scale", [1.0, 0.25])
+@pytest.mark.parametrize("sub", [0, 1, 2])
+@pytest.mark.parametrize("prec", [0, 3])
+def test_pack_and_unpack_bits_of_two_fields(prec, sub, scale):
+    """Subsets and two right-hand sides, a site count that fills no last CTA; the sites
+    of the other parity stay as they were.  All-zero sites and fields included."""
+    import torch
+    from paper_2202_07388_gb300 import oq
+    dims = (2, 6, 10, 6)
+    vol = 720
+    rng = np.random.default_rng(952)
+    x = rng.standard_normal((2, vol, 24))
+    x[0, ::7] = 0.0
+    x[1, 100:400] = -0.0
+    h = oq.Handle(dims)
+    packed = h.new_packed(prec, sub, nrhs=2)
+    h.pack(torch.from_numpy(x).cuda(), packed, prec, sub, scale=scale, nrhs=2)
+    t = {0: np.float64, 3: np.float16}[prec]
+    ref = (x * scale).astype(t)
+    par = (np.indices(dims).sum(axis=0) % 2).reshape(-1)
+    chunk = 16 // np.dtype(t).itemsize
+    want = [ref[r][par == p].reshape(-1, 24 // chunk, chunk).transpose(1, 0, 2).reshape(-1)
+            for r in (0, 1) for p in ((0, 1) if sub == oq.FULL else (sub,))]
+    got = packed.cpu().numpy().view(np.uint8)
+    assert np.array_equal(got, np.concatenate(want).view(np.uint8))
+    back = torch.full((2, vol, 24), 7.0, dtype=torch.float64, device="cuda")
+    h.unpack(packed, back, prec, sub, scale=scale, nrhs=2)
+    exp = ref.astype(np.float64) / scale
+    if sub != oq.FULL:
+        exp[:, par != sub] = 7.0
+    assert np.array_equal(back.cpu().numpy().view(np.uint64), exp.view(np.uint64))
     h.close()
