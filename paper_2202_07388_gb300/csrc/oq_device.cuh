@@ -313,12 +313,16 @@ __device__ __forceinline__ uint32_t pack_f16x2(float a, float b) {
 // Fields that another kernel of the stream may still be writing when this one
 // starts (programmatic dependent launch) are read with ordinary loads: a
 // non-coherent load may be moved above the wait for that kernel.  Links and
-// clover blocks never change under a launch and keep the non-coherent path.
-template <typename T>
-__device__ __forceinline__ T ld_field(const T* p) { return *p; }
+// clover blocks never change under a launch and keep the non-coherent path.  NC:
+// that path for a field that the kernel does not write, in a kernel launched
+// without programmatic dependence.
+template <bool NC = false, typename T>
+__device__ __forceinline__ T ld_field(const T* p) {
+  return NC ? ldg_nc(p) : *p;
+}
 
 // Load the 12 complex components of site i from a packed spinor field.
-template <int P>
+template <int P, bool NC = false>
 __device__ __forceinline__ void load_spinor(const void* base, long Vh, long i,
                                             Spinor<typename PrecTraits<P>::R>& s) {
   typedef typename PrecTraits<P>::R R;
@@ -327,7 +331,7 @@ __device__ __forceinline__ void load_spinor(const void* base, long Vh, long i,
     const double2* b = reinterpret_cast<const double2*>(base);
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
-      double2 v = ld_field(b + c * Vh + i);
+      double2 v = ld_field<NC>(b + c * Vh + i);
       f[c] = cx<R>{R(v.x), R(v.y)};
     }
   } else if constexpr (P == P_DF64) {
@@ -335,14 +339,14 @@ __device__ __forceinline__ void load_spinor(const void* base, long Vh, long i,
     const float4* b = reinterpret_cast<const float4*>(base);
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
-      float4 v = ld_field(b + c * Vh + i);
+      float4 v = ld_field<NC>(b + c * Vh + i);
       f[c] = cx<R>{dfloat(v.x, v.y), dfloat(v.z, v.w)};
     }
   } else if constexpr (P == P_F32) {
     const float4* b = reinterpret_cast<const float4*>(base);
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
-      float4 v = ld_field(b + c * Vh + i);
+      float4 v = ld_field<NC>(b + c * Vh + i);
       f[2 * c] = cx<R>{v.x, v.y};
       f[2 * c + 1] = cx<R>{v.z, v.w};
     }
@@ -350,7 +354,7 @@ __device__ __forceinline__ void load_spinor(const void* base, long Vh, long i,
     const uint4* b = reinterpret_cast<const uint4*>(base);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      uint4 v = ld_field(b + c * Vh + i);
+      uint4 v = ld_field<NC>(b + c * Vh + i);
       uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
