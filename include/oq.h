@@ -460,7 +460,7 @@ int oq_cgne_solve_even(oq_handle h, int lat, const oq_solver_params* p, const do
  * e.g. the QCD+QED charges of a U(3) ensemble), one right-hand side each
  * (eta_dev[k], psi_dev[k]: host arrays of device pointers to canonical
  * binary64 full-lattice fields).  Every stencil pass of all systems is one
- * launch of a persistent grid over a (system, site block) tile list; chunks
+ * launch over a (system, site block) tile list, a CTA per tile; chunks
  * of regular iterations are captured once into a CUDA graph and replayed.
  * All systems must use the same link format.  Runs on a library-owned
  * stream after synchronising `stream`; returns when done.  st: nsys entries. */
@@ -480,7 +480,10 @@ int oq_cgne_solve_batch(oq_handle h, int nsys, const int* lats, const oq_solver_
  * res ||eta|| / n_blocks; cycles end when one does not lower the SAP
  * residual).  Krylov vectors, SAP and regular steps: binary32 (p->sdtype
  * must be OQ_F32); solution, restart residuals and reductions: binary64.
- * nkv (<= 64) vectors per restart, nmx GCR steps at most. */
+ * nkv (<= 64) vectors per restart, nmx GCR steps at most.  Work fields stay
+ * with the handle for later solves; with ncy > 0 among them copies of the links
+ * and clover in block order, 480 (12-real links) or 576 bytes per site (a solve
+ * that cannot have those reads the uploaded fields instead). */
 int oq_sap_gcr_solve(oq_handle h, int lat, const oq_solver_params* p, const double* eta_dev,
                      double* psi_dev, int nrhs, oq_status* st, void* stream);
 

@@ -338,7 +338,7 @@ struct oq_ctx {
       // capped at 128 registers; within 10 % of the tuner's choice from 8^4 to
       // 48x24^3 with 2 to 12 rhs, where one rhs per thread in 32 x nrhs CTAs
       // took 1.2 to 1.9 times as long (12 rhs F16 Dhat on 48x24^3: 495 against
-      // 814 us; 4 rhs F32 on 32x16^3: 62 against 78 us).
+      // 814 us; 4 rhs F32 on 32x16^3: 58 against 78 us).
       l.bx = 64;
       l.by = 1;
       l.nr = 2;

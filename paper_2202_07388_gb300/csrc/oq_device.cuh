@@ -636,7 +636,7 @@ __device__ __forceinline__ void store_half(void* base, long Fs, long f, const Ha
 // a boundary sign, the product is exact and the result is that of a separate
 // multiplication and addition; 12 operations of 36 fewer per hop, which is 8 %
 // of the binary64 stencil passes, bound by the binary64 pipe: adjoint Dw with 2 rhs
-// on 24x12x10x14 takes 192 us instead of 203.)
+// on 24x12x10x14 takes 193 us instead of 203.)
 template <int MU, int S, typename R>
 __device__ __forceinline__ void accum_reconstruct(Spinor<R>& acc, const HalfSpinor<R>& h, R w) {
   const R n = -w;

@@ -1,6 +1,6 @@
 """Uneven batch: QCD+QED operators (U(3) = SU(3) x U(1) links with charges
 2/3 and -1/3) on lattices of three sizes solved by one batched CGNE
-(persistent tile-list launches, graph-captured regular iterations).  Every
+(tile-list launches, graph-captured regular iterations).  Every
 solution is checked with the FP64 oracle's operator (binary64 residual of the
 normal equations <= 1e-10), and the batch agrees with one-system solves."""
 import numpy as np
